@@ -7,11 +7,18 @@
 
 namespace smash {
 
-constexpr int kBW = 8;                 // warps per block = rows per tile
+constexpr int kBW = 8;                 // warps per block
 constexpr int kBNT = kBW * 32;
 
 // Classification of a row.
-enum : uint8_t { kRowEmpty = 0, kRowSmall = 1, kRowBig = 2, kRowHuge = 3 };
+enum : uint8_t { kRowEmpty = 0, kRowSmall = 1, kRowBig = 2, kRowHuge = 3, kRowMed = 4 };
+// Products of a narrow row (its product's B fits a warp's dense accumulator):
+// up to kMedFlop it is served with its neighbours (a warp claims 32 rows at
+// once), up to kBigFlop by a warp that claims it alone, above by a block.
+constexpr int kMedFlop = 512;
+constexpr int kBigFlop = 8192;
+constexpr int kSegEntries = 8192;
+constexpr int kSegRows = 2048;
 
 struct BatchMat {
     const int64_t *a_rp;
@@ -25,26 +32,30 @@ struct BatchMat {
     int32_t a_rows;
     int32_t b_rows;
     int32_t ncols;
-    int32_t pad;
+    int32_t mode;     // dense accumulator of a warp (warp_dense.cuh), -1: B too wide, hash tables
     int64_t row_off;  // first row of this product in the flattened row space
-    int64_t tile_off; // first tile of this product
+    int64_t seg_off;  // first of its segments in the pass over the narrow B (segments of kSegEntries
+                      // entries, then of kSegRows rows)
 };
 
 struct BatchArgs {
     const BatchMat *mats;
     int nmat;
     int64_t nrows;          // all products' rows
-    int64_t ntiles;
     const int64_t *row_start;   // [nmat+1]
-    const int64_t *tile_start;  // [nmat+1]
     uint8_t *cls;           // [nrows]
     int *ub;                // [nrows] min(flop, cols)
     int *nnz;               // [nrows]
     int *big;               // [nrows] list of big rows
     int *huge;              // [nrows] list of huge rows
-    int *counters;          // [12]: 0 nbig, 1 nhuge, 2..4 item tokens, 5 matrix token, 6..7 barrier,
-                            // 8..9 row-chunk tokens of the two row phases
+    int *med;               // [nrows] list of narrow rows claimed one at a time
+    int *longs;             // [nrows] list of rows counted by a warp (k_batch_rowinfo_long)
+    int *counters;          // [16]: 0 nbig, 1 nhuge, 2..3 item tokens, 4 med token, 5 matrix token, 6..7 barrier,
+                            // 8..9 row-chunk tokens of the two row phases, 12 nmed, 13 nlong
     unsigned long long *sums;   // [4]: sum ub, sum flop
+    long long *descents;    // [nmat] 0: every row of B ascends (warp_dense.cuh)
+    int64_t nseg;           // segments of all products
+    int chunk;              // rows a warp claims at once (1 .. 32)
     int64_t *rp_pool;       // row pointers: product m at row_start[m] + m
     int32_t *ci_pool;
     void *val_pool;
@@ -55,12 +66,13 @@ struct BatchArgs {
     int warp_bits;          // rows whose table needs at most 2^warp_bits slots: one warp (<= tw_bits)
     int block_bits;         // ... at most 2^block_bits slots: the whole block (<= tw_bits + 3); larger:
                             // the regular per-product path
-    int dense_max;          // per-warp dense accumulator when cols <= dense_max
+    int warp_bytes;         // shared memory of one warp: its table or dense accumulator
+    int dense_words;        // words of the widest dense accumulator
     HashCfg hc;             // colbits filled per product
     float inv_load;
-    // dense-accumulator rows in one pass: the first phase computes their values
-    // and stages each sorted row at stage_off[g] (room: min(flop, cols)); the
-    // last phase copies it to its exact place (null: two passes, as the rest)
+    // narrow rows take one pass: the first phase computes their values and
+    // stages each sorted row at stage_off[g] (room: min(flop, cols)); the last
+    // phase copies it to its exact place
     const int64_t *stage_off;
     int32_t *stage_ci;
     void *stage_val;
@@ -68,11 +80,13 @@ struct BatchArgs {
     int missing;            // test hook: arrivals a barrier waits for beyond the grid (0: none)
 };
 
-size_t batched_smem(int dtype, int tw_bits);
-int batched_dense_max(int dtype, int tw_bits);
+// Shared memory of a block whose warps have warp_bytes each; wide: some B is
+// too wide for a dense accumulator (its rows take hash tables).
+size_t batched_smem(int dtype, int warp_bytes, bool wide);
+size_t batched_table_bytes(int dtype, int tw_bits);   // a warp's table of 2^tw_bits slots
 void launch_batch_rowinfo(const BatchArgs &p, int sms, cudaStream_t s);
-int batched_grid(int dtype, int tw_bits, int sms);
+int batched_grid(int dtype, int warp_bytes, bool wide, int sms);
 // p_dev: the arguments in device memory (read by every block at start).
-int launch_batched(int dtype, const BatchArgs *p_dev, int tw_bits, int grid, cudaStream_t s);
+int launch_batched(int dtype, const BatchArgs *p_dev, int warp_bytes, bool wide, int grid, cudaStream_t s);
 
 }  // namespace smash

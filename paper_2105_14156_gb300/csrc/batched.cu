@@ -6,6 +6,7 @@
 
 #include "batch_types.h"
 #include "internal.h"
+#include "warp_dense.cuh"
 
 using namespace smash;
 using namespace smash::host;
@@ -26,9 +27,9 @@ struct BatchState {
     cudaStream_t cs = nullptr;       // private stream for graph recording
     cudaGraph_t graph = nullptr;     // the recorded launch, replayed while its key holds
     cudaGraphExec_t exec = nullptr;
-    // what the recorded launch depends on: argument buffer, grid, type, table size
-    const void *key_args = nullptr;
-    int key_grid = 0, key_dt = -1, key_bits = 0;
+    // what the recorded launch depends on: argument and counter buffers, grid, type, shared memory
+    const void *key_args = nullptr, *key_ctr = nullptr;
+    int key_grid = 0, key_dt = -1, key_bytes = 0, key_wide = 0;
 };
 std::map<smash_handle *, BatchState> g_batch;
 
@@ -44,13 +45,14 @@ void drop_graph(BatchState &b) {
 // The persistent launch (with the reset of its work tokens and barrier words)
 // is recorded once as a CUDA graph and replayed on s; its arguments are
 // copied to p_dev before each replay (p_host: pinned). It is recorded again
-// when the argument buffer, grid, type or table size changes; a direct launch
+// when a buffer, the grid, the type or the shared memory changes; a direct launch
 // is the fallback if recording is not possible.
-int run_batched_graph(BatchState &b, int dt, const BatchArgs *p_host, BatchArgs *p_dev, int grid, cudaStream_t s) {
+int run_batched_graph(BatchState &b, int dt, const BatchArgs *p_host, BatchArgs *p_dev, bool wide, int grid,
+                      cudaStream_t s) {
     if (cudaMemcpyAsync(p_dev, p_host, sizeof(BatchArgs), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return SMASH_ERR_CUDA;
-    const bool same = b.exec && b.key_args == p_dev && b.key_grid == grid && b.key_dt == dt &&
-                      b.key_bits == p_host->tw_bits;
+    const bool same = b.exec && b.key_args == p_dev && b.key_ctr == p_host->counters && b.key_grid == grid &&
+                      b.key_dt == dt && b.key_bytes == p_host->warp_bytes && b.key_wide == (wide ? 1 : 0);
     bool ok = true;
     if (!same) {
         drop_graph(b);
@@ -58,16 +60,18 @@ int run_batched_graph(BatchState &b, int dt, const BatchArgs *p_host, BatchArgs 
         if (ok && cudaStreamBeginCapture(b.cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) ok = false;
         if (ok) {
             const bool m = cudaMemsetAsync(p_host->counters + 2, 0, sizeof(int) * 10, b.cs) == cudaSuccess;
-            const int e = launch_batched(dt, p_dev, p_host->tw_bits, grid, b.cs);
+            const int e = launch_batched(dt, p_dev, p_host->warp_bytes, wide, grid, b.cs);
             const bool endok = cudaStreamEndCapture(b.cs, &b.graph) == cudaSuccess;
             ok = m && e == 0 && endok && b.graph;
         }
         if (ok) ok = cudaGraphInstantiate(&b.exec, b.graph, 0) == cudaSuccess;
         if (ok) {
             b.key_args = p_dev;
+            b.key_ctr = p_host->counters;
             b.key_grid = grid;
             b.key_dt = dt;
-            b.key_bits = p_host->tw_bits;
+            b.key_bytes = p_host->warp_bytes;
+            b.key_wide = wide ? 1 : 0;
         }
     }
     if (ok) ok = cudaGraphLaunch(b.exec, s) == cudaSuccess;
@@ -75,7 +79,7 @@ int run_batched_graph(BatchState &b, int dt, const BatchArgs *p_host, BatchArgs 
     cudaGetLastError();
     drop_graph(b);
     if (cudaMemsetAsync(p_host->counters + 2, 0, sizeof(int) * 10, s) != cudaSuccess) return SMASH_ERR_CUDA;
-    if (launch_batched(dt, p_dev, p_host->tw_bits, grid, s) != 0) {
+    if (launch_batched(dt, p_dev, p_host->warp_bytes, wide, grid, s) != 0) {
         cudaGetLastError();
         return SMASH_ERR_CUDA;
     }
@@ -94,10 +98,11 @@ int ensure_pinned(BatchState &b, size_t need) {
 
 struct Layout {
     BatchMat *mats;
-    int64_t *row_start, *tile_start;
+    int64_t *row_start;
     uint8_t *cls;
-    int *ub, *nnz, *big, *huge, *counters;
+    int *ub, *nnz, *big, *huge, *med, *longs, *counters;
     unsigned long long *sums;
+    long long *descents;
     int64_t *base, *totals;
 };
 
@@ -159,13 +164,12 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     if (!h || count < 0 || (count > 0 && (!A || !B || !C))) return SMASH_ERR_INVALID_ARG;
     if (dtype != SMASH_F32 && dtype != SMASH_F64) return SMASH_ERR_UNSUPPORTED;
     int st;
-    int64_t nrows = 0, ntiles = 0;
+    int64_t nrows = 0;
     for (int m = 0; m < count; ++m) {
         if ((st = check_csr(&A[m], true))) return st;
         if ((st = check_csr(&B[m], true))) return st;
         if (A[m].cols != B[m].rows) return SMASH_ERR_SHAPE_MISMATCH;
         nrows += A[m].rows;
-        ntiles += (A[m].rows + kBW - 1) / kBW;
     }
     if (nrows >= (1ll << 31)) return SMASH_ERR_UNSUPPORTED;
     DeviceGuard g(h->device);
@@ -193,14 +197,11 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     size_t need = 0;
     carve_size<BatchMat>(need, count);
     carve_size<int64_t>(need, count + 1);
-    carve_size<int64_t>(need, count + 1);
     carve_size<uint8_t>(need, nrows);
-    carve_size<int>(need, nrows);
-    carve_size<int>(need, nrows);
-    carve_size<int>(need, nrows);
-    carve_size<int>(need, nrows);
-    carve_size<int>(need, 12);
+    for (int q = 0; q < 6; ++q) carve_size<int>(need, nrows);   // ub, nnz, big, huge, med, longs
+    carve_size<int>(need, 16);
     carve_size<unsigned long long>(need, 4);
+    carve_size<long long>(need, count);
     carve_size<int64_t>(need, count + 1);
     carve_size<int64_t>(need, count);
     carve_size<BatchArgs>(need, 1);
@@ -209,25 +210,31 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     Layout L;
     L.mats = c.take<BatchMat>(count);
     L.row_start = c.take<int64_t>(count + 1);
-    L.tile_start = c.take<int64_t>(count + 1);
     L.cls = c.take<uint8_t>(nrows);
     L.ub = c.take<int>(nrows);
     L.nnz = c.take<int>(nrows);
     L.big = c.take<int>(nrows);
     L.huge = c.take<int>(nrows);
-    L.counters = c.take<int>(12);
+    L.med = c.take<int>(nrows);
+    L.longs = c.take<int>(nrows);
+    L.counters = c.take<int>(16);
     L.sums = c.take<unsigned long long>(4);
+    L.descents = c.take<long long>(count);
     L.base = c.take<int64_t>(count + 1);
     L.totals = c.take<int64_t>(count);
     BatchArgs *args_dev = c.take<BatchArgs>(1);
     // descriptors (pinned host -> device)
-    const size_t hbytes = sizeof(BatchMat) * count + 2 * sizeof(int64_t) * (count + 1) + sizeof(BatchArgs) + 64;
+    const size_t hbytes = sizeof(BatchMat) * count + sizeof(int64_t) * (count + 1) + sizeof(BatchArgs) + 64;
     if ((st = ensure_pinned(bs, hbytes + 4096))) return st;
     cudaStreamSynchronize(s);   // the pinned staging may still feed a previous copy
     BatchMat *hm = (BatchMat *)bs.pinned;
     int64_t *hrs = (int64_t *)(hm + count);
-    int64_t *hts = hrs + count + 1;
-    int64_t ro = 0, to = 0;
+    int64_t ro = 0;
+    // a product whose B fits a warp's dense accumulator is narrow, the others
+    // are wide: their rows take hash tables
+    bool wide = false;
+    size_t dense_bytes = 0;
+    int64_t nseg = 0;
     for (int m = 0; m < count; ++m) {
         BatchMat &d = hm[m];
         d.a_rp = A[m].row_ptr;
@@ -241,37 +248,47 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
         d.a_rows = (int32_t)A[m].rows;
         d.b_rows = (int32_t)B[m].rows;
         d.ncols = (int32_t)B[m].cols;
-        d.pad = 0;
+        d.mode = -1;
+        if (B[m].cols * (int64_t)vsz <= kDenseWarpBytes) {
+            d.mode = dense_mode(B[m].nnz, B[m].rows, d.ncols, (int)vsz);
+            const size_t bytes = dense_warp_bytes(d.mode, d.ncols, (int)vsz);
+            if (bytes > dense_bytes) dense_bytes = bytes;
+        } else {
+            wide = true;
+        }
+        d.seg_off = nseg;
+        if (d.mode >= 0)
+            nseg += (B[m].nnz + kSegEntries - 1) / kSegEntries + (B[m].rows + kSegRows - 1) / kSegRows;
         d.row_off = ro;
-        d.tile_off = to;
         hrs[m] = ro;
-        hts[m] = to;
         ro += A[m].rows;
-        to += (A[m].rows + kBW - 1) / kBW;
     }
     hrs[count] = ro;
-    hts[count] = to;
+    size_t warp_bytes = wide ? batched_table_bytes(dt, bs.tw_bits) : 128;
+    if (dense_bytes > warp_bytes) warp_bytes = dense_bytes;
     if (cudaMemcpyAsync(L.mats, hm, sizeof(BatchMat) * count, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(L.row_start, hrs, sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(L.tile_start, hts, sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(L.counters, 0, sizeof(int) * 12, s) != cudaSuccess ||
-        cudaMemsetAsync(L.sums, 0, sizeof(unsigned long long) * 4, s) != cudaSuccess)
+        cudaMemsetAsync(L.counters, 0, sizeof(int) * 16, s) != cudaSuccess ||
+        cudaMemsetAsync(L.sums, 0, sizeof(unsigned long long) * 4, s) != cudaSuccess ||
+        cudaMemsetAsync(L.descents, 0, sizeof(long long) * count, s) != cudaSuccess)
         return SMASH_ERR_CUDA;
     BatchArgs p;
     memset(&p, 0, sizeof(p));
     p.mats = L.mats;
     p.nmat = count;
     p.nrows = nrows;
-    p.ntiles = ntiles;
     p.row_start = L.row_start;
-    p.tile_start = L.tile_start;
     p.cls = L.cls;
     p.ub = L.ub;
     p.nnz = L.nnz;
     p.big = L.big;
     p.huge = L.huge;
+    p.med = L.med;
+    p.longs = L.longs;
     p.counters = L.counters;
     p.sums = L.sums;
+    p.descents = L.descents;
+    p.nseg = nseg;
     p.base = L.base;
     p.totals = L.totals;
     p.err = (int *)h->err.ptr;
@@ -280,24 +297,26 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     p.block_bits = bs.tw_bits + bs.block_more;
     p.wait_spins = bs.wait_spins;
     p.missing = bs.missing;
-    p.dense_max = batched_dense_max(dt, bs.tw_bits);
+    p.warp_bytes = (int)warp_bytes;
+    p.dense_words = (int)(dense_bytes / vsz);
     p.hc = HashCfg{h->params.hash_kind, 0};
     p.inv_load = 1.0f / h->params.max_load;
     {
-        LaunchTimer lt(h, s, "batch_rowinfo", -1, 256, nrows, 0, 0, 0);
+        LaunchTimer lt(h, s, "batch_rowinfo", -1, 256, nrows, 0, 0, 0, 2);
         launch_batch_rowinfo(p, h->sms, s);
     }
     if ((st = last_cuda_status())) return st;
     // sizes for the pools
     char *hb = (char *)h->host;
-    if (cudaMemcpyAsync(hb, L.counters, sizeof(int) * 2, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(hb, L.counters, sizeof(int) * 16, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaMemcpyAsync(hb + 64, L.sums, sizeof(unsigned long long) * 2, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return SMASH_ERR_CUDA;
-    int nbig, nhuge;
+    int nbig, nhuge, nmed;
     unsigned long long sum_ub, sum_f;
     memcpy(&nbig, hb, 4);
     memcpy(&nhuge, hb + 4, 4);
+    memcpy(&nmed, hb + 48, 4);
     memcpy(&sum_ub, hb + 64, 8);
     memcpy(&sum_f, hb + 72, 8);
     ls.big_rows = nbig;
@@ -316,11 +335,8 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     p.rp_pool = rp_pool;
     p.ci_pool = ci_pool;
     p.val_pool = val_pool;
-    // staging of the one-pass (dense-accumulator) rows: room min(flop, cols)
-    // per row at the exclusive prefix of those rooms
-    p.stage_off = nullptr;
-    p.stage_ci = nullptr;
-    p.stage_val = nullptr;
+    // staging of the narrow products' rows (one pass): room min(flop, cols) per
+    // row at the exclusive prefix of those rooms
     {
         size_t need = 0;
         carve_size<int64_t>(need, (size_t)nrows + 1);
@@ -392,16 +408,19 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
         }
     }
     // the persistent launch
-    const int grid_max = batched_grid(dt, bs.tw_bits, h->sms);
-    const long long items = (long long)nbig + ntiles;
+    const int grid_max = batched_grid(dt, p.warp_bytes, wide, h->sms);
+    // rows a warp claims at once: four claims per warp of a full grid
+    const long long share = nrows / ((long long)grid_max * kBW * 4 + 1);
+    p.chunk = share < 1 ? 1 : share > 32 ? 32 : (int)share;
+    const long long items = nbig + (nmed + (nrows + p.chunk - 1) / p.chunk + kBW - 1) / kBW;
     int grid = (int)(items < grid_max ? items : grid_max);
     if (grid < 1) grid = 1;
     {
         LaunchTimer lt(h, s, "batched_persistent", -1, 256, nrows, 0, (long long)sum_f, 0);
         // the arguments through pinned memory, after the descriptors
-        BatchArgs *p_pin = (BatchArgs *)(((uintptr_t)(hts + count + 1) + 63) & ~(uintptr_t)63);
+        BatchArgs *p_pin = (BatchArgs *)(((uintptr_t)(hrs + count + 1) + 63) & ~(uintptr_t)63);
         *p_pin = p;
-        if ((st = run_batched_graph(bs, dt, p_pin, args_dev, grid, s))) return fail(st);
+        if ((st = run_batched_graph(bs, dt, p_pin, args_dev, wide, grid, s))) return fail(st);
     }
     // a barrier that ran out of time (or any failed check) leaves the row
     // pointers incomplete: stop before anything reads them
@@ -461,7 +480,8 @@ int smash_batched_autotune(smash_handle *h, int count, const smash_csr *A, const
     // threads per row) and by the whole block (256 threads per row)
     for (int cand = 0; cand < 4 * 2 * 2; ++cand) {
         const int bits = 8 + cand / 4, wl = (cand >> 1) & 1, bm = 2 + (cand & 1);
-        if (batched_smem(dtype == SMASH_F64, bits) > (size_t)max_smem_per_block()) continue;
+        const int dt = dtype == SMASH_F64 ? 1 : 0;
+        if (batched_smem(dt, (int)batched_table_bytes(dt, bits), true) > (size_t)max_smem_per_block()) continue;
         bst.tw_bits = bits;
         bst.warp_less = wl;
         bst.block_more = bm;

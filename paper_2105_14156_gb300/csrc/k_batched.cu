@@ -6,20 +6,26 @@
 // schedule) across products: every block repeatedly claims the next work item
 // of a global list with one atomic add, so products of very different sizes
 // keep all SMs busy. Items are (a) single large rows, processed by the whole
-// block with one block-wide hash table, listed first so they start early, and
-// (b) tiles of 8 consecutive rows of one product, one row per warp, each warp
-// with its own accumulator: a dense array over the columns of B when B is
-// narrow (the paper's "dense row"), else a small hash table.
+// block, listed first so they start early, (b) medium rows, one warp each, and
+// (c) chunks of consecutive rows, claimed by a warp. A row's accumulator is
+// a dense array over the columns of B when B is narrow (warp_dense.cuh), one
+// per warp, else a hash table.
+//
+// Why three sizes: with all rows of narrow products in chunks of 32, the 32
+// heaviest rows of a skewed graph fell to one warp, and every other block
+// waited for it at the grid barrier (36 of 53 stall cycles per issue; 1 of 12
+// now).
 //
 // One cooperative launch runs four phases separated by grid barriers (each
 // wait bounded; a barrier that times out sets an error word and the kernel
-// returns): symbolic counts, per-product row-pointer scans, product base
+// returns): counts (and the values of narrow products' rows), per-product row-pointer scans, product base
 // offsets, numeric values with sorted write-out. Rows too large for one
 // block's table are done around the kernel by the regular per-product path.
 #include "device_common.cuh"
 #include "kernels.h"
 #include "writeout.cuh"
 #include "batch_types.h"
+#include "warp_dense.cuh"
 
 namespace smash {
 
@@ -56,49 +62,135 @@ __device__ __forceinline__ int colbits(int n) {
     return b;
 }
 
-// Row classification over all products' rows (one warp per row).
-__global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p) {
+// Row classification over all products' rows. One thread per row, four
+// entries in flight; rows of more than kLongBatchRow entries go to a list that
+// k_batch_rowinfo_long spreads over all warps, a warp per row (the long rows of
+// a skewed graph sit together: counted by the warp that finds them they took
+// 0.24 ms of the 512-product batch).
+constexpr int kLongBatchRow = 48;
+
+__device__ __forceinline__ long long batch_b_len(const BatchMat &M, int k, int *err) {
+    if ((unsigned)k >= (unsigned)M.b_rows) {
+        raise_err(err, kErrBadIndex);
+        return 0;
+    }
+    const int64_t s = __ldg(M.b_rp + k), t = __ldg(M.b_rp + k + 1);
+    if (s >= 0 && t >= s && t <= M.b_nnz) return t - s;
+    raise_err(err, kErrBadRowPtr);
+    return 0;
+}
+
+// Class, room and lists of row g with f products; returns its room.
+__device__ __forceinline__ long long batch_classify(const BatchArgs &p, const BatchMat &M, int64_t g, long long f) {
+    const long long ub = f < (long long)M.ncols ? f : (long long)M.ncols;
+    uint8_t c;
+    if (ub == 0) c = kRowEmpty;
+    else if (M.mode >= 0) c = f <= kMedFlop ? kRowSmall : f <= kBigFlop ? kRowMed : kRowBig;
+    else if (table_bits(ub, p.inv_load) <= p.warp_bits) c = kRowSmall;
+    else if (table_bits(ub, p.inv_load) <= p.block_bits) c = kRowBig;
+    else c = kRowHuge;
+    p.cls[g] = c;
+    p.ub[g] = (int)ub;
+    p.nnz[g] = 0;
+    if (c == kRowBig) p.big[atomicAdd(p.counters + 0, 1)] = (int)g;
+    if (c == kRowHuge) p.huge[atomicAdd(p.counters + 1, 1)] = (int)g;
+    if (c == kRowMed) p.med[atomicAdd(p.counters + 12, 1)] = (int)g;
+    return ub;
+}
+
+// The first row_blocks blocks count rows, the others pass over the narrow
+// products' B (whether its rows ascend).
+__global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p, int row_blocks) {
     const int lane = lane_id();
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    if ((int)blockIdx.x >= row_blocks) {
+        for (int64_t q = blockIdx.x - row_blocks; q < p.nseg; q += gridDim.x - row_blocks) {
+            int lo = 0, hi = p.nmat;   // last product whose segments start at or before q
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (p.mats[mid].seg_off <= q) lo = mid;
+                else hi = mid;
+            }
+            const BatchMat &M = p.mats[lo];
+            int64_t x = q - M.seg_off;
+            const int64_t eseg = (M.b_nnz + kSegEntries - 1) / kSegEntries;
+            long long d;
+            if (x < eseg) {
+                const int64_t e0 = x * kSegEntries;
+                const int64_t e1 = e0 + kSegEntries < M.b_nnz ? e0 + kSegEntries : M.b_nnz;
+                d = descents_between(M.b_ci, e0, e1, M.ncols, threadIdx.x, 256);
+            } else {
+                const int64_t r0 = (x - eseg) * kSegRows;
+                const int64_t r1 = r0 + kSegRows < M.b_rows ? r0 + kSegRows : M.b_rows;
+                d = -descents_at_starts(M.b_rp, M.b_ci, M.b_nnz, r0, r1, threadIdx.x, 256);
+            }
+            d = warp_sum(d);
+            if (lane == 0 && d) atomicAdd((unsigned long long *)p.descents + lo, (unsigned long long)d);
+        }
+        return;
+    }
+    const int64_t threads = (int64_t)row_blocks * blockDim.x;
     unsigned long long my_ub = 0, my_f = 0;
-    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < p.nrows; g += warps) {
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < p.nrows; g += threads) {
         const int mi = find_mat(p.row_start, p.nmat, g);
         const BatchMat &M = p.mats[mi];
         const int64_t r = g - p.row_start[mi];
         int64_t ab = __ldg(M.a_rp + r), ae = __ldg(M.a_rp + r + 1);
         if (ab < 0 || ae < ab || ae > M.a_nnz) {
-            if (lane == 0) raise_err(p.err, kErrBadRowPtr);
+            raise_err(p.err, kErrBadRowPtr);
             ab = ae = 0;
         }
-        long long f = 0;
-        for (int64_t e = ab + lane; e < ae; e += 32) {
-            const int k = __ldg(M.a_ci + e);
-            if ((unsigned)k < (unsigned)M.b_rows) {
-                const int64_t s = __ldg(M.b_rp + k), t = __ldg(M.b_rp + k + 1);
-                if (s >= 0 && t >= s && t <= M.b_nnz) f += t - s;
-                else raise_err(p.err, kErrBadRowPtr);
-            } else {
-                raise_err(p.err, kErrBadIndex);
-            }
+        if (ae - ab > kLongBatchRow) {
+            p.longs[atomicAdd(p.counters + 13, 1)] = (int)g;
+            continue;
         }
+        long long f = 0;
+        for (int64_t e = ab; e < ae; e += 4) {
+            int k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = e + u < ae ? __ldg(M.a_ci + e + u) : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (e + u < ae) f += batch_b_len(M, k[u], p.err);
+        }
+        my_ub += (unsigned long long)batch_classify(p, M, g, f);
+        my_f += (unsigned long long)f;
+    }
+    my_ub = warp_sum(my_ub);
+    my_f = warp_sum(my_f);
+    if (lane == 0) {
+        atomicAdd(p.sums + 0, my_ub);
+        atomicAdd(p.sums + 1, my_f);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_batch_rowinfo_long(BatchArgs p) {
+    const int lane = lane_id();
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int n = p.counters[13];
+    unsigned long long my_ub = 0, my_f = 0;
+    for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n; q += warps) {
+        const int64_t g = p.longs[q];
+        const int mi = find_mat(p.row_start, p.nmat, g);
+        const BatchMat &M = p.mats[mi];
+        const int64_t r = g - p.row_start[mi];
+        const int64_t ab = __ldg(M.a_rp + r), ae = __ldg(M.a_rp + r + 1);   // checked by k_batch_rowinfo
+        long long f = 0;
+        for (int64_t e0 = ab + lane; e0 < ae; e0 += 128) {
+            int k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = e0 + 32 * u < ae ? __ldg(M.a_ci + e0 + 32 * u) : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (e0 + 32 * u < ae) f += batch_b_len(M, k[u], p.err);
+        }
+        __syncwarp();
         f = warp_sum(f);
         if (lane == 0) {
-            const long long ub = f < (long long)M.ncols ? f : (long long)M.ncols;
-            uint8_t c;
-            if (ub == 0) c = kRowEmpty;
-            else if (M.ncols <= p.dense_max || table_bits(ub, p.inv_load) <= p.warp_bits) c = kRowSmall;
-            else if (table_bits(ub, p.inv_load) <= p.block_bits) c = kRowBig;
-            else c = kRowHuge;
-            p.cls[g] = c;
-            p.ub[g] = (int)ub;
-            p.nnz[g] = 0;
-            if (c == kRowBig) p.big[atomicAdd(p.counters + 0, 1)] = (int)g;
-            if (c == kRowHuge) p.huge[atomicAdd(p.counters + 1, 1)] = (int)g;
-            my_ub += (unsigned long long)ub;
+            my_ub += (unsigned long long)batch_classify(p, M, g, f);
             my_f += (unsigned long long)f;
         }
     }
-    if (lane == 0) {
+    if (lane == 0 && my_f) {
         atomicAdd(p.sums + 0, my_ub);
         atomicAdd(p.sums + 1, my_f);
     }
@@ -144,7 +236,66 @@ struct BatchSmem {
     ProdScratch<V> sc;      // block-wide product staging
 };
 
-// One small row by one warp: count (NUM = false) or values + write-out.
+// A row of a narrow product: values, count and the sorted row (staged), by one
+// warp whose dense accumulator is acc.
+template <typename V>
+__device__ __forceinline__ void narrow_emit(const BatchArgs &p, const BatchMat &M, int64_t g, V *acc) {
+    const int64_t so = p.stage_off[g];
+    const int room = p.ub[g];
+    int32_t *ci = p.stage_ci + so;
+    V *val = (V *)p.stage_val + so;
+    const int n = dense_emit(acc, M.mode, M.ncols, [&](int pos, int j, V v) {
+        if (pos < room) {
+            ci[pos] = j;
+            val[pos] = v;
+        }
+    });
+    if (lane_id() == 0) {
+        p.nnz[g] = n < room ? n : room;
+        if (n > room) raise_err(p.err, kErrTableFull);
+    }
+}
+
+template <typename V>
+__device__ __forceinline__ void narrow_row(const BatchArgs &p, const BatchMat &M, int mi, int64_t g, int64_t r,
+                                           V *acc) {
+    const Operands<V> op = mat_ops<V>(M);
+    int64_t ab, ae;
+    a_row_range(op, r, ab, ae, p.err);
+    dense_accumulate(op, M.mode, p.descents[mi] == 0, ab, ae, 32, acc, p.err);
+    narrow_emit(p, M, g, acc);
+}
+
+// The same by the whole block: every warp takes each kBW-th batch of 32
+// entries of the row, the warps' accumulators are added up in the first
+// warp's, which writes the row out.
+template <typename V>
+__device__ void narrow_block_row(const BatchArgs &p, const BatchMat &M, int mi, int64_t g, int64_t r,
+                                 unsigned char *tab) {
+    const Operands<V> op = mat_ops<V>(M);
+    const int w = threadIdx.x >> 5;
+    int64_t ab, ae;
+    a_row_range(op, r, ab, ae, p.err);
+    dense_accumulate(op, M.mode, p.descents[mi] == 0, ab + 32 * w, ae, 32 * kBW, (V *)(tab + (size_t)w * p.warp_bytes),
+                     p.err);
+    __syncthreads();
+    const int words = dense_copies(M.mode) * dense_stride(M.ncols);
+    for (int x = threadIdx.x; x < words; x += kBNT) {
+        V v = ((V *)tab)[x];
+        for (int q = 1; q < kBW; ++q) {
+            V *o = (V *)(tab + (size_t)q * p.warp_bytes) + x;
+            v += *o;
+            *o = dense_unused(V(0));
+        }
+        ((V *)tab)[x] = v;
+    }
+    __syncthreads();
+    if (w == 0) narrow_emit(p, M, g, (V *)tab);
+    __syncthreads();
+}
+
+// One small row of a wide product by one warp: count (NUM = false) or values
+// + write-out.
 template <typename V, bool NUM>
 __device__ void warp_row(const BatchArgs &p, const BatchMat &M, int64_t g, int64_t r, unsigned char *wtab, int64_t c0,
                          int n_exp, int64_t base) {
@@ -153,90 +304,6 @@ __device__ void warp_row(const BatchArgs &p, const BatchMat &M, int64_t g, int64
     int64_t ab, ae;
     a_row_range(op, r, ab, ae, p.err);
     const int T = 1 << p.tw_bits;
-    if (M.ncols <= p.dense_max && NUM && p.stage_ci) {
-        // one-pass row: copy the row staged by the first phase to its place
-        const int64_t so = p.stage_off[g];
-        for (int q = lane; q < n_exp; q += 32) {
-            p.ci_pool[base + c0 + q] = p.stage_ci[so + q];
-            ((V *)p.val_pool)[base + c0 + q] = ((const V *)p.stage_val)[so + q];
-        }
-        return;
-    }
-    if (M.ncols <= p.dense_max && !NUM && p.stage_ci) {
-        // one-pass row: values, count and the sorted row (staged) at once
-        const int words = (M.ncols + 31) >> 5;
-        V *acc = (V *)wtab;
-        unsigned *bm = (unsigned *)(wtab + (((size_t)M.ncols * sizeof(V) + 15) & ~(size_t)15));
-        for (int w = lane; w < words; w += 32) bm[w] = 0u;
-        for (int j = lane; j < M.ncols; j += 32) acc[j] = V(0);
-        __syncwarp();
-        warp_products<V, true>(op, ab, ae, p.err, [&](int j, V a, V bkj) {
-            atomicAdd(acc + j, a * bkj);
-            const unsigned bit = 1u << (j & 31);
-            if (!(*(volatile unsigned *)(bm + (j >> 5)) & bit)) atomicOr(bm + (j >> 5), bit);
-        });
-        __syncwarp();
-        const int64_t so = p.stage_off[g];
-        const int room = p.ub[g];
-        int run = 0;
-        for (int w = 0; w < words; ++w) {
-            const unsigned bits = bm[w];
-            const int j = (w << 5) + lane;
-            if ((bits >> lane) & 1u) {
-                const int pos = run + __popc(bits & lanemask_lt());
-                if (pos < room) {
-                    p.stage_ci[so + pos] = j;
-                    ((V *)p.stage_val)[so + pos] = acc[j];
-                }
-            }
-            run += __popc(bits);
-        }
-        if (lane == 0) {
-            p.nnz[g] = run;
-            if (run > room) raise_err(p.err, kErrTableFull);
-        }
-        __syncwarp();
-        return;
-    }
-    if (M.ncols <= p.dense_max) {
-        // dense accumulator over the columns of B (values, then the bitmap)
-        const int words = (M.ncols + 31) >> 5;
-        V *acc = (V *)wtab;
-        unsigned *bm = (unsigned *)(wtab + (((size_t)M.ncols * sizeof(V) + 15) & ~(size_t)15));
-        for (int w = lane; w < words; w += 32) bm[w] = 0u;
-        if (NUM)
-            for (int j = lane; j < M.ncols; j += 32) acc[j] = V(0);
-        __syncwarp();
-        warp_products<V, NUM>(op, ab, ae, p.err, [&](int j, V a, V bkj) {
-            if (NUM) atomicAdd(acc + j, a * bkj);
-            const unsigned bit = 1u << (j & 31);
-            if (!(*(volatile unsigned *)(bm + (j >> 5)) & bit)) atomicOr(bm + (j >> 5), bit);
-        });
-        __syncwarp();
-        if (!NUM) {
-            int c = 0;
-            for (int w = lane; w < words; w += 32) c += __popc(bm[w]);
-            c = warp_sum(c);
-            if (lane == 0) p.nnz[g] = c;
-        } else {
-            int run = 0;
-            for (int w = 0; w < words; ++w) {
-                const unsigned bits = bm[w];
-                const int j = (w << 5) + lane;
-                if ((bits >> lane) & 1u) {
-                    const int pos = run + __popc(bits & lanemask_lt());
-                    if (pos < n_exp) {
-                        p.ci_pool[base + c0 + pos] = j;
-                        ((V *)p.val_pool)[base + c0 + pos] = acc[j];
-                    }
-                }
-                run += __popc(bits);
-            }
-            if (lane == 0 && run != n_exp) raise_err(p.err, kErrCountMismatch);
-        }
-        __syncwarp();
-        return;
-    }
     // hash table of the warp
     const int tb = table_bits(p.ub[g], p.inv_load);
     const int Tr = 1 << tb;
@@ -315,71 +382,147 @@ __device__ void block_row(const BatchArgs &p, const BatchMat &M, int64_t g, int6
     __syncthreads();
 }
 
-// Work of one phase: the big rows first, one per block (claimed with one
-// counter); then every warp claims chunks of 32 consecutive rows of the
-// flattened row space on its own (a second counter) and serves the small rows
-// among them, with no block-wide wait between rows of unequal cost.
-constexpr int kRowChunk = 32;
-
-template <typename V, bool NUM>
-__device__ bool run_items(const BatchArgs &p, int *token, int *chunks, const BatchSmem<V> &sm, int nbig) {
-    __shared__ long long s_item;
+// Work of one phase: the big rows first, one per block, then the medium rows,
+// one per warp (claimed with one counter each); then every warp claims chunks
+// of consecutive rows of the flattened row space on its own (32, fewer when
+// that would leave warps without work) and serves the small rows among them,
+// with no block-wide wait between rows of unequal cost.
+// The rows of narrow products are computed and staged in the first phase
+// (NUM = false) and copied to their places in the last (NUM = true), a chunk's
+// rows one after another, four loads per lane in flight.
+template <typename V, bool NUM, bool WIDE>
+__device__ void run_items(const BatchArgs &p, const BatchSmem<V> &sm) {
+    __shared__ int s_item;
     const int w = threadIdx.x >> 5;
     const int lane = lane_id();
-    const size_t wbytes = ((size_t)1 << p.tw_bits) * (4 + sizeof(V));
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(token, 1);
-        __syncthreads();
-        const long long it = s_item;
-        __syncthreads();
-        if (it >= nbig) break;
-        const int64_t g = p.big[it];
-        const int mi = find_mat(p.row_start, p.nmat, g);
-        const BatchMat &M = p.mats[mi];
-        const int64_t r = g - p.row_start[mi];
-        int64_t c0 = 0;
-        int n_exp = 0;
-        int64_t base = 0;
-        if (NUM) {
-            const int64_t *rp = p.rp_pool + p.row_start[mi] + mi;
-            c0 = rp[r];
-            n_exp = (int)(rp[r + 1] - rp[r]);
-            base = p.base[mi];
-        }
-        block_row<V, NUM>(p, M, g, r, sm, c0, n_exp, base);
-    }
-    // small rows: `chunks` counts the chunks of kRowChunk rows handed out
-    unsigned char *wtab = sm.tab + (size_t)w * wbytes;
-    for (;;) {
-        int ch = 0;
-        if (lane == 0) ch = atomicAdd(chunks, 1);
-        ch = __shfl_sync(kFull, ch, 0);
-        const int64_t g0 = (int64_t)ch * kRowChunk;
-        if (g0 >= p.nrows) break;
-        const int64_t g1 = g0 + kRowChunk < p.nrows ? g0 + kRowChunk : p.nrows;
-        // the small rows of the chunk, one at a time
-        const bool mine = g0 + lane < g1 && p.cls[g0 + lane] == kRowSmall;
-        for (unsigned todo = __ballot_sync(kFull, mine); todo; todo &= todo - 1) {
-            const int64_t g = g0 + __ffs(todo) - 1;
+    const int nbig = p.counters[0];
+    unsigned char *wtab = sm.tab + (size_t)w * p.warp_bytes;
+    V *acc = (V *)wtab;
+    bool clean = false;   // the dense accumulator's words are unused (a hash table shares its room)
+    if (!NUM || WIDE) {
+        for (;;) {
+            if (threadIdx.x == 0) s_item = atomicAdd(p.counters + (NUM ? 3 : 2), 1);
+            __syncthreads();
+            const int it = s_item;
+            __syncthreads();
+            if (it >= nbig) break;
+            const int64_t g = p.big[it];
             const int mi = find_mat(p.row_start, p.nmat, g);
             const BatchMat &M = p.mats[mi];
             const int64_t r = g - p.row_start[mi];
-            int64_t c0 = 0;
-            int n_exp = 0;
-            int64_t base = 0;
-            if (NUM) {
-                const int64_t *rp = p.rp_pool + p.row_start[mi] + mi;
-                c0 = rp[r];
-                n_exp = (int)(rp[r + 1] - rp[r]);
-                base = p.base[mi];
+            if (M.mode >= 0) {
+                if (!NUM) {
+                    if (!clean) dense_clear(acc, p.dense_words);
+                    clean = true;
+                    __syncthreads();
+                    narrow_block_row<V>(p, M, mi, g, r, sm.tab);
+                }
+            } else if constexpr (WIDE) {
+                int64_t c0 = 0;
+                int n_exp = 0;
+                int64_t base = 0;
+                if (NUM) {
+                    const int64_t *rp = p.rp_pool + p.row_start[mi] + mi;
+                    c0 = rp[r];
+                    n_exp = (int)(rp[r + 1] - rp[r]);
+                    base = p.base[mi];
+                }
+                clean = false;
+                block_row<V, NUM>(p, M, g, r, sm, c0, n_exp, base);
             }
-            warp_row<V, NUM>(p, M, g, r, wtab, c0, n_exp, base);
         }
     }
-    return true;
+    if (!NUM) {
+        const int nmed = p.counters[12];
+        for (;;) {
+            int it = 0;
+            if (lane == 0) it = atomicAdd(p.counters + 4, 1);
+            it = __shfl_sync(kFull, it, 0);
+            if (it >= nmed) break;
+            const int64_t g = p.med[it];
+            const int mi = find_mat(p.row_start, p.nmat, g);
+            if (!clean) dense_clear(acc, p.dense_words);
+            clean = true;
+            __syncwarp();
+            narrow_row<V>(p, p.mats[mi], mi, g, g - p.row_start[mi], acc);
+        }
+    }
+    for (;;) {
+        int ch = 0;
+        if (lane == 0) ch = atomicAdd(p.counters + (NUM ? 9 : 8), 1);
+        ch = __shfl_sync(kFull, ch, 0);
+        const int64_t g0 = (int64_t)ch * p.chunk;
+        if (g0 >= p.nrows) break;
+        // lane l: row g0 + l, its product and, in the last phase, its places
+        const int64_t gl = g0 + lane;
+        const int cls = lane < p.chunk && gl < p.nrows ? p.cls[gl] : kRowEmpty;
+        int ml = 0, nl = 0;
+        bool narrow = false;
+        int64_t dl = 0, sl = 0;
+        if (cls != kRowEmpty) {
+            ml = find_mat(p.row_start, p.nmat, gl);
+            narrow = p.mats[ml].mode >= 0;
+            if (NUM && narrow) {
+                dl = p.base[ml] + p.rp_pool[gl + ml];
+                sl = p.stage_off[gl];
+                nl = p.nnz[gl];
+            }
+        }
+        if (NUM) {
+            for (unsigned todo = __ballot_sync(kFull, narrow); todo; todo &= todo - 1) {
+                const int x = __ffs(todo) - 1;
+                const int n = __shfl_sync(kFull, nl, x);
+                const int64_t d = __shfl_sync(kFull, dl, x), s = __shfl_sync(kFull, sl, x);
+                for (int q0 = lane; q0 < n; q0 += 128) {
+                    int32_t c[4];
+                    V v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (q0 + 32 * u < n) {
+                            c[u] = p.stage_ci[s + q0 + 32 * u];
+                            v[u] = ((const V *)p.stage_val)[s + q0 + 32 * u];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (q0 + 32 * u < n) {
+                            p.ci_pool[d + q0 + 32 * u] = c[u];
+                            ((V *)p.val_pool)[d + q0 + 32 * u] = v[u];
+                        }
+                    }
+                }
+            }
+        }
+        for (unsigned todo = __ballot_sync(kFull, cls == kRowSmall && (WIDE || !NUM) && !(NUM && narrow)); todo;
+             todo &= todo - 1) {
+            const int x = __ffs(todo) - 1;
+            const int64_t g = g0 + x;
+            const int mi = __shfl_sync(kFull, ml, x);
+            const BatchMat &M = p.mats[mi];
+            const int64_t r = g - p.row_start[mi];
+            if (!WIDE || M.mode >= 0) {
+                if (!clean) dense_clear(acc, p.dense_words);
+                clean = true;
+                __syncwarp();
+                narrow_row<V>(p, M, mi, g, r, acc);
+            } else if constexpr (WIDE) {
+                int64_t c0 = 0;
+                int n_exp = 0;
+                int64_t base = 0;
+                if (NUM) {
+                    const int64_t *rp = p.rp_pool + p.row_start[mi] + mi;
+                    c0 = rp[r];
+                    n_exp = (int)(rp[r + 1] - rp[r]);
+                    base = p.base[mi];
+                }
+                clean = false;
+                warp_row<V, NUM>(p, M, g, r, wtab, c0, n_exp, base);
+            }
+        }
+    }
 }
 
-template <typename V>
+template <typename V, bool WIDE>
 __global__ void __launch_bounds__(kBNT) k_batched(const BatchArgs *pp) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_w[32];
@@ -391,12 +534,10 @@ __global__ void __launch_bounds__(kBNT) k_batched(const BatchArgs *pp) {
     const BatchArgs &p = s_p;
     BatchSmem<V> sm;
     sm.tab = smem;
-    const size_t tab_bytes = ((size_t)kBW << p.tw_bits) * (4 + sizeof(V));
-    sm.sc = carve_prod_scratch<V, kBNT>(smem + tab_bytes);
-    const int nbig = p.counters[0];
+    sm.sc = carve_prod_scratch<V, kBNT>(smem + (size_t)kBW * p.warp_bytes);
     int *bar = p.counters + 6;
-    // phase 1: symbolic counts
-    run_items<V, false>(p, p.counters + 2, p.counters + 8, sm, nbig);
+    // phase 1: counts (rows of narrow products: values too, staged)
+    run_items<V, false, WIDE>(p, sm);
     if (!grid_barrier(bar, p.err, p.wait_spins, p.missing)) return;
     // phase 2: row pointers of each product (one product per block at a time)
     __shared__ int s_m;
@@ -452,60 +593,54 @@ __global__ void __launch_bounds__(kBNT) k_batched(const BatchArgs *pp) {
     }
     if (!grid_barrier(bar, p.err, p.wait_spins, p.missing)) return;
     // phase 4: values
-    run_items<V, true>(p, p.counters + 3, p.counters + 9, sm, nbig);
+    run_items<V, true, WIDE>(p, sm);
 }
 
 // ---------------------------------------------------------------------------
-size_t batched_smem(int dtype, int tw_bits) {
-    const size_t vs = dtype ? 8 : 4;
-    const size_t sc = dtype ? num_scratch_bytes<double, kBNT>() : num_scratch_bytes<float, kBNT>();
-    return ((size_t)kBW << tw_bits) * (4 + vs) + sc;
-}
+size_t batched_table_bytes(int dtype, int tw_bits) { return ((size_t)1 << tw_bits) * (dtype ? 12 : 8); }
 
-int batched_dense_max(int dtype, int tw_bits) {
-    const size_t vs = dtype ? 8 : 4;
-    const size_t wbytes = ((size_t)1 << tw_bits) * (4 + vs);
-    // values (rounded to 16 bytes) + bitmap must fit one warp's table
-    long long c = (long long)((wbytes - 16) * 8 / (8 * vs + 1));
-    c &= ~31ll;
-    return (int)c;
+size_t batched_smem(int dtype, int warp_bytes, bool wide) {
+    const size_t sc = dtype ? num_scratch_bytes<double, kBNT>() : num_scratch_bytes<float, kBNT>();
+    return (size_t)kBW * warp_bytes + (wide ? sc : 0);
 }
 
 void launch_batch_rowinfo(const BatchArgs &p, int sms, cudaStream_t s) {
     if (p.nrows == 0) return;
-    const int64_t blocks = (p.nrows + 7) / 8;
+    const int64_t blocks = (p.nrows + 255) / 256;
     const int64_t cap = (int64_t)sms * 8;
-    k_batch_rowinfo<<<(int)(blocks < cap ? blocks : cap), 256, 0, s>>>(p);
+    const int rb = (int)(blocks < cap ? blocks : cap);
+    const int64_t seg_cap = (int64_t)sms * 4;
+    k_batch_rowinfo<<<rb + (int)(p.nseg < seg_cap ? p.nseg : seg_cap), 256, 0, s>>>(p, rb);
+    k_batch_rowinfo_long<<<(int)(blocks < sms ? blocks : sms) * 4, 256, 0, s>>>(p);
 }
 
-int batched_grid(int dtype, int tw_bits, int sms) {
-    const size_t smem = batched_smem(dtype, tw_bits);
+using BatchKernel = void (*)(const BatchArgs *);
+static BatchKernel batched_kernel(int dtype, bool wide) {
+    if (dtype) return wide ? (BatchKernel)k_batched<double, true> : (BatchKernel)k_batched<double, false>;
+    return wide ? (BatchKernel)k_batched<float, true> : (BatchKernel)k_batched<float, false>;
+}
+
+int batched_grid(int dtype, int warp_bytes, bool wide, int sms) {
+    const size_t smem = batched_smem(dtype, warp_bytes, wide);
+    BatchKernel k = batched_kernel(dtype, wide);
     int per = 0;
-    if (dtype) {
-        cudaFuncSetAttribute(k_batched<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batched<double>, kBNT, smem);
-    } else {
-        cudaFuncSetAttribute(k_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batched<float>, kBNT, smem);
-    }
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kBNT, smem);
     return per * sms;
 }
 
-int launch_batched(int dtype, const BatchArgs *p_dev, int tw_bits, int grid, cudaStream_t s) {
-    const size_t smem = batched_smem(dtype, tw_bits);
+int launch_batched(int dtype, const BatchArgs *p_dev, int warp_bytes, bool wide, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(kBNT, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = batched_smem(dtype, warp_bytes, wide);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e;
-    if (dtype) e = cudaLaunchKernelEx(&cfg, k_batched<double>, p_dev);
-    else e = cudaLaunchKernelEx(&cfg, k_batched<float>, p_dev);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, batched_kernel(dtype, wide), p_dev);
     return e == cudaSuccess ? 0 : (int)e;
 }
 

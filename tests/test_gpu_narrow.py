@@ -1,0 +1,105 @@
+"""Products whose B is narrow enough for a warp's dense accumulator, at the
+sizes where its lane groups, its unrolled steps and its choice of rows can go
+wrong: mean row lengths of B on both sides of each group width, rows of B of
+one to many steps, column counts around a multiple of 32 and around the widest
+accumulator, rows of A for a chunk, a warp and a block, unsorted and repeated
+columns. Values are held to |c - c*| <= tol * sum |a||b| (1e-5 float32, 1e-12
+float64: the bounds (m - 1) * 2^-24 and (m - 1) * 2^-53 of m-term sums in any
+order stay below them for the m <= 100 here; small integers must be exact)."""
+import numpy as np
+import pytest
+
+from paper_2105_14156_gb300.rmat import Csr, csr_from_coo
+from tests.gpu_util import assert_matches_oracle
+from tests.helpers import random_csr
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def handle():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2105_14156_gb300 import build, smash
+    build.build()
+    h = smash.Handle(0)
+    yield h
+    h.close()
+
+
+def rows_of(lens, cols, values, seed):
+    """A CSR matrix whose row r holds lens[r] distinct, ascending columns."""
+    rng = np.random.default_rng(seed)
+    r = np.repeat(np.arange(len(lens)), lens)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lens]) if sum(lens) else np.zeros(0, np.int64)
+    rp, ci = csr_from_coo(len(lens), cols, r, c)
+    if values == "int":
+        val = rng.integers(1, 5, ci.size).astype(np.float32)
+    else:
+        val = rng.uniform(-1, 1, ci.size).astype(np.float32 if values == "f32" else np.float64)
+    return Csr(len(lens), cols, rp, ci, val)
+
+
+def skewed_rows(n, k, values, seed, longest):
+    """n rows of 0 .. ~10 entries, one of `longest` and one of all k."""
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(0, min(k, 10) + 1, n)
+    lens[n // 3] = min(k, longest)
+    lens[n - 1] = k
+    return rows_of(lens.tolist(), k, values, seed + 1)
+
+
+# (cols, entries per row of B): every lane-group width, rows of one step, of
+# two, and of more, and the widest accumulators
+B_SHAPES = [(1, [1]), (31, [1, 2]), (32, [0, 4, 8]), (33, [6, 9, 16]), (100, [8, 17]), (256, [12, 16, 33]),
+            (300, [15, 16, 17, 32, 33, 130]), (1000, [40, 64, 65, 129, 600]), (3072, [30, 700]), (3073, [30]),
+            (6144, [30, 2000]), (6145, [30])]
+
+
+def b_matrix(cols, lens, k, values, seed):
+    return rows_of([min(lens[q % len(lens)], cols) for q in range(k)], cols, values, seed)
+
+
+def run_batch(handle, pairs):
+    from paper_2105_14156_gb300 import smash
+    dev = [(smash.to_device(A), smash.to_device(B)) for A, B in pairs]
+    Cs, _, owner = handle.spgemm_batched(dev)
+    host = [C.to_host() for C in Cs]
+    owner.free()
+    return host
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+def test_batched_narrow_shapes(handle, values):
+    pairs = [(skewed_rows(70 + 3 * q, 40, values, 11 * q, 37), b_matrix(cols, lens, 40, values, 7 * q + 1))
+             for q, (cols, lens) in enumerate(B_SHAPES)]
+    for (A, B), C in zip(pairs, run_batch(handle, pairs)):
+        assert_matches_oracle(C, A, B, exact=values == "int")
+
+
+@pytest.mark.parametrize("values", ["f32", "f64"])
+def test_batched_narrow_row_sizes(handle, values):
+    """Rows for a chunk (512 products or fewer), a warp and a block (above 8192), and their neighbours."""
+    k = 700
+    B = b_matrix(256, [16], k, values, 3)
+    lens = [32, 33, 31, 511, 512, 513, 0, 1, 700, 699, 64, 65] + [5] * 50
+    A = rows_of(lens, k, values, 4)
+    for C in run_batch(handle, [(A, B), (A, B)]):
+        assert_matches_oracle(C, A, B)
+
+
+@pytest.mark.parametrize("values", ["f64", "int"])
+def test_batched_narrow_unsorted_and_repeated(handle, values):
+    """Unsorted or repeated columns in one B of a batch, next to a B that ascends and a wide one."""
+    A = random_csr(90, 60, 0.2, 21, values=values)
+    B = random_csr(60, 200, 0.1, 22, values=values, sort_cols=False, dup_frac=0.3)
+    S = random_csr(60, 200, 0.1, 23, values=values)
+    D = Csr(S.rows, S.cols, S.row_ptr, S.col_idx.copy(), S.val)
+    s = int(S.row_ptr[7])
+    assert S.row_ptr[8] - s >= 2
+    D.col_idx[s + 1] = D.col_idx[s]   # one repeated column, else ascending
+    W = random_csr(60, 20000, 0.002, 24, values=values)
+    pairs = [(A, B), (A, S), (A, D), (A, W)]
+    for (x, y), C in zip(pairs, run_batch(handle, pairs)):
+        assert_matches_oracle(C, x, y, exact=values == "int")
