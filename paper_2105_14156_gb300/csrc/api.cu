@@ -289,7 +289,8 @@ int run_symbolic(smash_handle *h, const RawOperands &op, int64_t n, Plan &pl, in
     // buffers of the dense and spill bins, before the launches fork
     const int nsub = (int)((op.ncols + kSubCols - 1) / kSubCols);
     int spill_tb = 0;
-    if (counts[kBinDense]) {
+    const bool narrow = use_narrow_sym(h, op.ncols);
+    if (counts[kBinDense] && !narrow) {
         if ((st = ensure(h, h->wslot, sizeof(int) * (size_t)n, s))) return st;
         if ((st = ensure(h, h->wcnt, sizeof(uint16_t) * (size_t)counts[kBinDense] * nsub, s))) return st;
         if (cudaMemsetAsync(h->wslot.ptr, 0xff, sizeof(int) * (size_t)n, s) != cudaSuccess) return SMASH_ERR_CUDA;
@@ -309,7 +310,10 @@ int run_symbolic(smash_handle *h, const RawOperands &op, int64_t n, Plan &pl, in
         cudaStream_t bs = fk.get(q++);
         const int *rows = pl.bb.rows + offsets[b];
         int *tok = pl.bb.tokens + b;
-        if (b == kBinDense) {
+        if (b == kBinDense && narrow) {
+            LaunchTimer lt(h, bs, "sym_narrow", b, 256, counts[b], sums[b], sums[16 + b], sums[32 + b]);
+            launch_narrow_count(op, rows, counts[b], sums[b], sums[16 + b], tok, h->sms, nnz_out, err, bs);
+        } else if (b == kBinDense) {
             // the bitmap pass also counts each row's columns per block of
             // kSubCols columns, for the numeric dense kernel
             WinCount wc;
@@ -453,12 +457,15 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
     // (capacity mode: the counts of the learned planning)
     const RowGather *kept =
         out.row_nnz ? cap_rec : (rcache_matches(h, op) ? (const RowGather *)h->rcache.ptr : nullptr);
-    // Dense rows take column windows when their products pay for slicing B
+    // Dense rows of a narrow B: a warp owns all columns. Other dense rows take
+    // column windows when their products pay for slicing B
     // (a pass over B's rows and entries); otherwise the global hash. Their
     // counts and the slices of B are prepared on s before the bins fork.
     const int bd = kBinDense;
     int cpc = 0, nw = 0, per = 1;
-    const bool windows = counts[bd] && dense_windows(h, op, dt, sums[16 + bd], cpc, nw, per);
+    const bool narrow = counts[bd] && use_narrow_num(h, op.ncols, dt);
+    const bool windows = counts[bd] && !narrow && dense_windows(h, op, dt, sums[16 + bd], cpc, nw, per);
+    if (narrow && (st = ensure(h, h->split, 256, s))) return st;
     HashLaunch hld = hash_launch(h, 0, op.ncols);
     hld.dense_blocks = dense_blocks_of(h, dt);
     WinCount wc;
@@ -501,7 +508,7 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
     // global-memory tables of the spill bin (and of dense rows without windows)
     int spill_tb = 0;
     for (int b : {(int)kBinSpill, (int)kBinDense}) {
-        if (!counts[b] || (b == kBinDense && windows)) continue;
+        if (!counts[b] || (b == kBinDense && (windows || narrow))) continue;
         const int tb = table_bits(maxsize[b], rule.inv_load);
         spill_tb = tb > spill_tb ? tb : spill_tb;
     }
@@ -520,7 +527,12 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
         if (!counts[b]) continue;
         const int *rows = pl.bb.rows + offsets[b];
         int *tok = pl.bb.tokens + b;
-        if (b == kBinDense && windows) {
+        if (b == kBinDense && narrow) {
+            cudaStream_t bs = fk.get(q++);
+            LaunchTimer lt(h, bs, "num_narrow", b, 256, counts[b], sums[b], sums[16 + b], sums[32 + b], 2);
+            launch_narrow_num(dt, op, rows, counts[b], sums[b], sums[16 + b], tok, h->sms, (long long *)h->split.ptr,
+                              out, err, bs);
+        } else if (b == kBinDense && windows) {
             cudaStream_t bs = fk.get(q++);
             // (row, window) items
             LaunchTimer lt(h, bs, "num_dense_window", b, 1024 / hld.dense_blocks, counts[b], sums[b], sums[16 + b],

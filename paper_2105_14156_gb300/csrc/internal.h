@@ -145,8 +145,9 @@ inline int ensure(smash_handle *h, DevBuf &b, size_t need, cudaStream_t s, bool 
     size_t want = need + need / 4;
     want = (want + 4095) & ~size_t(4095);
     void *p = h->alloc(want, h->ctx);
-    if (!p) {
-        want = (need + 4095) & ~size_t(4095);
+    const size_t least = (need + 4095) & ~size_t(4095);
+    if (!p && least < want) {
+        want = least;
         p = h->alloc(want, h->ctx);
     }
     if (!p) return SMASH_ERR_ALLOC;
@@ -560,6 +561,16 @@ inline bool tiny_first(const smash_handle *h, const BinRule &r, int bin, int cou
     return tb <= r.tiny_tbits && tb <= kTinyNumTBits && count >= tiny_min_rows(h);
 }
 
+// Whether the dense rows of a phase run with a warp (heavy ones: a block) per
+// row that owns all columns of B (k_narrow.cu). A chosen number of resident
+// blocks, or owner computes, asks for the kernels that those parameters shape.
+inline bool use_narrow_sym(const smash_handle *h, int64_t ncols) {
+    return h->params.sym_dense_blocks == 0 && narrow_symbolic(ncols);
+}
+inline bool use_narrow_num(const smash_handle *h, int64_t ncols, int dtype) {
+    return h->params.dense_blocks == 0 && !h->params.dense_owner && narrow_numeric(dtype, ncols);
+}
+
 inline BinRule sym_rule(const smash_handle *h, int64_t ncols) {
     BinRule r;
     r.inv_load = 1.0f / h->params.max_load;
@@ -581,7 +592,10 @@ inline BinRule num_rule(const smash_handle *h, int64_t ncols, int dtype) {
     // column window that fits shared memory
     const bool dense_fits = ncols <= dense_bitmap_max_cols() && num_window_cols(dtype, dense_blocks_of(h, dtype), false) > 0;
     r.dense_ok = (h->params.dense_ratio > 0 && dense_fits) ? 1 : 0;
-    r.dense_min = r.dense_ok ? (ncols + h->params.dense_ratio - 1) / h->params.dense_ratio : (1ll << 62);
+    // (a warp that owns all columns clears and scans them for about a quarter
+    // of what a block's window costs, so it takes rows four times as short)
+    const int64_t ratio = (int64_t)h->params.dense_ratio * (use_narrow_num(h, ncols, dtype) ? 4 : 1);
+    r.dense_min = r.dense_ok ? (ncols + ratio - 1) / ratio : (1ll << 62);
     if (r.dense_min < 1) r.dense_min = 1;
     int mt = h->params.num_max_tbits;
     // The largest tables are one 1024-thread group; if their rows would want

@@ -224,6 +224,19 @@ void launch_sym_tiny(const RawOperands &op, const int *rows, int count, int tbit
                      int *nnz_out, int *err, cudaStream_t s);
 void launch_num_tiny(int dtype, const RawOperands &op, const int *rows, int count, int tbits, float max_load,
                      int sms, const NumOut &out, int *err, cudaStream_t s);
+// Narrow B (k_narrow.cu): dense rows whose columns one warp owns. Whether B's
+// columns fit a warp's flags / accumulator; the symbolic limit is the double
+// accumulator's, so that a phase pair never mixes a narrow symbolic phase with
+// column windows that would have to count their columns again.
+constexpr int kNarrowSymCols = 3072;
+bool narrow_symbolic(int64_t ncols);
+bool narrow_numeric(int dtype, int64_t ncols);
+// entries, products: of the listed rows (entries of A).
+void launch_narrow_count(const RawOperands &op, const int *rows, int count, long long entries, long long products,
+                         int *token, int sms, int *nnz_out, int *err, cudaStream_t s);
+// descents: device scratch of one long long.
+void launch_narrow_num(int dtype, const RawOperands &op, const int *rows, int count, long long entries,
+                       long long products, int *token, int sms, long long *descents, const NumOut &out, int *err, cudaStream_t s);
 // Column windows of the dense rows (k_split.cu): slices of B regrouped by
 // window of cpc columns; woff[B.rows][nslices+1] (nslices > 1 only).
 struct BSlices {

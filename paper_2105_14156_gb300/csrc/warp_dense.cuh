@@ -21,10 +21,10 @@
 // for loads of B otherwise.
 //
 // Occupancy needs no bitmap: an unused word holds -0.0, which no sum of
-// products reaches (a product is formed as a * b + 0.0, and a sum that rounds
-// to zero is +0.0 unless both terms are -0.0), and which adding leaves no
-// trace (-0.0 + x = x). The copies are added up, and their words returned to
-// -0.0, while the row is written out in column order.
+// products reaches (a product that is -0.0 is added as +0.0, and a sum is -0.0
+// only when both terms are) and which leaves no trace in a sum (-0.0 + x = x).
+// The copies are added up, and their words returned to -0.0, while the row is
+// written out in column order.
 #pragma once
 
 #include "device_common.cuh"
@@ -43,9 +43,10 @@ __host__ __device__ constexpr int dense_stride(int ncols) { return (ncols + 31) 
 // Most bytes a warp's accumulator may take (eight warps of a block: 192 KB).
 constexpr int kDenseWarpBytes = 24 * 1024;
 
-__host__ __device__ inline int dense_mode(int64_t b_nnz, int64_t b_rows, int ncols, int vsz) {
-    int m = b_nnz < 3 * b_rows ? kDenseFlat : b_nnz <= 8 * b_rows ? kDenseW8 : b_nnz <= 16 * b_rows ? kDenseW16
-                                                                                                       : kDenseW32;
+// entries: of `rows` rows of B (all, or each as often as a product reads it).
+__host__ __device__ inline int dense_mode(int64_t entries, int64_t rows, int ncols, int vsz) {
+    int m = entries < 3 * rows ? kDenseFlat : entries <= 8 * rows ? kDenseW8 : entries <= 16 * rows ? kDenseW16
+                                                                                                      : kDenseW32;
     while (dense_copies(m) > 1 && (int64_t)dense_copies(m) * dense_stride(ncols) * vsz > kDenseWarpBytes) ++m;
     return m;
 }
@@ -74,31 +75,23 @@ __device__ __forceinline__ void dense_clear(V *acc, int words) {
 
 constexpr int kDenseUnroll = 4;   // steps whose loads of B are issued together
 
-// One step of W lanes per row of B: every active lane adds a * b to column j
-// of its group's copy. (The barrier orders the step before the next one's
-// loads of the same words.)
-template <typename V>
-__device__ __forceinline__ void dense_step(V *mine, bool act, int j, V a, V b) {
-    if (act) mine[j] += dense_product(a, b);
-    __syncwarp();
-}
-
-// Adds the products of A entries in batches of 32 that start at first, first
-// + step, ... below ae, with W lanes to a row of B (ascending columns below
-// op.ncols). Rows of up to 2 W entries take one or two steps of their lane
-// group (the second steps of a batch packed together), longer ones all lanes.
-template <typename V, int W>
-__device__ __forceinline__ void dense_rows(const Operands<V> &op, int64_t first, int64_t ae, int64_t step, V *acc,
-                                           int stride, int *err) {
+// Every product of the A entries in batches of 32 that start at first, first +
+// step, ... below ae, with W lanes to a row of B: f(group, act, j, a, b) is
+// called by all 32 lanes together once per step (act: the lane holds a product
+// of its lane group's row; a, b: 0 when !NUM). Rows of up to 2 W entries take
+// one or two steps of their lane group (the second steps of a batch packed
+// together), longer ones all lanes as group 0. Columns are not checked.
+template <typename V, int W, bool NUM, typename F>
+__device__ __forceinline__ void dense_rows(const Operands<V> &op, int64_t first, int64_t ae, int64_t step, int *err,
+                                           F &&f) {
     constexpr int S = 32 / W;
     const int lane = lane_id();
     const int sub = lane / W, sl = lane & (W - 1);
-    V *mine = acc + sub * stride;
     for (int64_t base = first; base < ae; base += step) {
         int len = 0;
         int64_t bs = 0;
         V av = V(0);
-        if (base + lane < ae) load_a_entry<V, true>(op, base + lane, len, bs, av, err);
+        if (base + lane < ae) load_a_entry<V, NUM>(op, base + lane, len, bs, av, err);
         const int n = (int)(ae - base < 32 ? ae - base : 32);
         const int own = len > 2 * W ? 0 : len;   // entries added by the lane group
         for (int e = 0; e < n; e += S * kDenseUnroll) {
@@ -109,18 +102,20 @@ __device__ __forceinline__ void dense_rows(const Operands<V> &op, int64_t first,
             for (int u = 0; u < kDenseUnroll; ++u) {
                 const int src = e + u * S + sub;   // at most 31: n <= 32 and S * kDenseUnroll divides 32
                 const int64_t st = __shfl_sync(kFull, bs, src) + sl;
-                act[u] = sl < __shfl_sync(kFull, own, src);
-                au[u] = __shfl_sync(kFull, av, src);
-                jv[u] = 0;
+                const int l = __shfl_sync(kFull, own, src);
+                act[u] = sl < l;
+                au[u] = V(0);
                 bv[u] = V(0);
+                if constexpr (NUM) au[u] = __shfl_sync(kFull, av, src);
+                jv[u] = 0;
                 if (act[u]) {
                     jv[u] = __ldg(op.b_ci + st);
-                    bv[u] = __ldg(op.b_val + st);
+                    if constexpr (NUM) bv[u] = __ldg(op.b_val + st);
                 }
             }
 #pragma unroll
             for (int u = 0; u < kDenseUnroll; ++u)
-                if (u == 0 || e + u * S < n) dense_step<V>(mine, act[u], jv[u], au[u], bv[u]);
+                if (u == 0 || e + u * S < n) f(sub, act[u], jv[u], au[u], bv[u]);
         }
         // second steps: the rows left over, S at a time
         for (unsigned todo = __ballot_sync(kFull, own > W); todo;) {
@@ -137,54 +132,71 @@ __device__ __forceinline__ void dense_rows(const Operands<V> &op, int64_t first,
             __syncwarp();
             const int64_t st = __shfl_sync(kFull, bs, src) + W + sl;
             const int l = __shfl_sync(kFull, own, src);
-            const V a = __shfl_sync(kFull, av, src);
+            V a = V(0), b = V(0);
+            if constexpr (NUM) a = __shfl_sync(kFull, av, src);
             const bool act = have && W + sl < l;
             int j = 0;
-            V b = V(0);
             if (act) {
                 j = __ldg(op.b_ci + st);
-                b = __ldg(op.b_val + st);
+                if constexpr (NUM) b = __ldg(op.b_val + st);
             }
-            dense_step<V>(mine, act, j, a, b);
+            f(sub, act, j, a, b);
         }
-        // long rows of B, all lanes on the first copy
-        for (unsigned todo = __ballot_sync(kFull, len > 2 * W); todo; todo &= todo - 1) {
-            const int src = __ffs(todo) - 1;
-            const int64_t st = __shfl_sync(kFull, bs, src) + lane;
-            const int l = __shfl_sync(kFull, len, src);
-            const V a = __shfl_sync(kFull, av, src);
-            for (int o = 0; o < l; o += 32 * kDenseUnroll) {
-                int jv[kDenseUnroll];
-                V bv[kDenseUnroll];
+        // long rows of B, all lanes: 32 entries of one row a step, the steps of
+        // consecutive rows in flight together
+        unsigned todo = __ballot_sync(kFull, len > 2 * W);
+        int src = __ffs(todo) - 1, o = 0;
+        while (src >= 0) {
+            int jv[kDenseUnroll];
+            bool act[kDenseUnroll];
+            V au[kDenseUnroll], bv[kDenseUnroll];
 #pragma unroll
-                for (int u = 0; u < kDenseUnroll; ++u) {
-                    jv[u] = 0;
-                    bv[u] = V(0);
-                    if (o + 32 * u + lane < l) {
-                        jv[u] = __ldg(op.b_ci + st + o + 32 * u);
-                        bv[u] = __ldg(op.b_val + st + o + 32 * u);
+            for (int u = 0; u < kDenseUnroll; ++u) {
+                act[u] = false;
+                jv[u] = 0;
+                au[u] = V(0);
+                bv[u] = V(0);
+                if (src >= 0) {   // the same for all lanes
+                    const int64_t st = __shfl_sync(kFull, bs, src) + o + lane;
+                    const int l = __shfl_sync(kFull, len, src);
+                    if constexpr (NUM) au[u] = __shfl_sync(kFull, av, src);
+                    act[u] = o + lane < l;
+                    if (act[u]) {
+                        jv[u] = __ldg(op.b_ci + st);
+                        if constexpr (NUM) bv[u] = __ldg(op.b_val + st);
+                    }
+                    o += 32;
+                    if (o >= l) {
+                        todo &= todo - 1;
+                        src = __ffs(todo) - 1;
+                        o = 0;
                     }
                 }
-#pragma unroll
-                for (int u = 0; u < kDenseUnroll; ++u) dense_step<V>(acc, o + 32 * u + lane < l, jv[u], a, bv[u]);
             }
+#pragma unroll
+            for (int u = 0; u < kDenseUnroll; ++u) f(0, act[u], jv[u], au[u], bv[u]);
         }
     }
 }
 
-// The same by mode (ascend: every row of B ascends below op.ncols). All 32
-// lanes call it.
+// Adds the products to the warp's accumulator copies (ascend: every row of B
+// ascends below op.ncols). All 32 lanes call it.
 template <typename V>
 __device__ __forceinline__ void dense_accumulate(const Operands<V> &op, int mode, bool ascend, int64_t first,
                                                  int64_t ae, int64_t step, V *acc, int *err) {
     const int stride = dense_stride(op.ncols);
     if (!ascend) mode = kDenseFlat;
+    // (the barrier orders a step before the next one's loads of the same words)
+    auto add = [&](int group, bool act, int j, V a, V b) {
+        if (act) acc[group * stride + j] += dense_product(a, b);
+        __syncwarp();
+    };
     if (mode == kDenseW8) {
-        dense_rows<V, 8>(op, first, ae, step, acc, stride, err);
+        dense_rows<V, 8, true>(op, first, ae, step, err, add);
     } else if (mode == kDenseW16) {
-        dense_rows<V, 16>(op, first, ae, step, acc, stride, err);
+        dense_rows<V, 16, true>(op, first, ae, step, err, add);
     } else if (mode == kDenseW32) {
-        dense_rows<V, 32>(op, first, ae, step, acc, stride, err);
+        dense_rows<V, 32, true>(op, first, ae, step, err, add);
     } else {
         for (int64_t base = first; base < ae; base += step)
             warp_products<V, true>(op, base, ae - base < 32 ? ae : base + 32, err, [&](int j, V a, V b) {

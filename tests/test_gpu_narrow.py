@@ -103,3 +103,42 @@ def test_batched_narrow_unsorted_and_repeated(handle, values):
     pairs = [(A, B), (A, S), (A, D), (A, W)]
     for (x, y), C in zip(pairs, run_batch(handle, pairs)):
         assert_matches_oracle(C, x, y, exact=values == "int")
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+@pytest.mark.parametrize("cols,lens", B_SHAPES)
+def test_narrow_phases(handle, cols, lens, values):
+    """The two phases and the one-pass product on every shape, heavy rows (more than 256 entries) among them."""
+    from paper_2105_14156_gb300 import smash
+    k = 300
+    B = b_matrix(cols, lens, k, values, 5)
+    A = skewed_rows(150, k, values, 6, 257)
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=values == "int")
+    C, _, owner = handle.spgemm_learned(dA, dB, None)
+    assert_matches_oracle(C.to_host(), A, B, exact=values == "int")
+    owner.free()
+
+
+@pytest.mark.parametrize("values", ["f64", "int"])
+def test_narrow_phases_unsorted_and_repeated(handle, values):
+    from paper_2105_14156_gb300 import smash
+    A = random_csr(300, 400, 0.1, 31, values=values)
+    B = random_csr(400, 900, 0.02, 32, values=values, sort_cols=False, dup_frac=0.3)
+    C = handle.spgemm(smash.to_device(A), smash.to_device(B), check=True).to_host()
+    assert_matches_oracle(C, A, B, exact=values == "int")
+
+
+def test_narrow_wrong_sizes_are_reported(handle):
+    """A row pointer of C that is not this product's: an error status, nothing written past a row's room."""
+    import torch
+    from paper_2105_14156_gb300 import smash
+    A, B = random_csr(64, 50, 0.3, 41, values="f32"), random_csr(50, 300, 0.2, 42, values="f32")
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    c_rp, nnz = handle.symbolic(dA, dB)
+    short = torch.arange(65, dtype=torch.int64, device="cuda") * 70   # rows hold about 280 entries
+    with pytest.raises(smash.SmashError) as e:
+        handle.numeric(dA, dB, short, 64 * 70)
+        handle.check()
+    assert e.value.status == 1
+    assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B)
