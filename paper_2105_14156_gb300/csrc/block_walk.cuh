@@ -1,0 +1,127 @@
+// Products of one row of A shared out over the warps of a block without
+// staging or barriers, for the kernels whose block owns one accumulator (the
+// column windows of the numeric phase, the column bitmap of the symbolic one).
+//
+// Every warp loads each batch of 32 entries of the row for itself (lane l:
+// where entry l's row of B starts, its length, a_ik; the warps' loads of the
+// same words hit in L1), lays the batch's products on one line with a scan, and
+// walks its own kWarps-th part of the line. Inside a row of B of which at least
+// 128 products are left, four coalesced loads are issued per lane and round and
+// nothing else is done per product; shorter pieces take steps of 32 products
+// that may span several rows of B (a lane's entry is the number of entries that
+// end at or before its product).
+//
+// Measured against staging the entries in shared memory with a block scan and
+// three barriers a batch, and finding the entry in every step (group_products):
+// the bitmap pass of the skewed 262,144-row square (2.8 G products) 5.9 -> 3.6 ms
+// (61 -> 33 instructions per 32 products), the float64 windows of the 65,536-row
+// one 4.0 -> 3.9 ms (bound by the adds), whole calls 6.06 -> 4.22 ms and 6.51 ->
+// 6.03 ms.
+#pragma once
+
+#include "device_common.cuh"
+
+namespace smash {
+
+// Position of the n-th (0-based) set bit of x (n < popc(x)), by halving.
+__device__ __forceinline__ int nth_set_bit(unsigned x, int n) {
+    int pos = 0;
+    int c = __popc(x & 0xffffu);
+    if (n >= c) { n -= c; x >>= 16; pos += 16; }
+    c = __popc(x & 0xffu);
+    if (n >= c) { n -= c; x >>= 8; pos += 8; }
+    c = __popc(x & 0xfu);
+    if (n >= c) { n -= c; x >>= 4; pos += 4; }
+    c = __popc(x & 0x3u);
+    if (n >= c) { n -= c; x >>= 2; pos += 2; }
+    if (n >= (int)(x & 1u)) pos += 1;
+    return pos;
+}
+
+constexpr int kWalkUnroll = 4;
+
+// f(j, a, b) for every product of A entries [ab, ae) in warp w's share (j: the
+// column, checked by f; a, b: 0 when !NUM). With a sliced B only the entries of
+// op.slice. All 32 lanes call it; f may diverge.
+template <typename V, bool NUM, int kWarps, typename F>
+__device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, int64_t ae, int w, int *err, F &&f) {
+    const int lane = lane_id();
+    for (int64_t base = ab; base < ae; base += 32) {
+        int len = 0;
+        int64_t bs = 0;
+        V av = V(0);
+        if (base + lane < ae) load_a_entry<V, NUM>(op, base + lane, len, bs, av, err);
+        const unsigned nz = __ballot_sync(kFull, len > 0);
+        if (nz == 0u) continue;
+        const int nv = __popc(nz);
+        if (nv < 32 && nz != (1u << nv) - 1u) {
+            // entries without products move out of the way
+            const int src = lane < nv ? nth_set_bit(nz, lane) : 0;
+            len = __shfl_sync(kFull, len, src);
+            bs = __shfl_sync(kFull, bs, src);
+            if constexpr (NUM) av = __shfl_sync(kFull, av, src);
+            if (lane >= nv) len = 0;
+        }
+        const int incl = warp_incl_scan(len);
+        const int total = __shfl_sync(kFull, incl, 31);
+        const int64_t start = bs - (incl - len);   // product p of this entry reads B at start + p
+        const int per = (total + kWarps - 1) / kWarps;
+        int q = min(w * per, total);
+        const int hi = min(q + per, total);
+        while (q < hi) {
+            const int c0 = __popc(__ballot_sync(kFull, incl <= q));   // entry of product q
+            const int last = __shfl_sync(kFull, incl, c0);
+            const int end = last < hi ? last : hi;
+            int jv[kWalkUnroll];
+            V a_u[kWalkUnroll], b_u[kWalkUnroll];
+            if (end - q >= 32 * kWalkUnroll) {
+                const int64_t st = __shfl_sync(kFull, start, c0);
+                V a = V(0);
+                if constexpr (NUM) a = __shfl_sync(kFull, av, c0);
+                const int32_t *pc = op.b_ci + st + lane;
+                const V *pv = op.b_val + st + lane;
+                for (; end - q >= 32 * kWalkUnroll; q += 32 * kWalkUnroll) {
+#pragma unroll
+                    for (int u = 0; u < kWalkUnroll; ++u) {
+                        jv[u] = __ldg(pc + q + 32 * u);
+                        b_u[u] = V(0);
+                        if constexpr (NUM) b_u[u] = __ldg(pv + q + 32 * u);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kWalkUnroll; ++u) f(jv[u], a, b_u[u]);
+                }
+                __syncwarp();
+                continue;
+            }
+            bool act[kWalkUnroll];
+#pragma unroll
+            for (int u = 0; u < kWalkUnroll; ++u) {
+                const int p = q + 32 * u;
+                act[u] = p + lane < hi;
+                jv[u] = 0;
+                a_u[u] = V(0);
+                b_u[u] = V(0);
+                if (p < hi) {   // the same for all lanes
+                    const int c = __popc(__ballot_sync(kFull, incl <= p));
+                    const int e = incl - p;
+                    const unsigned ends = __reduce_or_sync(kFull, (e >= 1 && e <= 31) ? (1u << e) : 0u);
+                    const int ci = c + __popc(ends & ((2u << lane) - 1u));
+                    const int64_t st = __shfl_sync(kFull, start, ci);
+                    if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci);
+                    if (act[u]) {
+                        jv[u] = __ldg(op.b_ci + st + p + lane);
+                        if constexpr (NUM) b_u[u] = __ldg(op.b_val + st + p + lane);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kWalkUnroll; ++u)
+                if (act[u]) f(jv[u], a_u[u], b_u[u]);
+            __syncwarp();
+            q = min(q + 32 * kWalkUnroll, hi);
+        }
+    }
+    __syncwarp();
+}
+
+}  // namespace smash

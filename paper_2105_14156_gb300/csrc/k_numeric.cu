@@ -21,7 +21,9 @@
 #include <climits>
 
 #include "device_common.cuh"
+#include "block_walk.cuh"
 #include "kernels.h"
+#include "warp_dense.cuh"
 #include "writeout.cuh"
 
 namespace smash {
@@ -181,21 +183,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_hash(Operands<V> op, cons
 // the row, known from the per-block column counts of the bitmap pass. No two
 // blocks ever wait on each other.
 
-// Position of the n-th (0-based) set bit of x (n < popc(x)), by halving.
-__device__ __forceinline__ int nth_set_bit(unsigned x, int n) {
-    int pos = 0;
-    int c = __popc(x & 0xffffu);
-    if (n >= c) { n -= c; x >>= 16; pos += 16; }
-    c = __popc(x & 0xffu);
-    if (n >= c) { n -= c; x >>= 8; pos += 8; }
-    c = __popc(x & 0xfu);
-    if (n >= c) { n -= c; x >>= 4; pos += 4; }
-    c = __popc(x & 0x3u);
-    if (n >= c) { n -= c; x >>= 2; pos += 2; }
-    if (n >= (int)(x & 1u)) pos += 1;
-    return pos;
-}
-
 constexpr int kEnumUnroll = 4;   // steps of 32 products whose loads are issued together
 
 // Every product of A entries [ab, ae) whose column lies in slice op.slice of
@@ -275,6 +262,16 @@ __device__ __forceinline__ void slice_enum(const Operands<V> &op, int64_t ab, in
     }
 }
 
+// Item of the window kernel handed to the block by its first thread.
+struct WinItem {
+    long long item;   // row of the bin * nw + window (past the end: no more)
+    int i, w;         // row of A, window
+    int skip;         // capacity mode: the row is known not to fit
+};
+
+// Merge: the block's warps share each batch of 32 entries of the row (block_walk),
+// add their products atomically to the window's accumulator, whose unused words
+// hold -0.0 (warp_dense.cuh): the add that finds one sets the column's bit.
 // OWN (owner computes): warp q of the block owns the window's columns of
 // every kWarps-th group of 32 columns from group q on (B sliced by warp:
 // slices [w * kWarps, (w + 1) * kWarps) make up window w; interleaved, so
@@ -284,67 +281,108 @@ __device__ __forceinline__ void slice_enum(const Operands<V> &op, int64_t ab, in
 // column take turns (each writes its lane to the column's owner byte, the
 // lane that reads itself back adds; the others try again), so no atomic and
 // no compare-and-swap retry, and each product costs one add.
+//
+// Bound by the shared-memory pipe (70 % of the cycles in float: an atomic add is
+// a load and a compare-and-swap) and, in double, by the FP64 pipe (60 %).
 template <typename V, int NT, bool OWN>
 __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *rows, int count, int nw, int cpc,
                                                    int subs_per_win, WinCount wc, WinArena ar, NumOutT<V> out,
                                                    unsigned long long *token, int *err) {
     const bool arena = ar.ci != nullptr;
     constexpr int kWarps = NT / 32;
-    constexpr int kMaxChunks = kMaxWinCols / 1024;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long s_item[2], s_aoff;
-    __shared__ int s_off, s_cnt;
-    __shared__ int s_chunk[kMaxChunks + 1];
+    __shared__ WinItem s_next[2];
+    __shared__ long long s_aoff;
+    __shared__ int s_off, s_cnt, s_tot[kWarps];
     const int words = cpc >> 5;
     V *acc = (V *)smem;
     unsigned *bm = (unsigned *)(smem + (size_t)cpc * sizeof(V));
-    const ProdScratch<V> sc = carve_prod_scratch<V, NT>((unsigned char *)(bm + words));
     unsigned char *own = (unsigned char *)(bm + words);   // OWN: owner byte of each column
     const int t = threadIdx.x;
     const int lane = lane_id();
     const int wp = t >> 5;
-    for (int j = t; j < cpc; j += NT) acc[j] = V(0);
+    for (int j = t; j < cpc; j += NT) acc[j] = dense_unused(V(0));
     for (int w = t; w < words; w += NT) bm[w] = 0u;
     const int64_t items = (int64_t)count * nw;
-    // items are claimed one ahead (the claim's latency hides behind the
-    // current item); s_item[par] holds the claimed next item, written before
-    // the item's closing barrier and read after it
+    // Items are claimed one ahead by the first thread: the claim is made when an
+    // item starts, its row is looked up when the thread's share of the item's
+    // products is done, and the closing barrier hands it to the block.
+    auto look_up = [&](long long item) {
+        WinItem n{item, 0, 0, 0};
+        if (item < items) {
+            const int r = (int)(item / nw);
+            n.w = (int)(item - (int64_t)r * nw);
+            n.i = rows[r];
+            // (arena mode: a row that overflows is found when its room is reserved)
+            if (!arena && out.row_nnz) n.skip = out.row_nnz[n.i] < 0 ? 1 : 0;
+        }
+        return n;
+    };
     int par = 0;
-    if (t == 0) s_item[0] = (long long)atomicAdd(token, 1ull);
+    if (t == 0) s_next[0] = look_up((long long)atomicAdd(token, 1ull));
     __syncthreads();
     for (;;) {
-        const int64_t item = s_item[par];
+        const WinItem it = s_next[par];
         par ^= 1;
-        if (item >= items) break;
-        if (t == 0) s_item[par] = (long long)atomicAdd(token, 1ull);
-        const int r = (int)(item / nw);
-        const int w = (int)(item - (int64_t)r * nw);
-        const int i = rows[r];
-        // capacity mode: skip a row that overflowed. In arena mode other blocks
-        // update row_nnz[i] meanwhile: one thread reads it for the whole block.
-        bool skip = false;
-        if (out.row_nnz) {
-            if (t == 0) s_off = out.row_nnz[i] < 0 ? 1 : 0;
-            __syncthreads();
-            skip = s_off != 0;
-            __syncthreads();
-        }
+        if (it.item >= items) break;
+        const long long claim = t == 0 ? (long long)atomicAdd(token, 1ull) : 0;
+        const int i = it.i, w = it.w;
         int slot = -1;
         int64_t c0 = 0;
         int n_exp = 0;
-        if (!arena) {
+        bool skip = it.skip != 0;   // the same for the whole block
+        if (!arena && !skip) {
             slot = wc.wslot[i];
-            if (!skip && slot < 0) {
+            if (slot < 0) {
                 if (t == 0) raise_err(err, kErrCountMismatch);
                 skip = true;
+            } else if (!out_range(out, i, c0, n_exp, err)) {
+                skip = true;
             }
-            if (!skip && !out_range(out, i, c0, n_exp, err)) skip = true;
         }
         if (skip) {
+            if (t == 0) s_next[par] = look_up(claim);
             __syncthreads();
             continue;
         }
+        const int lo = w * cpc;
+        const int width = min(cpc, op.ncols - lo);
+        int64_t ab = 0, ae = 0;
+        a_row_range(op, i, ab, ae, err);
+        if constexpr (OWN) {
+            op.slice = w * kWarps + wp;
+            slice_enum<V>(op, ab, ae, err, [&](bool act, int j, V a, V bkj) {
+                const unsigned off = (unsigned)(j - lo);
+                bool pend = act && off < (unsigned)width && ((off >> 5) & (kWarps - 1)) == (unsigned)wp;
+                const V v = dense_product(a, bkj);
+                while (__any_sync(kFull, pend)) {
+                    if (pend) own[off] = (unsigned char)lane;
+                    __syncwarp();
+                    const bool win = pend && own[off] == (unsigned char)lane;
+                    if (win) {
+                        acc[off] += v;
+                        const unsigned bit = 1u << (off & 31);
+                        unsigned *bw = bm + (off >> 5);
+                        if (!(*(volatile unsigned *)bw & bit)) atomicOr(bw, bit);
+                    }
+                    __syncwarp();
+                    pend = pend && !win;
+                }
+            });
+        } else {
+            op.slice = w;
+            block_walk<V, true, kWarps>(op, ab, ae, wp, err, [&](int j, V a, V bkj) {
+                const unsigned off = (unsigned)(j - lo);
+                if (off < (unsigned)width) {
+                    if (!dense_used(atomicAdd(acc + off, dense_product(a, bkj))))
+                        atomicOr(bm + (off >> 5), 1u << (off & 31));
+                } else if ((unsigned)j >= (unsigned)op.ncols) {
+                    raise_err(err, kErrBadIndex);
+                }
+            });
+        }
         if (!arena && wp == 0) {
+            // columns of the row in the windows before this one, and in this one
             const uint16_t *sub = wc.wcnt + (size_t)slot * wc.nsub;
             const int s_lo = w * subs_per_win;
             const int s_hi = min(s_lo + subs_per_win, wc.nsub);
@@ -361,66 +399,27 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                 s_cnt = mine;
             }
         }
-        const int lo = w * cpc;
-        const int width = min(cpc, op.ncols - lo);
-        int64_t ab = 0, ae = 0;
-        a_row_range(op, i, ab, ae, err);
-        if constexpr (OWN) {
-            op.slice = w * kWarps + wp;
-            slice_enum<V>(op, ab, ae, err, [&](bool act, int j, V a, V bkj) {
-                const unsigned off = (unsigned)(j - lo);
-                bool pend = act && off < (unsigned)width && ((off >> 5) & (kWarps - 1)) == (unsigned)wp;
-                const V v = a * bkj;
-                while (__any_sync(kFull, pend)) {
-                    if (pend) own[off] = (unsigned char)lane;
-                    __syncwarp();
-                    const bool win = pend && own[off] == (unsigned char)lane;
-                    if (win) {
-                        acc[off] += v;
-                        const unsigned bit = 1u << (off & 31);
-                        unsigned *bw = bm + (off >> 5);
-                        if (!(*(volatile unsigned *)bw & bit)) atomicOr(bw, bit);
-                    }
-                    __syncwarp();
-                    pend = pend && !win;
-                }
-            });
-            __syncthreads();
-        } else {
-            op.slice = w;
-            group_products<V, true, NT, NT>(op, ab, ae, sc, err, [&](int j, V a, V bkj) {
-                const unsigned off = (unsigned)(j - lo);
-                if (off < (unsigned)width) {
-                    atomicAdd(acc + off, a * bkj);
-                    const unsigned bit = 1u << (off & 31);
-                    unsigned *bw = bm + (off >> 5);
-                    if (!(*(volatile unsigned *)bw & bit)) atomicOr(bw, bit);
-                }
-            });
-        }
-        // write-out in chunks of 32 bitmap words (1024 columns): chunk totals,
-        // their prefix, then every chunk's columns in order.
+        if (t == 0) s_next[par] = look_up(claim);
+        __syncthreads();
+        // write-out: every warp takes a run of the window's bitmap words (totals,
+        // their prefix over the warps), group by group of at most 32 words
         const int wwords = (width + 31) >> 5;
-        const int nch = (wwords + 31) >> 5;
-        for (int c = wp; c < nch; c += kWarps) {
-            const int x = 32 * c + lane;
-            const int tot = warp_sum(x < wwords ? __popc(bm[x]) : 0);
-            if (lane == 0) s_chunk[c] = tot;
+        const int run = (wwords + kWarps - 1) / kWarps;
+        const int x0 = min(wp * run, wwords), x1 = min(x0 + run, wwords);
+        {
+            int c = 0;
+            for (int x = x0 + lane; x < x1; x += 32) c += __popc(bm[x]);
+            c = __reduce_add_sync(kFull, c);
+            if (lane == 0) s_tot[wp] = c;
         }
         __syncthreads();
-        if (wp == 0) {
-            int run = 0;
-            for (int c0w = 0; c0w < nch; c0w += 32) {
-                const int c = c0w + lane;
-                const int v = c < nch ? s_chunk[c] : 0;
-                const int incl = warp_incl_scan(v);
-                if (c < nch) s_chunk[c] = run + incl - v;
-                run += __shfl_sync(kFull, incl, 31);
-            }
-            if (lane == 0) s_chunk[nch] = run;
+        int at, total;   // entries of the warps before this one, of all warps
+        {
+            const int c = lane < kWarps ? s_tot[lane] : 0;
+            const int incl = warp_incl_scan(c);
+            total = __shfl_sync(kFull, incl, 31);
+            at = __shfl_sync(kFull, incl - c, wp);
         }
-        __syncthreads();
-        const int total = s_chunk[nch];
         int base = 0;
         bool ok;
         if (arena) {
@@ -429,8 +428,8 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                 const long long off = (long long)atomicAdd(ar.top, (unsigned long long)total);
                 const bool fits = off + total <= ar.cap;
                 s_aoff = fits ? off : -1;
-                ar.desc_off[item] = fits ? off : -1;
-                ar.desc_cnt[item] = total;
+                ar.desc_off[it.item] = fits ? off : -1;
+                ar.desc_cnt[it.item] = total;
                 if (fits) atomicAdd(out.row_nnz + i, total);
                 else atomicOr(out.row_nnz + i, INT_MIN);
             }
@@ -442,32 +441,32 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
             if (t == 0 && total != s_cnt) raise_err(err, kErrCountMismatch);
             ok = total == s_cnt && (int64_t)base + total <= (int64_t)n_exp;
         }
-        int32_t *dst_ci = arena ? ar.ci : out.c_ci;
-        V *dst_val = arena ? (V *)ar.val : out.c_val;
-        for (int c = wp; c < nch; c += kWarps) {
-            const int x = 32 * c + lane;
-            const unsigned word = x < wwords ? bm[x] : 0u;
+        int32_t *dst_ci = (arena ? ar.ci : out.c_ci) + c0 + base;
+        V *dst_val = (arena ? (V *)ar.val : out.c_val) + c0 + base;
+        for (int xb = x0; xb < x1; xb += 32) {
+            const int nx = min(32, x1 - xb);
+            const unsigned word = lane < nx ? bm[xb + lane] : 0u;
+            if (lane < nx) bm[xb + lane] = 0u;
             const int incl = warp_incl_scan(__popc(word));
             const int T = __shfl_sync(kFull, incl, 31);
-            const int64_t cb = c0 + base + s_chunk[c];
-            if (T >= 256) {
-                // dense chunk: word by word, lane = bit
-                for (int q = 0; q < 32; ++q) {
+            if (T >= 8 * nx) {
+                // dense group: word by word, lane = bit
+                for (int q = 0; q < nx; ++q) {
                     const unsigned wq = __shfl_sync(kFull, word, q);
                     const int pre = __shfl_sync(kFull, incl, q) - __popc(wq);
                     if ((wq >> lane) & 1u) {
-                        const int col = ((32 * c + q) << 5) + lane;
+                        const int col = ((xb + q) << 5) + lane;
                         const V v = acc[col];
-                        acc[col] = V(0);
-                        const int64_t pos = cb + pre + __popc(wq & lanemask_lt());
+                        acc[col] = dense_unused(V(0));
+                        const int pos = at + pre + __popc(wq & lanemask_lt());
                         if (ok) {
-                            __stcs(dst_ci + (pos), lo + col);
-                            __stcs(dst_val + (pos), v);
+                            __stcs(dst_ci + pos, lo + col);
+                            __stcs(dst_val + pos, v);
                         }
                     }
                 }
             } else {
-                // sparse chunk: 32 consecutive outputs per step; the owner word of
+                // sparse group: 32 consecutive outputs per step; the owner word of
                 // output o is the first lane whose inclusive count exceeds o
                 for (int o0 = 0; o0 < T; o0 += 32) {
                     const int o = o0 + lane;
@@ -480,17 +479,17 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                     const unsigned wl = __shfl_sync(kFull, word, L);
                     const int el = __shfl_sync(kFull, incl, L) - __popc(wl);
                     if (o < T) {
-                        const int col = ((32 * c + L) << 5) + nth_set_bit(wl, o - el);
+                        const int col = ((xb + L) << 5) + nth_set_bit(wl, o - el);
                         const V v = acc[col];
-                        acc[col] = V(0);
+                        acc[col] = dense_unused(V(0));
                         if (ok) {
-                            __stcs(dst_ci + (cb + o), lo + col);
-                            __stcs(dst_val + (cb + o), v);
+                            __stcs(dst_ci + (at + o), lo + col);
+                            __stcs(dst_val + (at + o), v);
                         }
                     }
                 }
             }
-            if (x < wwords) bm[x] = 0u;
+            at += T;
         }
         __syncthreads();
     }
@@ -806,31 +805,23 @@ int dense_bitmap_max_cols() {
 
 static int window_threads(int blocks_per_sm) { return blocks_per_sm <= 1 ? 1024 : blocks_per_sm == 2 ? 512 : 256; }
 
-// Accumulator, occupancy bitmap, then the product staging (atomic adds) or
-// the columns' owner bytes (owner computes).
-template <typename V, int NT>
-static size_t window_smem(int cpc, bool own) {
-    return (size_t)cpc * sizeof(V) + (size_t)(cpc / 32) * 4 + (own ? (size_t)cpc : num_scratch_bytes<V, NT>());
-}
-
+// Accumulator, occupancy bitmap, then the columns' owner bytes (owner computes).
 template <typename V>
-static size_t window_smem_nt(int cpc, int nt, bool own) {
-    return nt == 1024 ? window_smem<V, 1024>(cpc, own)
-                      : nt == 512 ? window_smem<V, 512>(cpc, own) : window_smem<V, 256>(cpc, own);
+static size_t window_smem(int cpc, bool own) {
+    return (size_t)cpc * sizeof(V) + (size_t)(cpc / 32) * 4 + (own ? (size_t)cpc : 0);
 }
 
 int window_warps(int blocks_per_sm) { return window_threads(blocks_per_sm < 1 ? 1 : blocks_per_sm) / 32; }
 
 int num_window_cols(int dtype, int blocks_per_sm, bool own) {
     const int bps = blocks_per_sm < 1 ? 1 : blocks_per_sm;
-    const int nt = window_threads(bps);
     // per-block budget: the SM's shared memory shared by bps blocks (1 KB
     // reserved per block, ~1 KB of static shared variables)
     long long budget = (long long)max_smem_per_sm() / bps - 1024 - 1024;
     if (budget > max_smem_per_block() - 1024) budget = max_smem_per_block() - 1024;
     int best = 0;
     for (int cpc = kSubCols; cpc <= kMaxWinCols; cpc += kSubCols) {
-        const size_t need = dtype ? window_smem_nt<double>(cpc, nt, own) : window_smem_nt<float>(cpc, nt, own);
+        const size_t need = dtype ? window_smem<double>(cpc, own) : window_smem<float>(cpc, own);
         if ((long long)need <= budget) best = cpc;
     }
     return best;
@@ -854,7 +845,7 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     }
     const int nw = sl.nslices <= 1 ? 1 : sl.nslices / sl.per_win;
     const long long items = (long long)count * nw;
-    const size_t smem = window_smem<V, NT>(cpc, own);
+    const size_t smem = window_smem<V>(cpc, own);
     if (own) {
         auto kern = k_num_window<V, NT, true>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

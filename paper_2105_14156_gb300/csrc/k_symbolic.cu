@@ -12,6 +12,7 @@
 //                fraction of cols(B);
 //   k_sym_spill  the table in global memory (Version 3 moved it to DRAM), for
 //                rows too large for shared memory when the bitmap does not fit.
+#include "block_walk.cuh"
 #include "device_common.cuh"
 #include "kernels.h"
 
@@ -70,65 +71,73 @@ __device__ __forceinline__ void count_check(const NumCheck &nc, int i, int tot, 
 
 // Dense rows: a bitmap over the columns of B; count = popcount. With wc.wcnt
 // the row's distinct columns are also counted per block of kSubCols columns
-// (slot = wc.slot_base + r), for the numeric dense kernel.
+// (slot = wc.slot_base + r), for the numeric dense kernel. The warps share the
+// row's products (block_walk); a warp then takes every kWarps-th block of
+// kSubCols columns, four words a lane, and counts and clears it in one pass.
+// words: of the bitmap, a multiple of kSubCols / 32. Bound by instruction issue
+// and the shared-memory pipe (half the cycles each; figures in block_walk.cuh).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int *rows, int count, int *token,
                                                   int words, WinCount wc, int *nnz_out, NumCheck nc, int *err) {
     using G = Group<NT, NT>;
     constexpr int kWarps = NT / 32;
+    constexpr int kSubWords = kSubCols / 32;
+    static_assert(kSubWords == 128, "a warp counts a block of columns with one 16-byte load a lane");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_row[2][1];
+    __shared__ int s_part[kWarps];
     unsigned *bm = (unsigned *)smem;
-    const ProdScratch<float> sc = carve_prod_scratch<float, NT>(smem + (size_t)words * 4);
     const int t = threadIdx.x;
     const int lane = lane_id();
     const int wp = t >> 5;
-    RowClaim<G> claim(token, s_row);
+    for (int x = t; x < words; x += NT) bm[x] = 0u;
+    RowClaim<G> claim(token, s_row);   // (its barrier ends the clearing)
     for (;;) {
         const int r = claim.next(count);
         if (r >= count) break;
         const int i = rows[r];
         int64_t slot = -1;
         if (wc.wcnt && wc.skip_slotted) slot = wc.wslot[i];
-        if (slot >= 0) {
-            // counted before: only the size check
-            int c = 0;
+        const bool counted = slot >= 0;   // counted before: only the size check
+        int c = 0;
+        if (counted) {
             for (int q = t; q < wc.nsub; q += NT) c += wc.wcnt[slot * wc.nsub + q];
-            const int tot = G::template sum<int>(c, sc.red);
-            if (t == 0) count_check(nc, i, tot, err);
-            __syncthreads();
-            continue;
-        }
-        for (int w = t; w < words; w += NT) bm[w] = 0u;
-        __syncthreads();
-        int64_t ab, ae;
-        a_row_range(op, i, ab, ae, err);
-        group_products<float, false, NT, NT>(op, ab, ae, sc, err, [&](int j, float, float) {
-            const unsigned bit = 1u << (j & 31);
-            unsigned *w = bm + (j >> 5);
-            if (!(*(volatile unsigned *)w & bit)) atomicOr(w, bit);
-        });
-        __syncthreads();
-        int cnt = 0;
-        for (int w = t; w < words; w += NT) cnt += __popc(bm[w]);
-        const int tot = G::template sum<int>(cnt, sc.red);
-        if (wc.wcnt) {
+            c = __reduce_add_sync(kFull, c);
+        } else {
+            int64_t ab, ae;
+            a_row_range(op, i, ab, ae, err);
+            block_walk<float, false, kWarps>(op, ab, ae, wp, err, [&](int j, float, float) {
+                if ((unsigned)j < (unsigned)op.ncols) {
+                    const unsigned bit = 1u << (j & 31);
+                    unsigned *w = bm + (j >> 5);
+                    if (!(*(volatile unsigned *)w & bit)) atomicOr(w, bit);
+                } else {
+                    raise_err(err, kErrBadIndex);
+                }
+            });
             slot = wc.slot_base + r;
-            constexpr int kSubWords = kSubCols / 32;
-            for (int q = wp; q < wc.nsub; q += kWarps) {
-                const int w1 = min((q + 1) * kSubWords, words);
-                int c = 0;
-                for (int x = q * kSubWords + lane; x < w1; x += 32) c += __popc(bm[x]);
-                c = warp_sum(c);
-                if (lane == 0) wc.wcnt[slot * wc.nsub + q] = (uint16_t)c;
+            __syncthreads();
+            for (int q = wp; q * kSubWords < words; q += kWarps) {
+                uint4 *v = (uint4 *)(bm + q * kSubWords) + lane;
+                const uint4 x = *v;
+                *v = make_uint4(0u, 0u, 0u, 0u);
+                const int n = __reduce_add_sync(kFull, __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w));
+                c += n;
+                if (wc.wcnt && lane == 0 && q < wc.nsub) wc.wcnt[slot * wc.nsub + q] = (uint16_t)n;
             }
-            if (t == 0) wc.wslot[i] = (int)slot;
+            if (wc.wcnt && t == 0) wc.wslot[i] = (int)slot;
         }
-        if (t == 0) {
-            if (nnz_out) nnz_out[i] = tot;
-            else count_check(nc, i, tot, err);
-        }
+        if (lane == 0) s_part[wp] = c;
         __syncthreads();
+        if (wp == 0) {
+            const int tot = __reduce_add_sync(kFull, lane < kWarps ? s_part[lane] : 0);
+            if (lane == 0) {
+                if (nnz_out) nnz_out[i] = tot;
+                else count_check(nc, i, tot, err);
+            }
+        }
+        // s_part is written again only after the next row's first barrier
+        if (counted) __syncthreads();
     }
 }
 
@@ -233,19 +242,19 @@ void launch_sym_hash(const RawOperands &r, const int *rows, int count, int *toke
     }
 }
 
+static size_t sym_dense_words(int64_t ncols) { return (size_t)((ncols + kSubCols - 1) / kSubCols) * (kSubCols / 32); }
+
 // Block size and blocks per SM of the bitmap kernel: as many resident
 // threads as the bitmaps allow, then as many rows in flight as possible (or
 // the requested blocks per SM).
 static void sym_dense_shape(const HashLaunch &hl, int64_t ncols, int &nt, int &per_sm) {
-    const size_t words = (size_t)((ncols + 31) / 32);
+    const size_t words = sym_dense_words(ncols);
     const int sm_smem = max_smem_per_sm();
     const int nts[3] = {1024, 512, 256};
-    const size_t scr[3] = {prod_scratch_bytes<float, 1024>(), prod_scratch_bytes<float, 512>(),
-                           prod_scratch_bytes<float, 256>()};
     int best_nt = 1024, best_b = 1, best_thr = 0;
     for (int q = 0; q < 3; ++q) {
         if (best_thr == (1 << 30)) break;
-        const size_t per_block = words * 4 + scr[q] + 1024;
+        const size_t per_block = words * 4 + 256 + 1024;   // static variables, reserved by the driver
         if (per_block > (size_t)max_smem_per_block() + 1024) continue;
         int b = (int)((size_t)sm_smem / per_block);
         if (b > 2048 / nts[q]) b = 2048 / nts[q];
@@ -278,8 +287,8 @@ template <int NT>
 static void sym_dense_go(const Operands<float> &op, const int *rows, int count, int *token, int per_sm,
                          const HashLaunch &hl, const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err,
                          cudaStream_t s) {
-    const int words = (op.ncols + 31) / 32;
-    const size_t smem = (size_t)words * 4 + prod_scratch_bytes<float, NT>();
+    const int words = (int)sym_dense_words(op.ncols);
+    const size_t smem = (size_t)words * 4;
     auto kern = k_sym_dense<NT>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int grid = resident_grid(kern, NT, smem, hl.sms, count, per_sm);

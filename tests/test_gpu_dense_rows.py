@@ -1,0 +1,85 @@
+"""Dense rows whose products are shared out over a block's warps: rows of B
+around the lengths where a warp changes from steps over several rows to rounds
+inside one (32 and 128 products), rows of A around a batch of 32 entries,
+entries without products, bitmap words and windows with a ragged end, zero
+products of either sign. Values are held to |c - c*| <= tol * sum |a||b| (1e-5
+float32, 1e-12 float64; entries have at most a few hundred terms, and (m - 1) *
+2^-24 is 1.5e-5 at m = 256 for all-equal signs, a sixteenth of it for the
+random signs here); small integers, zeros among them, must be exact."""
+import numpy as np
+import pytest
+
+from paper_2105_14156_gb300.rmat import Csr, csr_from_coo
+from tests.gpu_util import assert_matches_oracle
+from tests.helpers import random_csr
+
+pytestmark = pytest.mark.gpu
+
+LENS = [0, 1, 31, 32, 33, 0, 64, 127, 128, 129, 160, 255, 256, 257, 1000, 4096, 6000]
+
+
+@pytest.fixture(scope="module")
+def handle():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2105_14156_gb300 import build, smash
+    build.build()
+    h = smash.Handle(0)
+    yield h
+    h.close()
+
+
+def values_of(rng, kind, n):
+    if kind == "int":
+        return rng.integers(-3, 4, n).astype(np.float64)
+    return rng.uniform(-1, 1, n).astype(np.float32 if kind == "f32" else np.float64)
+
+
+def operands(cols, kind, seed):
+    rng = np.random.default_rng(seed)
+    lens = [min(n, cols) for n in LENS * 3]
+    k = len(lens)
+    r = np.repeat(np.arange(k), lens)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lens])
+    rp, ci = csr_from_coo(k, cols, r, c)
+    B = Csr(k, cols, rp, ci, values_of(rng, kind, ci.size))
+    a_lens = [1, 2, 3, 31, 32, 33, k, 17, 5, 40]
+    r = np.repeat(np.arange(len(a_lens)), a_lens)
+    c = np.concatenate([rng.permutation(k)[:n] for n in a_lens])
+    rp, ci = csr_from_coo(len(a_lens), k, r, c)
+    return Csr(len(a_lens), k, rp, ci, values_of(rng, kind, ci.size)), B
+
+
+@pytest.mark.parametrize("kind", ["f32", "f64", "int"])
+@pytest.mark.parametrize("cols", [7000, 12287, 12289, 40961, 131071])
+def test_dense_row_shapes(handle, cols, kind):
+    from paper_2105_14156_gb300 import smash
+    A, B = operands(cols, kind, cols)
+    handle.set_params(dense_ratio=1 << 20, sym_dense_ratio=1 << 20)
+    try:
+        dA, dB = smash.to_device(A), smash.to_device(B)
+        assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=kind == "int")
+        C, _, owner = handle.spgemm_learned(dA, dB, None)
+        assert_matches_oracle(C.to_host(), A, B, exact=kind == "int")
+        owner.free()
+    finally:
+        handle.set_params(dense_ratio=4, sym_dense_ratio=64)
+
+
+def test_dense_row_bad_columns_are_reported(handle):
+    """A column of B past cols(B) in a dense row of either kind of pass: an error status, nothing out of range."""
+    from paper_2105_14156_gb300 import smash
+    A, B = operands(12289, "f32", 3)
+    B.col_idx[int(B.row_ptr[15]) - 1] = 12289   # the last column of a long row
+    handle.set_params(dense_ratio=1 << 20, sym_dense_ratio=1 << 20)
+    try:
+        dA, dB = smash.to_device(A), smash.to_device(B)
+        with pytest.raises(smash.SmashError) as e:
+            handle.symbolic(dA, dB)
+        assert e.value.status == 1
+        with pytest.raises(smash.SmashError) as e:
+            handle.spgemm_learned(dA, dB, None)
+        assert e.value.status == 1
+    finally:
+        handle.set_params(dense_ratio=4, sym_dense_ratio=64)
