@@ -386,7 +386,7 @@ struct Plan {
 inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t s, Plan &pl) {
     size_t need = 0;
     carve_size<uint8_t>(need, (size_t)n);
-    carve_size<int>(need, 16 * 3);
+    carve_size<int>(need, 16 * 4);
     carve_size<long long>(need, 16 + 4 + 1);
     carve_size<int>(need, (size_t)n);
     carve_size<int>(need, 17);
@@ -400,11 +400,11 @@ inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t 
     if (st) return st;
     Carver c(h->ws.ptr);
     pl.bb.bin = c.take<uint8_t>((size_t)n);
-    int *ctr = c.take<int>(16 * 3);
+    int *ctr = c.take<int>(16 * 4);
     long long *ll = c.take<long long>(16 + 4 + 1);
     pl.bb.counts = ctr;
     pl.bb.cursor = ctr + 16;
-    pl.bb.tokens = ctr + 32;
+    pl.bb.tokens = ctr + 48;
     pl.bb.maxsize = ll;
     pl.bb.stats = ll + 16;
     pl.total = ll + 20;
@@ -420,7 +420,7 @@ inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t 
         pl.scan = c.take<char>(scan_scratch_bytes(n));
     }
     // zero counters, cursors, tokens, maxsize, stats, total
-    if (cudaMemsetAsync(ctr, 0, 16 * 3 * sizeof(int), s) != cudaSuccess) return SMASH_ERR_CUDA;
+    if (cudaMemsetAsync(ctr, 0, 16 * 4 * sizeof(int), s) != cudaSuccess) return SMASH_ERR_CUDA;
     if (cudaMemsetAsync(ll, 0, (16 + 4 + 1) * sizeof(long long), s) != cudaSuccess) return SMASH_ERR_CUDA;
     if (cudaMemsetAsync(pl.bb.sums, 0, 48 * sizeof(long long), s) != cudaSuccess) return SMASH_ERR_CUDA;
     return SMASH_OK;

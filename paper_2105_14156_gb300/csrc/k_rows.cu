@@ -80,6 +80,13 @@ struct RowStats {
     }
 };
 
+// Rows of at least kHeavyFlop products come first in their bin's list: one block
+// may be busy with such a row for as long as all blocks are with the others (the
+// heaviest row of the skewed 262,144-row square, 1 % of its products: 2 of the
+// bitmap pass's MEASURE_HEAVY ms), so it must not start last.
+constexpr long long kHeavyFlop = 1 << 17;
+constexpr int kHeavyBit = 0x80;
+
 // Bins the warp's valid rows (one per lane) by `size` and adds them to the
 // block's statistics. Called by all 32 lanes.
 __device__ __forceinline__ void bin_rows(bool valid, int64_t i, int64_t len, long long f, long long size,
@@ -88,7 +95,7 @@ __device__ __forceinline__ void bin_rows(bool valid, int64_t i, int64_t len, lon
     int b = kBinEmpty;
     if (valid) {
         b = bin_for(size, f, rule);
-        bb.bin[i] = (uint8_t)b;
+        bb.bin[i] = (uint8_t)(f >= kHeavyFlop ? b | kHeavyBit : b);
         if (nnz_out && b == kBinEmpty) nnz_out[i] = 0;
     }
     // warps whose values all fit 26 bits reduce with the 32-bit warp
@@ -327,11 +334,13 @@ __global__ void __launch_bounds__(256) k_rowinfo_long(RawOperands op, const int6
     st.flush(bb);
 }
 
-// Scatter row ids into their bins. Each block reserves one range per bin.
+// Scatter row ids into their bins: heavy rows from the front of a bin's range
+// on, the others from its end down. Each block reserves one range per bin and
+// kind.
 constexpr int kScatNT = 256, kScatItems = 8;
 __global__ void __launch_bounds__(kScatNT) k_bin_scatter(int64_t n, BinBuffers bb) {
-    __shared__ int s_off[kNumBins + 1], s_cnt[kNumBins], s_base[kNumBins];
-    if (threadIdx.x < kNumBins) s_cnt[threadIdx.x] = 0;
+    __shared__ int s_off[kNumBins + 1], s_cnt[2 * kNumBins], s_base[2 * kNumBins];
+    if (threadIdx.x < 2 * kNumBins) s_cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         int acc = 0;
         for (int b = 0; b < kNumBins; ++b) {
@@ -344,29 +353,32 @@ __global__ void __launch_bounds__(kScatNT) k_bin_scatter(int64_t n, BinBuffers b
     }
     __syncthreads();
     int loc[kScatItems];
-    int bins[kScatItems];
+    int bins[kScatItems];   // bin, + kNumBins for a heavy row
     const int64_t base = (int64_t)blockIdx.x * kScatNT * kScatItems;
 #pragma unroll
     for (int it = 0; it < kScatItems; ++it) {
         const int64_t i = base + it * kScatNT + threadIdx.x;
         bins[it] = -1;
         if (i < n) {
-            const int b = bb.bin[i];
+            const int e = bb.bin[i];
+            const int b = e & (kHeavyBit - 1);
             if (b != kBinEmpty) {
-                bins[it] = b;
-                loc[it] = atomicAdd(&s_cnt[b], 1);
+                bins[it] = e & kHeavyBit ? b + kNumBins : b;
+                loc[it] = atomicAdd(&s_cnt[bins[it]], 1);
             }
         }
     }
     __syncthreads();
-    if (threadIdx.x < kNumBins && s_cnt[threadIdx.x])
+    if (threadIdx.x < 2 * kNumBins && s_cnt[threadIdx.x])
         s_base[threadIdx.x] = atomicAdd(bb.cursor + threadIdx.x, s_cnt[threadIdx.x]);
     __syncthreads();
 #pragma unroll
     for (int it = 0; it < kScatItems; ++it) {
         if (bins[it] >= 0) {
-            const int b = bins[it];
-            bb.rows[s_off[b] + s_base[b] + loc[it]] = (int)(base + it * kScatNT + threadIdx.x);
+            const int x = bins[it];
+            const int at = s_base[x] + loc[it];
+            bb.rows[x >= kNumBins ? s_off[x - kNumBins] + at : s_off[x + 1] - 1 - at] =
+                (int)(base + it * kScatNT + threadIdx.x);
         }
     }
 }

@@ -31,9 +31,9 @@ struct RawOperands {
 };
 
 struct BinBuffers {
-    uint8_t *bin;      // [n]
+    uint8_t *bin;      // [n]   (the top bit marks a row that comes first in its bin's list)
     int *counts;       // [16]  rows per bin
-    int *cursor;       // [16]  scatter cursors
+    int *cursor;       // [32]  scatter cursors
     int *tokens;       // [16]  work tokens (row claims) per bin
     long long *maxsize;  // [16] largest size bound per bin
     long long *stats;    // [4]  products, max row products
