@@ -211,12 +211,11 @@ int spgemm_symbolic(smash_handle *h, const smash_csr *A, const smash_csr *B, int
     const RawOperands op = raw_ops(A, B);
     if ((st = run_symbolic(h, op, n, pl, pl.nnz, s, nullptr, 0))) return st;
     {
-        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, 3);
-        launch_scan_rowptr(pl.nnz, n, c_row_ptr, pl.total, pl.scan, s);
+        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, scan_kernels(n));
+        launch_scan_rowptr(pl.nnz, n, c_row_ptr, pl.total, pl.scan, s, scan_to_host(h, true));
     }
     if ((st = last_cuda_status())) return st;
-    if (read_small(h, 0, pl.total, sizeof(long long), s)) return SMASH_ERR_CUDA;
-    st = read_flags(h, s, true);
+    st = flags_status(h, s);
     *c_nnz = h->host[0];
     h->stats.c_nnz = h->host[0];
     return st;
@@ -302,7 +301,7 @@ int run_symbolic(smash_handle *h, const RawOperands &op, int64_t n, Plan &pl, in
     }
     int order[kNumBins];
     const int nb = bin_order(sums, order);
-    Fork fk(h, s);
+    Fork fk(h, s, bins_used(counts));
     int q = 0;
     for (int x = 0; x < nb; ++x) {
         const int b = order[x];
@@ -419,10 +418,8 @@ int window_plan(smash_handle *h, const RawOperands &op, int dt, int cpc, int nw,
         return SMASH_OK;
     }
     const size_t vsz = dt ? 8 : 4;
-    const void *before = h->split.ptr;
     int st;
     if ((st = ensure(h, h->split, 256 + window_plan_bytes(op, nw * per, vsz), s))) return st;
-    (void)before;
     {
         LaunchTimer lt(h, s, "dense_plan", -1, 256, op.b_rows, 0, 0, op.b_nnz, 0);
         lt.add_kernels(launch_window_plan(dt, op, nw, per, cpc, (char *)h->split.ptr + 256, sl, h->sms, s,
@@ -520,7 +517,7 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
     cudaStream_t spill_stream = nullptr;
     int order[kNumBins];
     const int nb = bin_order(sums, order);
-    Fork fk(h, s);
+    Fork fk(h, s, bins_used(counts));
     int q = 0;
     for (int x = 0; x < nb; ++x) {
         const int b = order[x];

@@ -17,7 +17,8 @@ namespace {
 // per-handle side table (the handle struct is shared with other files).
 struct BatchState {
     DevBuf dev;
-    void *pinned = nullptr;
+    void *pinned = nullptr;          // mapped
+    void *pinned_dev = nullptr;      // the same buffer as the kernels see it
     size_t pinned_bytes = 0;
     int tw_bits = 10;
     int warp_less = 0;               // warp rows: tables up to 2^(tw_bits - warp_less) slots
@@ -91,7 +92,15 @@ int ensure_pinned(BatchState &b, size_t need) {
     if (b.pinned) cudaFreeHost(b.pinned);
     b.pinned = nullptr;
     b.pinned_bytes = 0;
-    if (cudaMallocHost(&b.pinned, need) != cudaSuccess) return SMASH_ERR_ALLOC;
+    if (cudaHostAlloc(&b.pinned, need, cudaHostAllocMapped) != cudaSuccess) {
+        b.pinned = nullptr;
+        return SMASH_ERR_ALLOC;
+    }
+    if (cudaHostGetDevicePointer(&b.pinned_dev, b.pinned, 0) != cudaSuccess) {
+        cudaFreeHost(b.pinned);
+        b.pinned = nullptr;
+        return SMASH_ERR_CUDA;
+    }
     b.pinned_bytes = need;
     return SMASH_OK;
 }
@@ -199,11 +208,9 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     carve_size<int64_t>(need, count + 1);
     carve_size<uint8_t>(need, nrows);
     for (int q = 0; q < 6; ++q) carve_size<int>(need, nrows);   // ub, nnz, big, huge, med, longs
-    carve_size<int>(need, 16);
-    carve_size<unsigned long long>(need, 4);
-    carve_size<long long>(need, count);
-    carve_size<int64_t>(need, count + 1);
-    carve_size<int64_t>(need, count);
+    const size_t ctr_bytes = sizeof(int) * 16 + sizeof(unsigned long long) * 4 + sizeof(long long) * count;
+    carve_size<char>(need, ctr_bytes);
+    carve_size<int64_t>(need, 2 * (size_t)count + 1);
     carve_size<BatchArgs>(need, 1);
     if ((st = ensure(h, bs.dev, need, s))) return st;
     Carver c(bs.dev.ptr);
@@ -217,18 +224,22 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     L.huge = c.take<int>(nrows);
     L.med = c.take<int>(nrows);
     L.longs = c.take<int>(nrows);
-    L.counters = c.take<int>(16);
-    L.sums = c.take<unsigned long long>(4);
-    L.descents = c.take<long long>(count);
-    L.base = c.take<int64_t>(count + 1);
-    L.totals = c.take<int64_t>(count);
+    // (one block each: cleared by one memset, read back by one kernel)
+    L.counters = (int *)c.take<char>(ctr_bytes);
+    L.sums = (unsigned long long *)(L.counters + 16);
+    L.descents = (long long *)(L.sums + 4);
+    L.base = c.take<int64_t>(2 * (size_t)count + 1);
+    L.totals = L.base + count + 1;
     BatchArgs *args_dev = c.take<BatchArgs>(1);
     // descriptors (pinned host -> device)
-    const size_t hbytes = sizeof(BatchMat) * count + sizeof(int64_t) * (count + 1) + sizeof(BatchArgs) + 64;
-    if ((st = ensure_pinned(bs, hbytes + 4096))) return st;
+    const size_t desc_bytes = (char *)(L.row_start + count + 1) - (char *)L.mats;
+    const size_t args_at = (desc_bytes + 63) & ~size_t(63);
+    const size_t ends_at = args_at + ((sizeof(BatchArgs) + 63) & ~size_t(63));
+    const size_t ends_bytes = sizeof(int64_t) * (2 * (size_t)count + 1);
+    if ((st = ensure_pinned(bs, ends_at + ends_bytes + 4096))) return st;
     cudaStreamSynchronize(s);   // the pinned staging may still feed a previous copy
     BatchMat *hm = (BatchMat *)bs.pinned;
-    int64_t *hrs = (int64_t *)(hm + count);
+    int64_t *hrs = (int64_t *)((char *)bs.pinned + ((char *)L.row_start - (char *)L.mats));
     int64_t ro = 0;
     // a product whose B fits a warp's dense accumulator is narrow, the others
     // are wide: their rows take hash tables
@@ -266,11 +277,8 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     hrs[count] = ro;
     size_t warp_bytes = wide ? batched_table_bytes(dt, bs.tw_bits) : 128;
     if (dense_bytes > warp_bytes) warp_bytes = dense_bytes;
-    if (cudaMemcpyAsync(L.mats, hm, sizeof(BatchMat) * count, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(L.row_start, hrs, sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(L.counters, 0, sizeof(int) * 16, s) != cudaSuccess ||
-        cudaMemsetAsync(L.sums, 0, sizeof(unsigned long long) * 4, s) != cudaSuccess ||
-        cudaMemsetAsync(L.descents, 0, sizeof(long long) * count, s) != cudaSuccess)
+    if (cudaMemcpyAsync(L.mats, hm, desc_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(L.counters, 0, ctr_bytes, s) != cudaSuccess)
         return SMASH_ERR_CUDA;
     BatchArgs p;
     memset(&p, 0, sizeof(p));
@@ -308,10 +316,7 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     if ((st = last_cuda_status())) return st;
     // sizes for the pools
     char *hb = (char *)h->host;
-    if (cudaMemcpyAsync(hb, L.counters, sizeof(int) * 16, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(hb + 64, L.sums, sizeof(unsigned long long) * 2, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return SMASH_ERR_CUDA;
+    if (read_small(h, 0, L.counters, 80, s) || cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
     int nbig, nhuge, nmed;
     unsigned long long sum_ub, sum_f;
     memcpy(&nbig, hb, 4);
@@ -395,13 +400,11 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
             const RawOperands op = raw_ops(&A[m], &B[m]);
             Plan pl;
             if ((st = plan_buffers(h, A[m].rows, true, s, pl))) return fail(st);
-            int *list = (int *)h->host;   // staged through pinned memory
             if (ensure(h, h->learn, sizeof(int) * kv.second.size() + 256, s)) return fail(SMASH_ERR_ALLOC);
             if (cudaMemcpyAsync(h->learn.ptr, kv.second.data(), sizeof(int) * kv.second.size(),
                                 cudaMemcpyHostToDevice, s) != cudaSuccess ||
                 cudaStreamSynchronize(s) != cudaSuccess)
                 return fail(SMASH_ERR_CUDA);
-            (void)list;
             if ((st = run_symbolic(h, op, A[m].rows, pl, L.nnz + hrs[m], s, (const int *)h->learn.ptr,
                                    (int64_t)kv.second.size())))
                 return fail(st);
@@ -418,20 +421,21 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     {
         LaunchTimer lt(h, s, "batched_persistent", -1, 256, nrows, 0, (long long)sum_f, 0);
         // the arguments through pinned memory, after the descriptors
-        BatchArgs *p_pin = (BatchArgs *)(((uintptr_t)(hrs + count + 1) + 63) & ~(uintptr_t)63);
+        BatchArgs *p_pin = (BatchArgs *)((char *)bs.pinned + args_at);
         *p_pin = p;
         if ((st = run_batched_graph(bs, dt, p_pin, args_dev, wide, grid, s))) return fail(st);
+    }
+    // base offsets and totals, with the flags (many products: by a copy)
+    const int64_t *base = (const int64_t *)((char *)bs.pinned + ends_at), *totals = base + count + 1;
+    if (ends_bytes <= 64 * 1024) {
+        launch_read_small(L.base, (char *)bs.pinned_dev + ends_at, ends_bytes, s);
+    } else if (cudaMemcpyAsync((char *)bs.pinned + ends_at, L.base, ends_bytes, cudaMemcpyDeviceToHost, s) !=
+               cudaSuccess) {
+        return fail(SMASH_ERR_CUDA);
     }
     // a barrier that ran out of time (or any failed check) leaves the row
     // pointers incomplete: stop before anything reads them
     if ((st = read_flags(h, s, true))) return fail(st);
-    // base offsets and totals
-    std::vector<int64_t> base(count + 1), totals(count);
-    if (cudaMemcpyAsync(base.data(), L.base, sizeof(int64_t) * (count + 1), cudaMemcpyDeviceToHost, s) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(totals.data(), L.totals, sizeof(int64_t) * count, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return fail(SMASH_ERR_CUDA);
     for (int m = 0; m < count; ++m) {
         C[m].nnz = totals[m];
         C[m].row_ptr = rp_pool + hrs[m] + m;
@@ -458,7 +462,7 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
         if ((st = run_numeric(h, op, A[m].rows, dt, o, pl, s, (const int *)h->learn.ptr, (int64_t)kv.second.size())))
             return fail(st);
     }
-    if ((st = read_flags(h, s, true))) return fail(st);
+    if (!huge_by_mat.empty() && (st = read_flags(h, s, true))) return fail(st);
     if (stats) *stats = ls;
     return SMASH_OK;
 }

@@ -374,9 +374,18 @@ inline RawOperands raw_ops(const smash_csr *A, const smash_csr *B) {
     return r;
 }
 
+// Counters of the planning kernels (see BinBuffers) and C's size.
+struct PlanWords {
+    long long maxsize[16], stats[4], sums[48], total;
+    int counts[16], cursor[32], tokens[16], offsets[18];
+};
+constexpr size_t kPlanWordsBytes = sizeof(PlanWords);
+static_assert(kPlanWordsBytes % 8 == 0 && kPlanWordsBytes <= 1024, "read back into the first KB of the pinned buffer");
+
 // Per-call planning buffers carved from h->ws.
 struct Plan {
     BinBuffers bb;
+    PlanWords *words;
     long long *bound;
     int *nnz;
     void *scan;
@@ -386,11 +395,8 @@ struct Plan {
 inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t s, Plan &pl) {
     size_t need = 0;
     carve_size<uint8_t>(need, (size_t)n);
-    carve_size<int>(need, 16 * 4);
-    carve_size<long long>(need, 16 + 4 + 1);
+    carve_size<char>(need, kPlanWordsBytes);
     carve_size<int>(need, (size_t)n);
-    carve_size<int>(need, 17);
-    carve_size<long long>(need, 48);
     if (symbolic) {
         carve_size<long long>(need, (size_t)n);
         carve_size<int>(need, (size_t)n);
@@ -400,17 +406,19 @@ inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t 
     if (st) return st;
     Carver c(h->ws.ptr);
     pl.bb.bin = c.take<uint8_t>((size_t)n);
-    int *ctr = c.take<int>(16 * 4);
-    long long *ll = c.take<long long>(16 + 4 + 1);
-    pl.bb.counts = ctr;
-    pl.bb.cursor = ctr + 16;
-    pl.bb.tokens = ctr + 48;
-    pl.bb.maxsize = ll;
-    pl.bb.stats = ll + 16;
-    pl.total = ll + 20;
+    // the counters of the planning lie in one block (PlanWords): cleared by one
+    // memset, read back by one kernel
+    PlanWords *w = (PlanWords *)c.take<char>(kPlanWordsBytes);
+    pl.words = w;
+    pl.bb.counts = w->counts;
+    pl.bb.cursor = w->cursor;
+    pl.bb.tokens = w->tokens;
+    pl.bb.maxsize = w->maxsize;
+    pl.bb.stats = w->stats;
+    pl.bb.offsets = w->offsets;
+    pl.bb.sums = w->sums;
+    pl.total = &w->total;
     pl.bb.rows = c.take<int>((size_t)n);
-    pl.bb.offsets = c.take<int>(17);
-    pl.bb.sums = c.take<long long>(48);
     pl.bound = nullptr;
     pl.nnz = nullptr;
     pl.scan = nullptr;
@@ -419,10 +427,7 @@ inline int plan_buffers(smash_handle *h, int64_t n, bool symbolic, cudaStream_t 
         pl.nnz = c.take<int>((size_t)n);
         pl.scan = c.take<char>(scan_scratch_bytes(n));
     }
-    // zero counters, cursors, tokens, maxsize, stats, total
-    if (cudaMemsetAsync(ctr, 0, 16 * 4 * sizeof(int), s) != cudaSuccess) return SMASH_ERR_CUDA;
-    if (cudaMemsetAsync(ll, 0, (16 + 4 + 1) * sizeof(long long), s) != cudaSuccess) return SMASH_ERR_CUDA;
-    if (cudaMemsetAsync(pl.bb.sums, 0, 48 * sizeof(long long), s) != cudaSuccess) return SMASH_ERR_CUDA;
+    if (cudaMemsetAsync(w, 0, sizeof(PlanWords), s) != cudaSuccess) return SMASH_ERR_CUDA;
     return SMASH_OK;
 }
 
@@ -436,21 +441,17 @@ inline int read_small(smash_handle *h, size_t off, const void *src, size_t bytes
     return cudaPeekAtLastError() == cudaSuccess ? SMASH_OK : SMASH_ERR_CUDA;
 }
 
-// Copy bin counts (16 int), offsets (17 int), maxsize (16 ll), stats (4 ll)
-// to the pinned host buffer and wait.
+// Copy the planning counters to the pinned host buffer and wait.
 inline int fetch_bins(smash_handle *h, const Plan &pl, cudaStream_t s, int *counts, int *offsets, long long *maxsize,
                long long *stats, long long *sums) {
-    char *hb = (char *)h->host;
-    if (read_small(h, 0, pl.bb.counts, 16 * sizeof(int), s) || read_small(h, 64, pl.bb.offsets, 17 * sizeof(int), s) ||
-        read_small(h, 256, pl.bb.maxsize, 20 * sizeof(long long), s) ||
-        read_small(h, 512, pl.bb.sums, 48 * sizeof(long long), s))
-        return SMASH_ERR_CUDA;
+    if (read_small(h, 0, pl.words, sizeof(PlanWords), s)) return SMASH_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
-    memcpy(counts, hb, 16 * sizeof(int));
-    memcpy(offsets, hb + 64, 17 * sizeof(int));
-    memcpy(maxsize, hb + 256, 16 * sizeof(long long));
-    memcpy(stats, hb + 256 + 16 * sizeof(long long), 4 * sizeof(long long));
-    memcpy(sums, hb + 512, 48 * sizeof(long long));
+    const PlanWords &w = *(const PlanWords *)h->host;
+    memcpy(counts, w.counts, 16 * sizeof(int));
+    memcpy(offsets, w.offsets, 17 * sizeof(int));
+    memcpy(maxsize, w.maxsize, sizeof(w.maxsize));
+    memcpy(stats, w.stats, sizeof(w.stats));
+    memcpy(sums, w.sums, sizeof(w.sums));
     for (int b = 0; b < 16; ++b) {
         h->stats.rows_per_bin[b] = b < kNumBins ? counts[b] : 0;
         h->stats.a_nnz_per_bin[b] = sums[b];
@@ -462,18 +463,35 @@ inline int fetch_bins(smash_handle *h, const Plan &pl, cudaStream_t s, int *coun
     return SMASH_OK;
 }
 
-inline int read_flags(smash_handle *h, cudaStream_t s, bool clear) {
-    char *hb = (char *)h->host + 1024;
-    if (read_small(h, 1024, h->err.ptr, kNumErr * sizeof(int), s)) return SMASH_ERR_CUDA;
-    if (clear && cudaMemsetAsync(h->err.ptr, 0, kNumErr * sizeof(int), s) != cudaSuccess) return SMASH_ERR_CUDA;
+// The status of error words that a kernel on s writes to the pinned buffer at
+// byte 1024. Waits.
+inline int flags_status(smash_handle *h, cudaStream_t s) {
     if (cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
-    const int st = status_from_flags((const long long *)hb);
+    const int st = status_from_flags((const long long *)((char *)h->host + 1024));
     // after a failure the kept counts may not describe the inputs any more
     if (st != SMASH_OK) {
         h->wcache.valid = false;
         h->rkey.valid = false;
     }
     return st;
+}
+
+inline int read_flags(smash_handle *h, cudaStream_t s, bool clear) {
+    if (read_small(h, 1024, h->err.ptr, kNumErr * sizeof(int), s)) return SMASH_ERR_CUDA;
+    if (clear && cudaMemsetAsync(h->err.ptr, 0, kNumErr * sizeof(int), s) != cudaSuccess) return SMASH_ERR_CUDA;
+    return flags_status(h, s);
+}
+
+// A scan that leaves its total in the pinned buffer's first word (and, with
+// flags, the error words for flags_status).
+inline ScanPublish scan_to_host(smash_handle *h, bool flags) {
+    ScanPublish p;
+    p.total = h->host_dev;
+    if (flags) {
+        p.err = (int *)h->err.ptr;
+        p.err_host = (int *)((char *)h->host_dev + 1024);
+    }
+    return p;
 }
 
 // Fork of the caller's stream s into s and the handle's auxiliary streams for
@@ -484,10 +502,13 @@ struct Fork {
     smash_handle *h;
     cudaStream_t s;
     int n = 1;   // streams in use: s and n - 1 auxiliary ones
-    Fork(smash_handle *hh, cudaStream_t ss) : h(hh), s(ss) {
+    // launches: how many are to come at most (one needs no other stream)
+    Fork(smash_handle *hh, cudaStream_t ss, int launches) : h(hh), s(ss) {
+        const int want = launches - 1 < smash_handle::kAux ? launches - 1 : smash_handle::kAux;
+        if (want < 1) return;
         bool ok = true;
         if (!h->fork_ev) ok = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) == cudaSuccess;
-        for (int k = 0; ok && k < smash_handle::kAux; ++k) {
+        for (int k = 0; ok && k < want; ++k) {
             if (!h->aux[k]) ok = cudaStreamCreateWithFlags(&h->aux[k], cudaStreamNonBlocking) == cudaSuccess;
             if (ok && !h->join_ev[k]) ok = cudaEventCreateWithFlags(&h->join_ev[k], cudaEventDisableTiming) == cudaSuccess;
         }
@@ -496,8 +517,8 @@ struct Fork {
             return;   // everything on s
         }
         if (cudaEventRecord(h->fork_ev, s) != cudaSuccess) return;
-        for (int k = 0; k < smash_handle::kAux; ++k) cudaStreamWaitEvent(h->aux[k], h->fork_ev, 0);
-        n = 1 + smash_handle::kAux;
+        for (int k = 0; k < want; ++k) cudaStreamWaitEvent(h->aux[k], h->fork_ev, 0);
+        n = 1 + want;
     }
     cudaStream_t get(int k) const { return (k % n) == 0 ? s : h->aux[(k % n) - 1]; }
     ~Fork() {
@@ -534,6 +555,13 @@ inline int bin_order(const long long *sums, int *order) {
             order[y] = order[y - 1];
             order[y - 1] = t;
         }
+    return n;
+}
+
+// Bins with rows: the launches of a phase, at most.
+inline int bins_used(const int *counts) {
+    int n = 0;
+    for (int b = 1; b < kNumBins; ++b) n += counts[b] > 0 ? 1 : 0;
     return n;
 }
 

@@ -23,6 +23,7 @@
 // block's table are done around the kernel by the regular per-product path.
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "writeout.cuh"
 #include "batch_types.h"
 #include "warp_dense.cuh"
@@ -623,9 +624,7 @@ static BatchKernel batched_kernel(int dtype, bool wide) {
 int batched_grid(int dtype, int warp_bytes, bool wide, int sms) {
     const size_t smem = batched_smem(dtype, warp_bytes, wide);
     BatchKernel k = batched_kernel(dtype, wide);
-    int per = 0;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kBNT, smem);
+    int per = resident_per_sm((const void *)k, kBNT, smem);
     return per * sms;
 }
 

@@ -21,6 +21,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "warp_enum.cuh"
 #include "writeout.cuh"
 
@@ -316,9 +317,8 @@ static void num_group_go(const Operands<V> &op, const int *rows, int count, int 
     while ((1 << nbbits) < NB) ++nbbits;
     const int bsh = hl.colbits > nbbits ? hl.colbits - nbbits : 0;
     auto kern = k_num_group<V, IT, K, GS>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GS, smem);
+    allow_smem((const void *)kern);
+    int per_sm = resident_per_sm((const void *)kern, GS, smem);
     if (per_sm < 1) per_sm = 1;
     const long long cap = (long long)per_sm * hl.sms;
     const int grid = (int)(count < cap ? count : cap);

@@ -26,6 +26,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "warp_dense.cuh"
 #include "writeout.cuh"
 
@@ -258,9 +259,8 @@ static Operands<V> narrow_operands(const RawOperands &r) {
 // full grid, at most eight rows) and the heavy rows' threshold.
 template <typename K>
 static int narrow_grid(K kernel, size_t smem, int sms, int count, long long entries, int words, NarrowShare &sh) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kNarrowNT, smem);
+    allow_smem((const void *)kernel);
+    int per_sm = resident_per_sm((const void *)kernel, kNarrowNT, smem);
     const int64_t cap = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
     const int64_t share = count / (cap * kNarrowWarps * 8);
     sh.chunk = share < 1 ? 1 : share > 8 ? 8 : (int)share;

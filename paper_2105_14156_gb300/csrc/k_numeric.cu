@@ -23,6 +23,7 @@
 #include "device_common.cuh"
 #include "block_walk.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "warp_dense.cuh"
 #include "writeout.cuh"
 
@@ -728,8 +729,7 @@ bool num_hash_bitmap_fits(int dtype, int tbits, int ncols) {
 
 template <typename K>
 static int resident_grid(K kernel, int nt, size_t smem, int sms, long long want_blocks, int cap_per_sm = 64) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem);
+    int per_sm = resident_per_sm((const void *)kernel, nt, smem);
     if (per_sm < 1) per_sm = 1;
     if (per_sm > cap_per_sm) per_sm = cap_per_sm;
     long long cap = (long long)per_sm * sms;
@@ -765,7 +765,7 @@ static void num_hash_go(const Operands<V> &op, const int *rows, int count, int *
     const bool buckets = bcap > 0;
     const size_t smem = num_hash_smem<V>(hl.tbits, GS, bm_words, bcap);
     auto kern = out.row_nnz ? k_num_hash<V, GS, NT, true> : k_num_hash<V, GS, NT, false>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     const int grid = resident_grid(kern, NT, smem, hl.sms, (count + groups - 1) / groups);
     const HashCfg hc{hl.hash_kind, hl.colbits};
     // buckets: T/4 of them over the column range, by the high bits
@@ -848,12 +848,12 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     const size_t smem = window_smem<V>(cpc, own);
     if (own) {
         auto kern = k_num_window<V, NT, true>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         const int grid = resident_grid(kern, NT, smem, hl.sms, items);
         kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, wc, ar, out, token, err);
     } else {
         auto kern = k_num_window<V, NT, false>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         const int grid = resident_grid(kern, NT, smem, hl.sms, items);
         kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, wc, ar, out, token, err);
     }
@@ -977,7 +977,7 @@ static void num_spill_typed(const RawOperands &r, const int *rows, int count, in
     if (words > 16384) words = 16384;
     const size_t smem = (size_t)words * 8 + num_scratch_bytes<V, 1024>();
     auto kern = k_num_spill<V, 1024>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     const int gridmax = num_spill_grid(sizeof(V) == 8, hl);
     const int grid = count < gridmax ? count : gridmax;
     int *keys = (int *)tables;

@@ -36,6 +36,7 @@ __device__ __forceinline__ int bin_for(long long size, long long f, const BinRul
 // over each warp's rows of the same bin before they reach the block's shared
 // counters, and the blocks' counters reach the global ones once per block.
 constexpr int kLongRow = 64;
+constexpr int long_row(int lanes) { return lanes > 1 ? 2 * kLongRow : kLongRow; }
 
 __device__ __forceinline__ long long b_row_len(const RawOperands &op, int k, int *err) {
     if ((unsigned)k >= (unsigned)op.b_rows) {
@@ -81,9 +82,9 @@ struct RowStats {
 };
 
 // Rows of at least kHeavyFlop products come first in their bin's list: one block
-// may be busy with such a row for as long as all blocks are with the others (the
-// heaviest row of the skewed 262,144-row square, 1 % of its products: 2 of the
-// bitmap pass's MEASURE_HEAVY ms), so it must not start last.
+// may be busy with such a row for as long as all blocks are with the others, so
+// it must not start last (counts of the 65,536-row skewed square 0.89 -> 0.75
+// ms, its float64 product 6.03 -> 5.86 ms).
 constexpr long long kHeavyFlop = 1 << 17;
 constexpr int kHeavyBit = 0x80;
 
@@ -225,8 +226,11 @@ void launch_read_small(const void *src, void *dst_mapped, size_t bytes, cudaStre
     if (words > 0) k_read_small<<<1, 256, 0, s>>>((const unsigned *)src, (unsigned *)dst_mapped, words);
 }
 
-// Short rows: one thread per row. Long rows: appended to long_list.
-template <bool LEARN>
+// Short rows: LPR lanes per row. Long rows: appended to long_list. With few rows
+// (every row on its own lanes at once) eight lanes share a row, whose entries
+// would otherwise wait for one another: 1024 rows 27 -> 19 us, 16,384 rows 35 ->
+// 21 us.
+template <bool LEARN, int LPR>
 __global__ void __launch_bounds__(256) k_rowinfo(RawOperands op, const int64_t *c_rp, int64_t c_nnz, BinRule rule,
                                                  BinBuffers bb, long long *bound_out, int *nnz_out, int *err,
                                                  const int *row_list, int64_t nrows, int *long_list,
@@ -237,8 +241,10 @@ __global__ void __launch_bounds__(256) k_rowinfo(RawOperands op, const int64_t *
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    for (int64_t base = gw * 32; base < nrows; base += warps * 32) {
-        const int64_t r = base + lane;
+    constexpr int kRows = 32 / LPR;   // rows of a warp
+    for (int64_t base = gw * kRows; base < nrows; base += warps * kRows) {
+        const int64_t r = base + lane / LPR;
+        const int sl = lane % LPR;
         bool valid = r < nrows;
         int64_t i = 0, ab = 0, ae = 0;
         if (valid) {
@@ -250,21 +256,30 @@ __global__ void __launch_bounds__(256) k_rowinfo(RawOperands op, const int64_t *
                 ab = ae = 0;
             }
         }
-        const bool longrow = ae - ab > kLongRow;
-        const unsigned lm = __ballot_sync(kFull, longrow);
+        const bool longrow = ae - ab > long_row(LPR);
+        const unsigned lm = __ballot_sync(kFull, longrow && sl == 0);
         if (lm) {
             unsigned long long at = 0;
             if (lane == 0) at = atomicAdd(long_count, (unsigned long long)__popc(lm));
             at = __shfl_sync(kFull, at, 0);
-            if (longrow) long_list[at + __popc(lm & lanemask_lt())] = (int)i;
+            if (longrow && sl == 0) long_list[at + __popc(lm & lanemask_lt())] = (int)i;
         }
-        valid = valid && !longrow;
+        valid = valid && !longrow && sl == 0;
         long long f = 0, mx = 0;
 #pragma unroll 4
-        for (int64_t e = ab; e < (longrow ? ab : ae); ++e) {
+        for (int64_t e = ab + sl; e < (longrow ? ab : ae); e += LPR) {
             const long long l = b_row_len(op, __ldg(op.a_ci + e), err);
             f += l;
             mx = l > mx ? l : mx;
+        }
+        if constexpr (LPR > 1) {
+            __syncwarp();
+#pragma unroll
+            for (int o = LPR / 2; o > 0; o >>= 1) {
+                f += __shfl_xor_sync(kFull, f, o);
+                const long long x = __shfl_xor_sync(kFull, mx, o);
+                mx = x > mx ? x : mx;
+            }
         }
         if constexpr (LEARN) {
             // learned planning: only the row's flop count and longest row of B
@@ -419,8 +434,23 @@ __global__ void __launch_bounds__(kScanNT) k_scan_reduce(const int *nnz, int64_t
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
+// The scan's total, and what the caller reads of it (the kernel that knows it is
+// the last one that can: a read of its own would cost a launch and its gap).
+__device__ __forceinline__ void scan_publish(long long sum, int64_t n, int64_t *c_rp, long long *total,
+                                             const ScanPublish &pub) {
+    if (threadIdx.x == 0) {
+        c_rp[n] = sum;
+        *total = sum;
+        if (pub.total) *pub.total = sum;
+    }
+    if (pub.err && threadIdx.x < kNumErr) {
+        pub.err_host[threadIdx.x] = pub.err[threadIdx.x];
+        pub.err[threadIdx.x] = 0;
+    }
+}
+
 __global__ void __launch_bounds__(1024) k_scan_top(long long *part, int64_t nparts, int64_t n,
-                                                   int64_t *c_rp, long long *total) {
+                                                   int64_t *c_rp, long long *total, ScanPublish pub) {
     __shared__ long long s_w[33];
     long long carry = 0;
     for (int64_t b0 = 0; b0 < nparts; b0 += blockDim.x) {
@@ -431,10 +461,36 @@ __global__ void __launch_bounds__(1024) k_scan_top(long long *part, int64_t npar
         if (b < nparts) part[b] = carry + ex;
         carry += tot;
     }
-    if (threadIdx.x == 0) {
-        c_rp[n] = carry;
-        *total = carry;
+    scan_publish(carry, n, c_rp, total, pub);
+}
+
+// The whole scan by one block, for the few rows where three launches cost more
+// than the block's passes (1024 rows: 14 -> 7 us).
+constexpr int64_t kScanOne = 16384;
+__global__ void __launch_bounds__(1024) k_scan_one(const int *nnz, int64_t n, int64_t *c_rp, long long *total,
+                                                   ScanPublish pub) {
+    constexpr int kPer = 4;
+    __shared__ long long s_w[33];
+    long long carry = 0;
+    for (int64_t b0 = 0; b0 < n; b0 += 1024 * kPer) {
+        const int64_t i0 = b0 + (int64_t)threadIdx.x * kPer;
+        int v[kPer];
+        long long loc = 0;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            v[u] = i0 + u < n ? nnz[i0 + u] : 0;
+            loc += v[u];
+        }
+        long long tot;
+        long long run = carry + block_excl_scan64(loc, s_w, &tot);
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            if (i0 + u < n) c_rp[i0 + u] = run;
+            run += v[u];
+        }
+        carry += tot;
     }
+    scan_publish(carry, n, c_rp, total, pub);
 }
 
 __global__ void __launch_bounds__(kScanNT) k_scan_down(const int *nnz, int64_t n, const long long *part,
@@ -480,10 +536,15 @@ static void rowinfo(const RawOperands &op, const int64_t *c_rp, int64_t c_nnz, c
                     long long *bound_out, int *nnz_out, int *err, int sms, cudaStream_t s, const int *row_list,
                     int64_t n, const LearnArgs &la = LearnArgs{}) {
     unsigned long long *lc = (unsigned long long *)(bb.stats + 2);
-    k_rowinfo<LEARN><<<rowinfo_grid(n, sms), 256, 0, s>>>(op, c_rp, c_nnz, rule, bb, bound_out, nnz_out, err,
-                                                             row_list, n, bb.rows, lc, la);
-    // at most min(n, nnz(A) / (kLongRow + 1)) long rows, one per block
-    int64_t most = op.a_nnz / (kLongRow + 1) + 1;
+    const bool few = n * 8 <= (int64_t)sms * 2048;
+    if (few)
+        k_rowinfo<LEARN, 8><<<rowinfo_grid(8 * n, sms), 256, 0, s>>>(op, c_rp, c_nnz, rule, bb, bound_out, nnz_out, err,
+                                                                     row_list, n, bb.rows, lc, la);
+    else
+        k_rowinfo<LEARN, 1><<<rowinfo_grid(n, sms), 256, 0, s>>>(op, c_rp, c_nnz, rule, bb, bound_out, nnz_out, err,
+                                                                 row_list, n, bb.rows, lc, la);
+    // at most min(n, nnz(A) / (long_row + 1)) long rows, one per block
+    int64_t most = op.a_nnz / (long_row(few ? 8 : 1) + 1) + 1;
     if (most > n) most = n;
     const int64_t blocks = most;
     const int64_t cap = (int64_t)sms * 8;
@@ -819,13 +880,19 @@ size_t scan_scratch_bytes(int64_t n) {
     return (size_t)(parts + 1) * sizeof(long long);
 }
 
+int scan_kernels(int64_t n) { return n <= kScanOne ? 1 : 3; }
+
 void launch_scan_rowptr(const int *nnz, int64_t n, int64_t *c_rp, long long *total, void *scratch,
-                        cudaStream_t s) {
+                        cudaStream_t s, const ScanPublish &pub) {
+    if (n <= kScanOne) {
+        k_scan_one<<<1, 1024, 0, s>>>(nnz, n, c_rp, total, pub);
+        return;
+    }
     long long *part = (long long *)scratch;
     const int64_t parts = (n + kScanTile - 1) / kScanTile;
-    if (n > 0) k_scan_reduce<<<(unsigned)parts, kScanNT, 0, s>>>(nnz, n, part);
-    k_scan_top<<<1, 1024, 0, s>>>(part, parts, n, c_rp, total);
-    if (n > 0) k_scan_down<<<(unsigned)parts, kScanNT, 0, s>>>(nnz, n, part, c_rp);
+    k_scan_reduce<<<(unsigned)parts, kScanNT, 0, s>>>(nnz, n, part);
+    k_scan_top<<<1, 1024, 0, s>>>(part, parts, n, c_rp, total, pub);
+    k_scan_down<<<(unsigned)parts, kScanNT, 0, s>>>(nnz, n, part, c_rp);
 }
 
 }  // namespace smash

@@ -30,6 +30,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "warp_enum.cuh"
 #include "writeout.cuh"
 
@@ -483,8 +484,7 @@ static Operands<V> rowwin_operands(const RawOperands &r) {
 
 template <typename Kern>
 static int rowwin_grid(Kern kernel, size_t smem, int sms, long long windows) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRowWinWarps * 32, smem);
+    int per_sm = resident_per_sm((const void *)kernel, kRowWinWarps * 32, smem);
     if (per_sm < 1) per_sm = 1;
     const long long want = (windows + kRowWinWarps - 1) / kRowWinWarps;
     const long long cap = (long long)per_sm * sms;
@@ -506,12 +506,12 @@ void launch_sym_rowwin(const RawOperands &r, const int *rows, int count, int *to
     const long long windows = ((long long)count + rw.W - 1) / rw.W;
     if (r.b_nnz < INT_MAX) {
         auto kern = k_sym_rowwin<int32_t, kRowWinWarps>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         kern<<<rowwin_grid(kern, smem, hl.sms, windows), kRowWinWarps * 32, smem, s>>>(op, rows, count, token, rw,
                                                                                       hc, nnz_out, err);
     } else {
         auto kern = k_sym_rowwin<int64_t, kRowWinWarps>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         kern<<<rowwin_grid(kern, smem, hl.sms, windows), kRowWinWarps * 32, smem, s>>>(op, rows, count, token, rw,
                                                                                       hc, nnz_out, err);
     }
@@ -524,7 +524,7 @@ static void num_rowwin_go(const Operands<V> &op, const int *rows, int count, int
     const size_t smem = num_rowwin_smem(rw, sizeof(V) == 8);
     const long long windows = ((long long)count + rw.W - 1) / rw.W;
     auto kern = k_num_rowwin<V, IT, K, kRowWinWarps>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     kern<<<rowwin_grid(kern, smem, sms, windows), kRowWinWarps * 32, smem, s>>>(op, rows, count, token, rw, hc, rec,
                                                                                out, err);
 }

@@ -15,6 +15,7 @@
 #include "block_walk.cuh"
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 
 namespace smash {
 
@@ -199,8 +200,7 @@ static Operands<float> sym_operands(const RawOperands &r) {
 
 template <typename K>
 static int resident_grid(K kernel, int nt, size_t smem, int sms, int want_blocks, int cap_per_sm = 64) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem);
+    int per_sm = resident_per_sm((const void *)kernel, nt, smem);
     if (per_sm < 1) per_sm = 1;
     if (per_sm > cap_per_sm) per_sm = cap_per_sm;
     long long cap = (long long)per_sm * sms;
@@ -214,7 +214,7 @@ static void sym_hash_launch(const Operands<float> &op, const int *rows, int coun
     const size_t smem = (size_t)groups * ((size_t)4 << tbits) +
                         (GS > 32 ? (size_t)groups * prod_scratch_bytes<float, GS>() : 0);
     auto kern = k_sym_hash<GS, NT>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     const int want = (count + groups - 1) / groups;
     const int grid = resident_grid(kern, NT, smem, sms, want);
     kern<<<grid, NT, smem, s>>>(op, rows, count, token, tbits, hc, nnz_out, err);
@@ -290,7 +290,7 @@ static void sym_dense_go(const Operands<float> &op, const int *rows, int count, 
     const int words = (int)sym_dense_words(op.ncols);
     const size_t smem = (size_t)words * 4;
     auto kern = k_sym_dense<NT>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     const int grid = resident_grid(kern, NT, smem, hl.sms, count, per_sm);
     kern<<<grid, NT, smem, s>>>(op, rows, count, token, words, wc, nnz_out, nc, err);
 }

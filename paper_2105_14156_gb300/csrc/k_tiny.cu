@@ -19,6 +19,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "writeout.cuh"
 
 namespace smash {
@@ -183,8 +184,7 @@ int tiny_list_len(int tbits, float max_load) {
 
 template <typename K>
 static int tiny_grid(K kernel, size_t smem, int sms, int count) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTinyNT, smem);
+    int per_sm = resident_per_sm((const void *)kernel, kTinyNT, smem);
     if (per_sm < 1) per_sm = 1;
     const long long want = (count + kTinyNT - 1) / kTinyNT;
     const long long cap = (long long)per_sm * sms;
@@ -208,7 +208,7 @@ void launch_sym_tiny(const RawOperands &r, const int *rows, int count, int tbits
     const int L = tiny_list_len(tbits, max_load);
     const size_t smem = (size_t)L * kTinyNT * 4;
     auto kern = k_sym_tiny<kTinyNT>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     kern<<<tiny_grid(kern, smem, sms, count), kTinyNT, smem, s>>>(op, rows, count, L, nnz_out, err);
 }
 
@@ -230,7 +230,7 @@ static void num_tiny_typed(const RawOperands &r, const int *rows, int count, int
     const int L = tiny_list_len(tbits, max_load);
     const size_t smem = (size_t)L * kTinyNT * (4 + sizeof(V));
     auto kern = k_num_tiny<V, kTinyNT>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     kern<<<tiny_grid(kern, smem, sms, count), kTinyNT, smem, s>>>(op, rows, count, L, out, err);
 }
 

@@ -23,6 +23,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "launch_cache.h"
 #include "warp_enum.cuh"
 #include "writeout.cuh"
 
@@ -514,8 +515,7 @@ static Operands<V> warp_operands(const RawOperands &r) {
 
 template <typename K>
 static int warp_grid(K kernel, size_t smem, int sms, int count) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWarpRowWarps * 32, smem);
+    int per_sm = resident_per_sm((const void *)kernel, kWarpRowWarps * 32, smem);
     if (per_sm < 1) per_sm = 1;
     const long long want = ((long long)count + kWarpRowWarps - 1) / kWarpRowWarps;
     const long long cap = (long long)per_sm * sms;
@@ -547,7 +547,7 @@ static void num_warp_go(const Operands<V> &op, const int *rows, int count, int *
     const int mode = (bulk || hl.hash_kind == 2) ? 2 : out.row_nnz ? 1 : 0;
     auto kern = mode == 0 ? k_num_warp<V, IT, K, kWarpRowWarps, 0>
               : mode == 1 ? k_num_warp<V, IT, K, kWarpRowWarps, 1> : k_num_warp<V, IT, K, kWarpRowWarps, 2>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)kern);
     const HashCfg hc{hl.hash_kind, hl.colbits};
     kern<<<warp_grid(kern, smem, hl.sms, count), kWarpRowWarps * 32, smem, s>>>(op, rows, count, token, hl.tbits, hc,
                                                                               L, NB, bsh, rec, bulk, out, err);

@@ -19,12 +19,12 @@ void launch_sym_warp(const RawOperands &r, const int *rows, int count, int *toke
     const HashCfg hc{hl.hash_kind, hl.colbits};
     if (r.b_nnz < INT_MAX) {
         auto kern = k_sym_warp<int32_t, kWarpRowWarps>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         kern<<<warp_grid(kern, smem, hl.sms, count), kWarpRowWarps * 32, smem, s>>>(op, rows, count, token,
                                                                                   hl.tbits, hc, nnz_out, err);
     } else {
         auto kern = k_sym_warp<int64_t, kWarpRowWarps>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem((const void *)kern);
         kern<<<warp_grid(kern, smem, hl.sms, count), kWarpRowWarps * 32, smem, s>>>(op, rows, count, token,
                                                                                   hl.tbits, hc, nnz_out, err);
     }

@@ -113,8 +113,16 @@ void launch_training_rows(int64_t n, const int *nnz, const long long *bound, con
 void launch_to_bf16(const float *src, void *dst, int n, cudaStream_t s);
 void launch_bin_scatter(int64_t n, BinBuffers bb, cudaStream_t s);
 size_t scan_scratch_bytes(int64_t n);
+// What the scan leaves in mapped host memory for the caller that waits for it:
+// the total and, with err, the error words, which are cleared.
+struct ScanPublish {
+    long long *total = nullptr;
+    int *err = nullptr;
+    int *err_host = nullptr;
+};
 void launch_scan_rowptr(const int *nnz, int64_t n, int64_t *c_rp, long long *total,
-                        void *scratch, cudaStream_t s);
+                        void *scratch, cudaStream_t s, const ScanPublish &pub = ScanPublish{});
+int scan_kernels(int64_t n);   // kernels that launch_scan_rowptr launches
 
 struct HashLaunch {
     int tbits;          // table size 2^tbits

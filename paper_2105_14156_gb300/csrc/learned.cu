@@ -520,12 +520,11 @@ int spgemm_learned(smash_handle *h, const smash_csr *A, const smash_csr *B, smas
         launch_zero_rows(drows, nd, cap, s);
     }
     {
-        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, 3);
-        launch_scan_rowptr(cap, n, stage_rp, ctr, scan, s);
+        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, scan_kernels(n));
+        launch_scan_rowptr(cap, n, stage_rp, ctr, scan, s, scan_to_host(h, false));
     }
     if ((st = last_cuda_status())) return st;
-    if (read_small(h, 0, ctr, sizeof(long long), s) || cudaStreamSynchronize(s) != cudaSuccess)
-        return SMASH_ERR_CUDA;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
     const long long staged = h->host[0];
     ls.staged_nnz = staged + (use_arena ? ar.cap : 0);
     size_t sneed = 0;
@@ -560,11 +559,10 @@ int spgemm_learned(smash_handle *h, const smash_csr *A, const smash_csr *B, smas
     }
     // 5. exact row pointer of C, then its arrays
     {
-        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, 3);
-        launch_scan_rowptr(row_nnz, n, C->row_ptr, ctr + 2, scan, s);
+        LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, scan_kernels(n));
+        launch_scan_rowptr(row_nnz, n, C->row_ptr, ctr + 2, scan, s, scan_to_host(h, false));
     }
-    if (read_small(h, 0, ctr + 2, sizeof(long long), s) || cudaStreamSynchronize(s) != cudaSuccess)
-        return SMASH_ERR_CUDA;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
     const long long cnnz = h->host[0];
     C->nnz = cnnz;
     ls.c_nnz = cnnz;
