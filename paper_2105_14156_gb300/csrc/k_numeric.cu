@@ -745,23 +745,31 @@ static void num_hash_go(const Operands<V> &op, const int *rows, int count, int *
     constexpr int groups = NT / GS;
     const int T = 1 << hl.tbits;
     const size_t lim = (size_t)max_smem_per_block();
-    int bm_words = 0;
-    if (GS == NT && bitmap_ratio > 0) {
-        const int words = (op.ncols + 31) / 32;
-        if (num_hash_smem<V>(hl.tbits, GS, words, T / 2) <= lim) bm_words = words;
-    }
     // bucket-rank write-out when its arrays fit next to the tables: room for
     // the rows' distinct columns, T/2 at loads up to 0.5, else 3T/4 (loads up
     // to 0.75) when that fits
     int bcap = inv_load >= 2.f ? T / 2 : T - T / 4;
-    // every row of the bin has more than (T/2)/inv_load columns (else it would
-    // sit in a smaller bin): when that already makes the bitmap write-out
-    // their choice, the bucket arrays would only take shared memory (and
-    // resident groups) away
-    const long long n_min = (long long)((T / 2) / inv_load) + 1;
-    if (bm_words > 0 && (long long)bm_words <= (long long)bitmap_ratio * n_min) bcap = 0;
-    if (bcap > 0 && num_hash_smem<V>(hl.tbits, GS, bm_words, bcap) > lim) bcap = T / 2;
-    if (bcap > 0 && num_hash_smem<V>(hl.tbits, GS, bm_words, bcap) > lim) bcap = 0;
+    if (num_hash_smem<V>(hl.tbits, GS, 0, bcap) > lim) bcap = T / 2;
+    if (num_hash_smem<V>(hl.tbits, GS, 0, bcap) > lim) bcap = 0;
+    // The bitmap write-out only where every row of the bin takes it (rows of
+    // more than (T/2)/inv_load columns; the bucket arrays would then only cost
+    // resident groups), or where some do and there is no bucket write-out. It
+    // holds a bit and a count per column of B: kept ready for rows that never
+    // choose it, it left one 64-thread block per SM at 524,288 columns
+    // (5.77 -> 2.12 ms for the mild square of that size, 1.05 -> 0.77 ms for the
+    // values of a 100,003-row float64 product).
+    int bm_words = 0;
+    if (GS == NT && bitmap_ratio > 0) {
+        const int words = (op.ncols + 31) / 32;
+        const long long least = (long long)((T / 2) / inv_load) + 1, most = (long long)(T / inv_load) + 1;
+        const bool fits = num_hash_smem<V>(hl.tbits, GS, words, 0) <= lim;
+        if (fits && words <= bitmap_ratio * least) {
+            bm_words = words;
+            bcap = 0;
+        } else if (fits && bcap == 0 && words <= bitmap_ratio * most) {
+            bm_words = words;
+        }
+    }
     const bool buckets = bcap > 0;
     const size_t smem = num_hash_smem<V>(hl.tbits, GS, bm_words, bcap);
     auto kern = out.row_nnz ? k_num_hash<V, GS, NT, true> : k_num_hash<V, GS, NT, false>;
