@@ -101,10 +101,10 @@ __host__ __device__ constexpr size_t warp_row_bytes(int T, int L, int NB) {
 // gathered by the learned planning). In exact mode a row whose length equals
 // its product count has no repeated column: nothing to merge, so its products
 // skip the table and go straight to the write-out's staging (keys[p], vals[p]
-// for product p). In capacity mode a row whose products fit its capacity is
+// for product p). A row with few repeated columns (exact mode: at most a quarter
+// more products than entries; capacity mode: products that fit the capacity) is
 // staged the same way and its equal columns are summed after the sort
-// (expand, sort, merge): cheaper than hashing when few columns repeat, which
-// is what such a capacity says.
+// (expand, sort, merge): cheaper than hashing it.
 // MODE: 0 exact mode, 1 capacity mode, 2 either, with the bulk copy-out and
 // the Version 1 write-back available (the first two leave out the code the
 // mode cannot reach: a smaller kernel, fewer instruction-cache misses).
@@ -145,13 +145,15 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
         if (!ok || !a_bounds_ok(ab, ae, op.a_nnz, err)) ab = ae = 0;
         int cnt = 0, full = 0;
         // direct: exact mode, the row's length equals its product count (no
-        // repeated column). merge: capacity mode, the row's products fit its
-        // capacity (the size model sees few repeated columns); its products
-        // are staged as they are and equal columns summed after the sort.
+        // repeated column). merge: few repeated columns (exact mode: at most a
+        // quarter more products than entries; capacity mode: the products fit
+        // the capacity, i.e. the size model sees few); the products are staged
+        // as they are and equal columns summed after the sort.
         const long long f_i = ok ? f_rec : -1;
         const bool cap = MODE == 1 || (MODE == 2 && out.row_nnz != nullptr);
         const bool direct = !cap && f_i >= 0 && n_exp <= lcap && f_i == (long long)n_exp;
-        const bool merge = cap && f_i >= 0 && f_i <= (long long)n_exp && f_i <= lcap && 2 * f_i <= T;
+        const bool merge = f_i >= 0 && f_i <= lcap && 2 * f_i <= T && !direct &&
+                           f_i <= (long long)n_exp + (cap ? 0 : n_exp >> 2);
         if (direct || merge) {
             warp_enum<V, IT, true>(op, ab, ae, es, err, [&](bool act, int j, V a, V b, int p) {
                 if (act && p < lcap) {
@@ -186,10 +188,13 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
             // (a merged row's length is known after the merge)
             if (lane == 0 && (over || !merge)) out.row_nnz[i] = over ? -1 : tot;
         } else {
-            over = full || tot != n_exp || tot > lcap;
+            // (staged products: as many as were counted; a merged row's length is
+            // checked after the merge)
+            const int want = merge ? (int)f_i : n_exp;
+            over = full || tot > lcap || tot != want;
             if (lane == 0) {
                 if (full || tot > lcap) raise_err(err, kErrTableFull);
-                else if (tot != n_exp) raise_err(err, kErrCountMismatch);
+                else if (tot != want) raise_err(err, kErrCountMismatch);
             }
         }
         __syncwarp();
@@ -294,12 +299,17 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
                     V v = vals[tot + q];
                     for (int y = q + 1; y < tot && keys[tot + y] == sk; ++y) v += vals[tot + y];
                     const int d = run_tot + __popc(m & lanemask_lt());
-                    __stcs(out.c_ci + (c0 + d), sk);
-                    __stcs(out.c_val + (c0 + d), v);
+                    if (d < n_exp) {
+                        __stcs(out.c_ci + (c0 + d), sk);
+                        __stcs(out.c_val + (c0 + d), v);
+                    }
                 }
                 run_tot += __popc(m);
             }
-            if (lane == 0) out.row_nnz[i] = run_tot;
+            if (lane == 0) {
+                if (cap) out.row_nnz[i] = run_tot;
+                else if (run_tot != n_exp) raise_err(err, kErrCountMismatch);
+            }
             __syncwarp();
             for (int q = lane; q < 2 * tot; q += 32) {
                 keys[q] = kEmpty;

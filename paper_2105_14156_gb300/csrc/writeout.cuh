@@ -214,17 +214,18 @@ __device__ __forceinline__ void writeout_bucket(int *keys, V *vals, int T, int *
 }
 
 // ----- write-out: bucket sort and merge of expanded products -----------------
-// For rows whose products were staged as they came (capacity mode, the
-// products fit the row's room): the same grouping by bucket as
+// For rows whose products were staged as they came (they fit the table's half,
+// and few of them share a column): the same grouping by bucket as
 // writeout_bucket, then each product's place in the column-sorted sequence
 // (equal columns ordered by their grouped position) in keys[0..tot),
 // vals[0..tot) (the table is empty by then), then one pass over the sequence
 // that sums each run of equal columns into one entry of C. Returns the number
-// of entries (runs); keys / vals are EMPTY / 0 again afterwards. Needs
-// tot <= cap of the grouped pairs and tot <= T.
+// of entries (runs; those past the row's room n_exp are not stored); keys / vals
+// are EMPTY / 0 again afterwards. Needs tot <= cap of the grouped pairs and
+// tot <= T.
 template <typename V, int GS, int NT>
 __device__ __forceinline__ int writeout_bucket_merge(int *keys, V *vals, int T, int *bc, int *gk, V *gv, int sh,
-                                                     int tot, const NumOutT<V> &out, int64_t c0, int *red) {
+                                                     int tot, int n_exp, const NumOutT<V> &out, int64_t c0, int *red) {
     using G = Group<GS, NT>;
     const int t = G::tid();
     const int NB = T >> 2;
@@ -285,8 +286,10 @@ __device__ __forceinline__ int writeout_bucket_merge(int *keys, V *vals, int T, 
             if (q == 0 || keys[q - 1] != k) {
                 V v = vals[q];
                 for (int y = q + 1; y < n && keys[y] == k; ++y) v += vals[y];
-                __stcs(out.c_ci + (c0 + d), k);
-                __stcs(out.c_val + (c0 + d), v);
+                if (d < n_exp) {
+                    __stcs(out.c_ci + (c0 + d), k);
+                    __stcs(out.c_val + (c0 + d), v);
+                }
                 ++d;
             }
         }
