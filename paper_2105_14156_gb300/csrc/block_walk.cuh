@@ -6,10 +6,11 @@
 // where entry l's row of B starts, its length, a_ik; the warps' loads of the
 // same words hit in L1), lays the batch's products on one line with a scan, and
 // walks its own kWarps-th part of the line. Inside a row of B of which at least
-// 128 products are left, four coalesced loads are issued per lane and round and
-// nothing else is done per product; shorter pieces take steps of 32 products
-// that may span several rows of B (a lane's entry is the number of entries that
-// end at or before its product).
+// kWalkAlone products are left, up to four coalesced loads are issued per lane
+// and round and nothing else is done per product; shorter pieces take steps of
+// 32 products that may span several rows of B (a lane's entry is the number of
+// entries that end at or before its product: some 25 instructions a step more,
+// against the idle lanes of a piece's last step).
 //
 // Measured against staging the entries in shared memory with a block scan and
 // three barriers a batch, and finding the entry in every step (group_products):
@@ -38,19 +39,33 @@ __device__ __forceinline__ int nth_set_bit(unsigned x, int n) {
     return pos;
 }
 
+// Where a column's accumulator and a bitmap word lie in shared memory. Columns of
+// skewed graphs crowd at multiples of powers of two (a low bit of an R-MAT
+// column is 0 with probability .76, so a quarter of them would share one of the
+// 32 banks); the low five bits are mixed with the bits above them, which keeps
+// every aligned group of 32 words in its place.
+// (skewed squares: float64 65,536 rows 5.90 -> 5.82 ms, one-pass float32 131,072
+// rows 11.31 -> 11.19 ms; not worth its instructions in the bitmap pass, 4.20 ->
+// 4.34 ms at 262,144 rows).
+__device__ __forceinline__ unsigned column_place(unsigned off) { return off ^ (((off >> 5) ^ (off >> 10)) & 31u); }
+__device__ __forceinline__ unsigned word_place(unsigned w) { return w ^ (((w >> 5) ^ (w >> 10)) & 31u); }
+
 constexpr int kWalkUnroll = 4;
+constexpr int kWalkAlone = 48;
 
 // f(j, a, b) for every product of A entries [ab, ae) in warp w's share (j: the
 // column, checked by f; a, b: 0 when !NUM). With a sliced B only the entries of
-// op.slice. All 32 lanes call it; f may diverge.
-template <typename V, bool NUM, int kWarps, typename F>
+// op.slice. All 32 lanes call it; f may diverge. IT: type of the positions in B
+// (int32_t when B has fewer than 2^31 entries).
+template <typename V, typename IT, bool NUM, int kWarps, typename F>
 __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, int64_t ae, int w, int *err, F &&f) {
     const int lane = lane_id();
     for (int64_t base = ab; base < ae; base += 32) {
         int len = 0;
-        int64_t bs = 0;
+        int64_t bs64 = 0;
         V av = V(0);
-        if (base + lane < ae) load_a_entry<V, NUM>(op, base + lane, len, bs, av, err);
+        if (base + lane < ae) load_a_entry<V, NUM>(op, base + lane, len, bs64, av, err);
+        IT bs = (IT)bs64;
         const unsigned nz = __ballot_sync(kFull, len > 0);
         if (nz == 0u) continue;
         const int nv = __popc(nz);
@@ -64,7 +79,7 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
         }
         const int incl = warp_incl_scan(len);
         const int total = __shfl_sync(kFull, incl, 31);
-        const int64_t start = bs - (incl - len);   // product p of this entry reads B at start + p
+        const IT start = bs - (IT)(incl - len);   // product p of this entry reads B at start + p
         const int per = (total + kWarps - 1) / kWarps;
         int q = min(w * per, total);
         const int hi = min(q + per, total);
@@ -74,12 +89,13 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
             const int end = last < hi ? last : hi;
             int jv[kWalkUnroll];
             V a_u[kWalkUnroll], b_u[kWalkUnroll];
-            if (end - q >= 32 * kWalkUnroll) {
-                const int64_t st = __shfl_sync(kFull, start, c0);
+            bool act[kWalkUnroll];
+            if (end - q >= kWalkAlone) {
+                const IT st = __shfl_sync(kFull, start, c0) + (IT)lane;
                 V a = V(0);
                 if constexpr (NUM) a = __shfl_sync(kFull, av, c0);
-                const int32_t *pc = op.b_ci + st + lane;
-                const V *pv = op.b_val + st + lane;
+                const int32_t *pc = op.b_ci + st;
+                const V *pv = op.b_val + st;
                 for (; end - q >= 32 * kWalkUnroll; q += 32 * kWalkUnroll) {
 #pragma unroll
                     for (int u = 0; u < kWalkUnroll; ++u) {
@@ -90,10 +106,25 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
 #pragma unroll
                     for (int u = 0; u < kWalkUnroll; ++u) f(jv[u], a, b_u[u]);
                 }
+                if (end - q >= kWalkAlone) {
+#pragma unroll
+                    for (int u = 0; u < kWalkUnroll; ++u) {
+                        act[u] = q + 32 * u + lane < end;
+                        jv[u] = 0;
+                        b_u[u] = V(0);
+                        if (act[u]) {
+                            jv[u] = __ldg(pc + q + 32 * u);
+                            if constexpr (NUM) b_u[u] = __ldg(pv + q + 32 * u);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kWalkUnroll; ++u)
+                        if (act[u]) f(jv[u], a, b_u[u]);
+                    q = end;
+                }
                 __syncwarp();
                 continue;
             }
-            bool act[kWalkUnroll];
 #pragma unroll
             for (int u = 0; u < kWalkUnroll; ++u) {
                 const int p = q + 32 * u;
@@ -104,13 +135,13 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
                 if (p < hi) {   // the same for all lanes
                     const int c = __popc(__ballot_sync(kFull, incl <= p));
                     const int e = incl - p;
-                    const unsigned ends = __reduce_or_sync(kFull, (e >= 1 && e <= 31) ? (1u << e) : 0u);
+                    const unsigned ends = __reduce_or_sync(kFull, (unsigned)(e - 1) < 31u ? 1u << e : 0u);
                     const int ci = c + __popc(ends & ((2u << lane) - 1u));
-                    const int64_t st = __shfl_sync(kFull, start, ci);
+                    const IT st = __shfl_sync(kFull, start, ci) + (IT)lane;
                     if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci);
                     if (act[u]) {
-                        jv[u] = __ldg(op.b_ci + st + p + lane);
-                        if constexpr (NUM) b_u[u] = __ldg(op.b_val + st + p + lane);
+                        jv[u] = __ldg(op.b_ci + st + p);
+                        if constexpr (NUM) b_u[u] = __ldg(op.b_val + st + p);
                     }
                 }
             }

@@ -269,6 +269,8 @@ __device__ __forceinline__ void slice_enum(const Operands<V> &op, int64_t ab, in
     }
 }
 
+constexpr int kWinList = 256;   // columns of a sparse group that the write-out lists
+
 // Item of the window kernel handed to the block by its first thread.
 struct WinItem {
     long long item;   // row of the bin * nw + window (past the end: no more)
@@ -304,10 +306,11 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
     const int words = cpc >> 5;
     V *acc = (V *)smem;
     unsigned *bm = (unsigned *)(smem + (size_t)cpc * sizeof(V));
-    unsigned char *own = (unsigned char *)(bm + words);   // OWN: owner byte of each column
     const int t = threadIdx.x;
     const int lane = lane_id();
     const int wp = t >> 5;
+    unsigned short *list = (unsigned short *)(bm + words) + wp * kWinList;
+    unsigned char *own = (unsigned char *)(bm + words) + kWarps * kWinList * 2;   // OWN: owner byte of each column
     for (int j = t; j < cpc; j += NT) acc[j] = dense_unused(V(0));
     for (int w = t; w < words; w += NT) bm[w] = 0u;
     const int64_t items = (int64_t)count * nw;
@@ -367,9 +370,9 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                     __syncwarp();
                     const bool win = pend && own[off] == (unsigned char)lane;
                     if (win) {
-                        acc[off] += v;
+                        acc[column_place(off)] += v;
                         const unsigned bit = 1u << (off & 31);
-                        unsigned *bw = bm + (off >> 5);
+                        unsigned *bw = bm + word_place(off >> 5);
                         if (!(*(volatile unsigned *)bw & bit)) atomicOr(bw, bit);
                     }
                     __syncwarp();
@@ -378,11 +381,11 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
             });
         } else {
             op.slice = w;
-            block_walk<V, true, kWarps>(op, ab, ae, wp, err, [&](int j, V a, V bkj) {
+            block_walk<V, int32_t, true, kWarps>(op, ab, ae, wp, err, [&](int j, V a, V bkj) {
                 const unsigned off = (unsigned)(j - lo);
                 if (off < (unsigned)width) {
-                    if (!dense_used(atomicAdd(acc + off, dense_product(a, bkj))))
-                        atomicOr(bm + (off >> 5), 1u << (off & 31));
+                    if (!dense_used(atomicAdd(acc + column_place(off), dense_product(a, bkj))))
+                        atomicOr(bm + word_place(off >> 5), 1u << (off & 31));
                 } else if ((unsigned)j >= (unsigned)op.ncols) {
                     raise_err(err, kErrBadIndex);
                 }
@@ -415,7 +418,7 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
         const int x0 = min(wp * run, wwords), x1 = min(x0 + run, wwords);
         {
             int c = 0;
-            for (int x = x0 + lane; x < x1; x += 32) c += __popc(bm[x]);
+            for (int x = x0 + lane; x < x1; x += 32) c += __popc(bm[word_place(x)]);
             c = __reduce_add_sync(kFull, c);
             if (lane == 0) s_tot[wp] = c;
         }
@@ -452,19 +455,21 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
         V *dst_val = (arena ? (V *)ar.val : out.c_val) + c0 + base;
         for (int xb = x0; xb < x1; xb += 32) {
             const int nx = min(32, x1 - xb);
-            const unsigned word = lane < nx ? bm[xb + lane] : 0u;
-            if (lane < nx) bm[xb + lane] = 0u;
+            unsigned *bw = bm + word_place(xb + lane);
+            const unsigned word = lane < nx ? *bw : 0u;
+            if (lane < nx) *bw = 0u;
             const int incl = warp_incl_scan(__popc(word));
             const int T = __shfl_sync(kFull, incl, 31);
-            if (T >= 8 * nx) {
+            if (T >= 8 * nx) {   // (T < 256 = kWinList otherwise)
                 // dense group: word by word, lane = bit
                 for (int q = 0; q < nx; ++q) {
                     const unsigned wq = __shfl_sync(kFull, word, q);
                     const int pre = __shfl_sync(kFull, incl, q) - __popc(wq);
                     if ((wq >> lane) & 1u) {
                         const int col = ((xb + q) << 5) + lane;
-                        const V v = acc[col];
-                        acc[col] = dense_unused(V(0));
+                        V *word_of = acc + column_place(col);
+                        const V v = *word_of;
+                        *word_of = dense_unused(V(0));
                         const int pos = at + pre + __popc(wq & lanemask_lt());
                         if (ok) {
                             __stcs(dst_ci + pos, lo + col);
@@ -473,28 +478,28 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                     }
                 }
             } else {
-                // sparse group: 32 consecutive outputs per step; the owner word of
-                // output o is the first lane whose inclusive count exceeds o
-                for (int o0 = 0; o0 < T; o0 += 32) {
-                    const int o = o0 + lane;
-                    int L = 0;
-#pragma unroll
-                    for (int st = 16; st >= 1; st >>= 1) {
-                        const int v = __shfl_sync(kFull, incl, L + st - 1);
-                        if (v <= o) L += st;
-                    }
-                    const unsigned wl = __shfl_sync(kFull, word, L);
-                    const int el = __shfl_sync(kFull, incl, L) - __popc(wl);
-                    if (o < T) {
-                        const int col = ((xb + L) << 5) + nth_set_bit(wl, o - el);
-                        const V v = acc[col];
-                        acc[col] = dense_unused(V(0));
-                        if (ok) {
-                            __stcs(dst_ci + (at + o), lo + col);
-                            __stcs(dst_val + (at + o), v);
-                        }
+                // sparse group: the set bits' places listed in order (each lane
+                // its word's), then 32 consecutive outputs per step
+                unsigned rest = word;
+                int pos = incl - __popc(word);
+                while (__any_sync(kFull, rest)) {
+                    if (rest) {
+                        list[pos++] = (unsigned short)((lane << 5) + __ffs(rest) - 1);
+                        rest &= rest - 1;
                     }
                 }
+                __syncwarp();
+                for (int o = lane; o < T; o += 32) {
+                    const int col = (xb << 5) + list[o];
+                    V *word_of = acc + column_place(col);
+                    const V v = *word_of;
+                    *word_of = dense_unused(V(0));
+                    if (ok) {
+                        __stcs(dst_ci + (at + o), lo + col);
+                        __stcs(dst_val + (at + o), v);
+                    }
+                }
+                __syncwarp();
             }
             at += T;
         }
@@ -819,23 +824,25 @@ int dense_bitmap_max_cols() {
 
 static int window_threads(int blocks_per_sm) { return blocks_per_sm <= 1 ? 1024 : blocks_per_sm == 2 ? 512 : 256; }
 
-// Accumulator, occupancy bitmap, then the columns' owner bytes (owner computes).
+// Accumulator, occupancy bitmap, the warps' lists, then the columns' owner bytes
+// (owner computes).
 template <typename V>
-static size_t window_smem(int cpc, bool own) {
-    return (size_t)cpc * sizeof(V) + (size_t)(cpc / 32) * 4 + (own ? (size_t)cpc : 0);
+static size_t window_smem(int cpc, int nt, bool own) {
+    return (size_t)cpc * sizeof(V) + (size_t)(cpc / 32) * 4 + (size_t)(nt / 32) * kWinList * 2 + (own ? (size_t)cpc : 0);
 }
 
 int window_warps(int blocks_per_sm) { return window_threads(blocks_per_sm < 1 ? 1 : blocks_per_sm) / 32; }
 
 int num_window_cols(int dtype, int blocks_per_sm, bool own) {
     const int bps = blocks_per_sm < 1 ? 1 : blocks_per_sm;
+    const int nt = window_threads(bps);
     // per-block budget: the SM's shared memory shared by bps blocks (1 KB
     // reserved per block, ~1 KB of static shared variables)
     long long budget = (long long)max_smem_per_sm() / bps - 1024 - 1024;
     if (budget > max_smem_per_block() - 1024) budget = max_smem_per_block() - 1024;
     int best = 0;
     for (int cpc = kSubCols; cpc <= kMaxWinCols; cpc += kSubCols) {
-        const size_t need = dtype ? window_smem<double>(cpc, own) : window_smem<float>(cpc, own);
+        const size_t need = dtype ? window_smem<double>(cpc, nt, own) : window_smem<float>(cpc, nt, own);
         if ((long long)need <= budget) best = cpc;
     }
     return best;
@@ -849,7 +856,7 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     int cpc = sl.cpc;
     int subs = cpc / kSubCols;
     if (sl.nslices <= 1) {
-        cpc = (op.ncols + 31) & ~31;   // one window holds every column
+        cpc = (op.ncols + 1023) & ~1023;   // one window holds every column (whole groups of word_place)
         subs = wc.nsub;
     } else {
         op.b_ci = sl.ci;
@@ -859,7 +866,7 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     }
     const int nw = sl.nslices <= 1 ? 1 : sl.nslices / sl.per_win;
     const long long items = (long long)count * nw;
-    const size_t smem = window_smem<V>(cpc, own);
+    const size_t smem = window_smem<V>(cpc, NT, own);
     if (own) {
         auto kern = k_num_window<V, NT, true>;
         allow_smem((const void *)kern);

@@ -77,7 +77,7 @@ __device__ __forceinline__ void count_check(const NumCheck &nc, int i, int tot, 
 // kSubCols columns, four words a lane, and counts and clears it in one pass.
 // words: of the bitmap, a multiple of kSubCols / 32. Bound by instruction issue
 // and the shared-memory pipe (half the cycles each; figures in block_walk.cuh).
-template <int NT>
+template <int NT, typename IT>
 __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int *rows, int count, int *token,
                                                   int words, WinCount wc, int *nnz_out, NumCheck nc, int *err) {
     using G = Group<NT, NT>;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
         } else {
             int64_t ab, ae;
             a_row_range(op, i, ab, ae, err);
-            block_walk<float, false, kWarps>(op, ab, ae, wp, err, [&](int j, float, float) {
+            block_walk<float, IT, false, kWarps>(op, ab, ae, wp, err, [&](int j, float, float) {
                 if ((unsigned)j < (unsigned)op.ncols) {
                     const unsigned bit = 1u << (j & 31);
                     unsigned *w = bm + (j >> 5);
@@ -289,7 +289,7 @@ static void sym_dense_go(const Operands<float> &op, const int *rows, int count, 
                          cudaStream_t s) {
     const int words = (int)sym_dense_words(op.ncols);
     const size_t smem = (size_t)words * 4;
-    auto kern = k_sym_dense<NT>;
+    auto kern = op.b_nnz < INT_MAX ? k_sym_dense<NT, int32_t> : k_sym_dense<NT, int64_t>;
     allow_smem((const void *)kern);
     const int grid = resident_grid(kern, NT, smem, hl.sms, count, per_sm);
     kern<<<grid, NT, smem, s>>>(op, rows, count, token, words, wc, nnz_out, nc, err);
