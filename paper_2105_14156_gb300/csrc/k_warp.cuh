@@ -70,14 +70,17 @@ __global__ void __launch_bounds__(NW * 32) k_sym_warp(Operands<float> op, const 
         if (r >= count) break;
         int64_t ab, ae;
         a_row_range(op, i, ab, ae, err);
-        int cnt = 0, full = 0;
-        warp_enum<float, IT, false>(op, ab, ae, es, err, [&](bool act, int j, float, float, int) {
+        int cnt = 0, full = 0;   // (this lane's inserts)
+        unsigned top;
+        warp_walk<float, IT, false>(op, ab, ae, es, err, top, [&](bool act, int j, float, float, int) {
             bool ins = false;
             if (act && cas_insert(keys, tbits, hc, j, ins) < 0) full = 1;
-            cnt += __popc(__ballot_sync(kFull, ins));
+            cnt += ins ? 1 : 0;
         });
         claim.prefetch(count);
-        if (__any_sync(kFull, full) && lane == 0) raise_err(err, kErrTableFull);
+        if (full) raise_err(err, kErrTableFull);
+        if (top >= (unsigned)op.ncols) raise_err(err, kErrBadIndex);
+        cnt = __reduce_add_sync(kFull, cnt);
         if (lane == 0) nnz_out[i] = cnt;
         __syncwarp();
         // back to EMPTY for the next row (16-byte stores)
@@ -97,8 +100,22 @@ __host__ __device__ constexpr size_t warp_row_bytes(int T, int L, int NB) {
 }
 
 // Bucket counts to bucket starts, by one warp: each lane a run of buckets.
+// Eight or four counts a lane are read and written as 16-byte words: one by one
+// the lanes' runs meet in four or eight of the 32 banks (48 of 212 us of the
+// 512-slot rows of a 524,288-row mild square).
 __device__ __forceinline__ void warp_prefix(int *bc, int NB) {
     const int run = (NB + 31) >> 5;
+    if (NB == 256 || NB == 128) {
+        int4 *w = (int4 *)bc + lane_id() * (run >> 2);
+        int4 x = w[0], y = run == 8 ? w[1] : make_int4(0, 0, 0, 0);
+        const int sx = x.x + x.y + x.z + x.w;
+        const int loc = sx + y.x + y.y + y.z + y.w;
+        int acc = warp_incl_scan(loc) - loc;
+        w[0] = make_int4(acc, acc + x.x, acc + x.x + x.y, acc + x.x + x.y + x.z);
+        acc += sx;
+        if (run == 8) w[1] = make_int4(acc, acc + y.x, acc + y.x + y.y, acc + y.x + y.y + y.z);
+        return;
+    }
     const int b0 = min(lane_id() * run, NB), b1 = min(b0 + run, NB);
     int loc = 0;
     for (int b = b0; b < b1; ++b) loc += bc[b];
@@ -178,25 +195,25 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
             dirty = 0;
             __syncwarp();
         }
+        unsigned top;
         if (MODE != 2 && (direct || merge)) {
-            warp_enum<V, IT, true>(op, ab, ae, es, err, [&](bool act, int j, V a, V b, int p) {
+            cnt = warp_walk<V, IT, true>(op, ab, ae, es, err, top, [&](bool act, int j, V a, V b, int p) {
                 if (act && p < lcap) {
                     keys[p] = j;
                     vals[p] = a * b;
-                    atomicAdd(bc + (j >> bsh), 1);   // bucket counts of the write-out
+                    // bucket counts of the write-out (which a bad column never reaches)
+                    atomicAdd(bc + min((unsigned)j >> bsh, (unsigned)NB - 1u), 1);
                 }
-                cnt += __popc(__ballot_sync(kFull, act));
             });
         } else if (MODE == 2 && direct) {
-            warp_enum<V, IT, true>(op, ab, ae, es, err, [&](bool act, int j, V a, V b, int p) {
+            cnt = warp_walk<V, IT, true>(op, ab, ae, es, err, top, [&](bool act, int j, V a, V b, int p) {
                 if (act && p < lcap) {
                     keys[p] = j;
                     vals[p] = a * b;
                 }
-                cnt += __popc(__ballot_sync(kFull, act));
             });
         } else {
-            warp_enum<V, IT, true>(op, ab, ae, es, err, [&](bool act, int j, V a, V b, int) {
+            warp_walk<V, IT, true>(op, ab, ae, es, err, top, [&](bool act, int j, V a, V b, int) {
                 bool ins = false;
                 int h = -1;
                 if (act) {
@@ -213,19 +230,22 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
             });
         }
         claim.prefetch(count);
+        // (a row with a bad column is not written)
+        const bool bad = __any_sync(kFull, top >= (unsigned)op.ncols);
+        if (bad && lane == 0) raise_err(err, kErrBadIndex);
         full = __any_sync(kFull, full);
         const int tot = cnt;
         bool over;
         if (cap) {
-            over = full || tot > n_exp || tot > lcap;
+            over = bad || full || tot > n_exp || tot > lcap;
             // (a merged row's length is known after the merge)
             if (lane == 0 && (over || !merge)) out.row_nnz[i] = over ? -1 : tot;
         } else {
             // (staged products: as many as were counted; a merged row's length is
             // checked after the merge)
             const int want = merge ? (int)f_i : n_exp;
-            over = full || tot > lcap || tot != want;
-            if (lane == 0) {
+            over = bad || full || tot > lcap || tot != want;
+            if (lane == 0 && !bad) {
                 if (full || tot > lcap) raise_err(err, kErrTableFull);
                 else if (tot != want) raise_err(err, kErrCountMismatch);
             }
@@ -277,14 +297,15 @@ __global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int 
                 const int e = bc[b];
                 const int s0 = b ? bc[b - 1] : 0;
                 int rk = s0;
-                for (int y = s0; y < e; ++y) {
-                    const int ky = keys[H + y];
-                    rk += (ky < k || (ky == k && y < q)) ? 1 : 0;
-                }
                 if (direct) {
+                    for (int y = s0; y < e; ++y) rk += keys[H + y] < k ? 1 : 0;
                     __stcs(out.c_ci + (c0 + rk), k);
                     __stcs(out.c_val + (c0 + rk), v);
                 } else {
+                    for (int y = s0; y < e; ++y) {
+                        const int ky = keys[H + y];
+                        rk += (ky < k || (ky == k && y < q)) ? 1 : 0;
+                    }
                     keys[rk] = k;
                     vals[rk] = v;
                 }

@@ -7,8 +7,8 @@
 // moved out of the way; a scan of the lengths lays the batch's products on
 // one line, and each step hands 32 consecutive products to the 32 lanes. The
 // entry of product q + l is the number of entries that end at or before it:
-// those ending before the step (one ballot) plus those ending inside it (one
-// OR-reduction of one bit per end, then a popcount below the lane). Loads of
+// those ending before the step plus those ending inside it (one OR-reduction of
+// one bit per end, then a popcount below the lane). Loads of
 // B are coalesced: consecutive lanes read consecutive entries of a row of B.
 #pragma once
 
@@ -69,16 +69,34 @@ __device__ __forceinline__ int cas_insert(int *keys, int tbits, HashCfg hc, int 
     return -1;
 }
 
+// 1 << t, 0 for t outside [0, 31] (the machine's shift; the language leaves it
+// open).
+__device__ __forceinline__ unsigned bit_or_none(int t) {
+    unsigned r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(t));
+    return r;
+}
+
 // Every product a_ik * b_kj of A entries [ab, ae), enumerated by one warp.
 // f(act, j, a, b, p) is called by all 32 lanes together once per step of 32
 // products (act: the lane holds a product; p: its index among the row's
 // products), so that it may use warp votes.
 // IT: type of the positions in B (int32_t when B has fewer than 2^31 entries).
+// As little per step as it takes: the entries that end inside a step are one
+// OR-reduction of shifted bits and also advance the first entry of the next
+// step, no step is skipped by a branch (a vote or a shuffle inside one costs
+// more than an idle step), and columns are not checked: `top` receives the
+// largest column as an unsigned number, for the caller to compare with cols(B)
+// once per row; f may use j as an index only where any value is harmless.
+// Returns the number of products.
+// (MEASURE_WALKER)
 template <typename V, typename IT, bool NUM, typename F>
-__device__ __forceinline__ void warp_enum(const Operands<V> &op, int64_t ab, int64_t ae, EntryScratch<V> &es,
-                                          int *err, F &&f) {
+__device__ __forceinline__ int warp_walk(const Operands<V> &op, int64_t ab, int64_t ae, EntryScratch<V> &es, int *err,
+                                         unsigned &top, F &&f) {
     const int lane = lane_id();
+    const unsigned lt = lanemask_lt();
     int pbase = 0;   // products of the earlier batches
+    top = 0u;
     for (int64_t base = ab; base < ae; base += 32) {
         int len = 0;
         int64_t bs = 0;
@@ -93,7 +111,7 @@ __device__ __forceinline__ void warp_enum(const Operands<V> &op, int64_t ab, int
         const int nv = __popc(nz);
         if (nv < 32 && nz != (1u << nv) - 1u) {
             if (len > 0) {
-                const int d = __popc(nz & lanemask_lt());
+                const int d = __popc(nz & lt);
                 es.start[d] = bs;
                 es.len[d] = len;
                 if constexpr (NUM) es.av[d] = av;
@@ -107,6 +125,7 @@ __device__ __forceinline__ void warp_enum(const Operands<V> &op, int64_t ab, int
         const int incl = warp_incl_scan(len);
         const int total = __shfl_sync(kFull, incl, 31);
         const IT start = (IT)(bs - (incl - len));   // product p of this entry reads B at start + p
+        int c0 = 0;                                 // entry of a step's first product
         for (int q0 = 0; q0 < total; q0 += 32 * kWarpUnroll) {
             int jv[kWarpUnroll];
             V a_u[kWarpUnroll], b_u[kWarpUnroll];
@@ -114,38 +133,29 @@ __device__ __forceinline__ void warp_enum(const Operands<V> &op, int64_t ab, int
 #pragma unroll
             for (int u = 0; u < kWarpUnroll; ++u) {
                 const int q = q0 + 32 * u;
-                act[u] = q + lane < total;
-                jv[u] = 0;
+                const unsigned ends = __reduce_or_sync(kFull, bit_or_none(incl - 1 - q));
+                const int ci = c0 + __popc(ends & lt);   // (past the last product: any lane)
+                c0 += __popc(ends);
+                const IT idx = __shfl_sync(kFull, start, ci & 31) + (IT)(q + lane);
                 a_u[u] = V(0);
                 b_u[u] = V(0);
-                if (q < total) {
-                    const int c0 = __popc(__ballot_sync(kFull, incl <= q));
-                    const int e = incl - q;
-                    const unsigned ends = __reduce_or_sync(kFull, (e >= 1 && e <= 31) ? (1u << e) : 0u);
-                    const int ci = c0 + __popc(ends & ((2u << lane) - 1u));
-                    const IT st = __shfl_sync(kFull, start, ci);
-                    if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci);
-                    if (act[u]) {
-                        const IT idx = st + (IT)(q + lane);
-                        jv[u] = __ldg(op.b_ci + idx);
-                        if constexpr (NUM) b_u[u] = __ldg(op.b_val + idx);
-                    }
+                if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci & 31);
+                jv[u] = 0;
+                act[u] = q + lane < total;
+                if (act[u]) {
+                    jv[u] = __ldg(op.b_ci + idx);
+                    if constexpr (NUM) b_u[u] = __ldg(op.b_val + idx);
                 }
             }
 #pragma unroll
             for (int u = 0; u < kWarpUnroll; ++u) {
-                if (q0 + 32 * u < total) {
-                    bool ok = act[u];
-                    if (ok && (unsigned)jv[u] >= (unsigned)op.ncols) {
-                        raise_err(err, kErrBadIndex);
-                        ok = false;
-                    }
-                    f(ok, jv[u], a_u[u], b_u[u], pbase + q0 + 32 * u + lane);
-                }
+                top = max(top, (unsigned)jv[u]);
+                f(act[u], jv[u], a_u[u], b_u[u], pbase + q0 + 32 * u + lane);
             }
         }
         pbase += total;
     }
+    return pbase;
 }
 
 // Every product of A entries [ab, ae), enumerated by a group of GS threads

@@ -145,6 +145,34 @@ __device__ __forceinline__ void writeout_bitonic(int *keys, V *vals, int T, int 
     }
 }
 
+// Bucket counts to bucket starts; returns their sum. Four buckets a thread (the
+// usual case) are one 16-byte word: read one by one, the threads' runs meet in
+// eight of the 32 banks.
+template <int GS, int NT>
+__device__ __forceinline__ int bucket_starts(int *bc, int NB, int *red) {
+    using G = Group<GS, NT>;
+    const int t = G::tid();
+    int sum;
+    if (NB == 4 * GS) {
+        int4 *w = (int4 *)bc + t;
+        const int4 x = *w;
+        const int run = G::template excl_scan<int>(x.x + x.y + x.z + x.w, red, &sum);
+        *w = make_int4(run, run + x.x, run + x.x + x.y, run + x.x + x.y + x.z);
+        return sum;
+    }
+    const int per = (NB + GS - 1) / GS;
+    const int b0 = min(t * per, NB), b1 = min(b0 + per, NB);
+    int loc = 0;
+    for (int b = b0; b < b1; ++b) loc += bc[b];
+    int run = G::template excl_scan<int>(loc, red, &sum);
+    for (int b = b0; b < b1; ++b) {
+        const int c = bc[b];
+        bc[b] = run;
+        run += c;
+    }
+    return sum;
+}
+
 // ----- write-out: bucket rank ------------------------------------------------
 // Counting sort by the high bits of the column, then a rank inside each
 // (small) bucket: NB = T/4 buckets, bucket(j) = j >> sh (monotone in j).
@@ -164,19 +192,7 @@ __device__ __forceinline__ void writeout_bucket(int *keys, V *vals, int T, int *
     using G = Group<GS, NT>;
     const int t = G::tid();
     const int NB = T >> 2;
-    {
-        const int per = (NB + GS - 1) / GS;
-        const int b0 = min(t * per, NB), b1 = min(b0 + per, NB);
-        int loc = 0;
-        for (int b = b0; b < b1; ++b) loc += bc[b];
-        int tsum;
-        int run = G::template excl_scan<int>(loc, red, &tsum);
-        for (int b = b0; b < b1; ++b) {
-            const int c = bc[b];
-            bc[b] = run;
-            run += c;
-        }
-    }
+    bucket_starts<GS, NT>(bc, NB, red);
     G::sync();
     // four slots per thread per round, so that their atomics overlap
     for (int s0 = t; s0 < span; s0 += 4 * GS) {
@@ -229,19 +245,8 @@ __device__ __forceinline__ int writeout_bucket_merge(int *keys, V *vals, int T, 
     using G = Group<GS, NT>;
     const int t = G::tid();
     const int NB = T >> 2;
-    int n;   // products counted into the buckets (a product with a bad column was not staged)
-    {
-        const int per = (NB + GS - 1) / GS;
-        const int b0 = min(t * per, NB), b1 = min(b0 + per, NB);
-        int loc = 0;
-        for (int b = b0; b < b1; ++b) loc += bc[b];
-        int run = G::template excl_scan<int>(loc, red, &n);
-        for (int b = b0; b < b1; ++b) {
-            const int c = bc[b];
-            bc[b] = run;
-            run += c;
-        }
-    }
+    // products counted into the buckets (a product with a bad column was not staged)
+    const int n = bucket_starts<GS, NT>(bc, NB, red);
     G::sync();
     // grouped by bucket; the staged slots go back to EMPTY / 0
     for (int s = t; s < tot; s += GS) {
