@@ -139,8 +139,13 @@ __device__ __forceinline__ void warp_prefix(int *bc, int NB) {
 // MODE: 0 exact mode, 1 capacity mode, 2 either, with the bulk copy-out and
 // the Version 1 write-back available (the first two leave out the code the
 // mode cannot reach: a smaller kernel, fewer instruction-cache misses).
+// Blocks per SM that the registers are capped for: what the shared memory of the
+// larger rows allows, 56 registers for the smaller (72 uncapped: 43 % of the
+// warps resident).
+constexpr int warp_rows_resident(int vsz, int K) { return vsz == 8 ? (K <= 4 ? 8 : 6) : (K <= 4 ? 9 : 8); }
+
 template <typename V, typename IT, int K, int NW, int MODE>
-__global__ void __launch_bounds__(NW * 32) k_num_warp(Operands<V> op, const int *rows, int count, int *token,
+__global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_num_warp(Operands<V> op, const int *rows, int count, int *token,
                                                       int tbits, HashCfg hc, int lcap, int nb, int bsh,
                                                       const RowGather *rec, int bulk, NumOutT<V> out, int *err) {
     using G = Group<32, NW * 32>;
