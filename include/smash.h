@@ -345,8 +345,8 @@ int smash_free_csr(smash_handle *h, smash_csr *C);
  * Batched products (not in the paper as such: Version 2's token scheduling
  * applied across many independent products). count pairs (A[m], B[m]) give
  * C[m] = A[m] * B[m]. One cooperative, persistent kernel claims work items
- * (single large rows, then tiles of 8 rows of one product) from a global
- * counter and runs the symbolic counts, the row-pointer scans, the products'
+ * (single large rows, one block each; medium rows, one warp each; chunks of
+ * up to 32 consecutive rows, a warp each) from global counters and runs the symbolic counts, the row-pointer scans, the products'
  * offsets and the numeric values, separated by grid barriers whose waits are
  * bounded (a timeout returns SMASH_ERR_TIMEOUT). Rows too large for one
  * block's table (flagged "huge") are computed around the launch by the
@@ -369,7 +369,9 @@ typedef struct {
 int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_csr *B, smash_dtype dtype,
                    smash_csr *C, smash_batched_stats *stats, void *stream);
 
-/* Per-warp hash-table size of the batched kernel, 2^bits slots, bits in [6, 12] (default 10). */
+/* Per-warp hash-table size of the batched kernel, 2^bits slots, bits in [6, 12] (default 10).
+ * (Products whose B is narrow enough for a warp to own every column, at most
+ * 24 KB of values, use dense accumulators instead, whatever the size.) */
 int smash_batched_set_table_bits(smash_handle *h, int bits);
 int smash_batched_get_table_bits(smash_handle *h, int *bits);
 

@@ -18,8 +18,8 @@
 //
 // One cooperative launch runs four phases separated by grid barriers (each
 // wait bounded; a barrier that times out sets an error word and the kernel
-// returns): counts (and the values of narrow products' rows), per-product row-pointer scans, product base
-// offsets, numeric values with sorted write-out. Rows too large for one
+// returns): counts (and the values of narrow products' rows), per-product
+// row-pointer scans, product base offsets, numeric values with sorted write-out. Rows too large for one
 // block's table are done around the kernel by the regular per-product path.
 #include "device_common.cuh"
 #include "kernels.h"

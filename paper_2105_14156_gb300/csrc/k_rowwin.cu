@@ -62,7 +62,7 @@ __host__ __device__ inline size_t rowwin_num_bytes(const RowWin &rw, int vsz) {
 }
 
 // Every product of the window's rows, enumerated by one warp (the row-window
-// counterpart of warp_enum): f(act, j, a, b, p, r) is called by all 32 lanes
+// counterpart of warp_walk): f(act, j, a, b, p, r) is called by all 32 lanes
 // together once per step of 32 products (p: the product's index on the
 // window's line, r: its row in the window).
 template <typename V, typename IT, bool NUM, typename F>
@@ -89,7 +89,7 @@ __device__ __forceinline__ void window_enum(const Operands<V> &op, int nrows, lo
             b_row_whole(op, __ldg(op.a_ci + apos), len, bs, err);
             if constexpr (NUM) av = op.a_val[apos];
         }
-        // entries with an empty row of B move out of the way (as in warp_enum)
+        // entries with an empty row of B move out of the way (as in warp_walk)
         const unsigned nz = __ballot_sync(kFull, len > 0);
         const int nv = __popc(nz);
         if (nv < 32 && nz != (1u << nv) - 1u) {

@@ -15,7 +15,7 @@
 // any other B the products are added atomically and checked one by one.
 //
 // Measured: 512 batched products of 256-column B (12.5 entries a row, float)
-// 4.48 -> 1.69 ms a call and 24 of 3000 columns (double) 1.41 -> 0.38 ms,
+// 4.40 -> 1.63 ms a call and 24 of 3000 columns (double) 1.46 -> 0.34 ms,
 // against atomic adds with a lane's row found by search, and hash tables with a
 // bitonic sort; the batched kernel now issues on 55 % of the cycles and waits
 // for loads of B otherwise.

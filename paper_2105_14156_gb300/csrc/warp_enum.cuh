@@ -1,6 +1,6 @@
 // Register-staged product enumeration of one warp and compare-and-swap-first
-// insertion, shared by the warp-row kernels (k_warp.cuh) and the batched
-// kernel (k_batched.cu).
+// insertion, shared by the warp rows (k_warp.cuh) and the row windows
+// (k_rowwin.cu), and the enumerator of a block's warps (k_group.cuh).
 //
 // Lane l of each batch of 32 entries of A_i holds entry l (where the row of B
 // it selects starts, its length and a_ik), entries whose row of B is empty
