@@ -9,7 +9,7 @@
 // kWalkAlone products are left, up to four coalesced loads are issued per lane
 // and round and nothing else is done per product; shorter pieces take steps of
 // 32 products that may span several rows of B (a lane's entry is the number of
-// entries that end at or before its product: some 25 instructions a step more,
+// entries that end at or before its product: some 12 instructions a step more,
 // against the idle lanes of a piece's last step).
 //
 // Measured against staging the entries in shared memory with a block scan and
@@ -17,7 +17,10 @@
 // the bitmap pass of the skewed 262,144-row square (2.8 G products) 5.9 -> 3.6 ms
 // (61 -> 33 instructions per 32 products), the float64 windows of the 65,536-row
 // one 4.0 -> 3.9 ms (bound by the adds), whole calls 6.06 -> 4.22 ms and 6.51 ->
-// 6.03 ms.
+// 6.03 ms. With whole rounds inside shorter rows of B (kWalkAlone 48 instead of
+// 128; 33 and 80 are no better), steps that carry their first entry instead of
+// looking it up with a vote, and fewer instructions per bit: 3.54 and 5.61 ms, and
+// the one-pass float32 131,072-row square 11.05 -> 10.65 ms.
 #pragma once
 
 #include "device_common.cuh"
@@ -53,10 +56,43 @@ __device__ __forceinline__ unsigned word_place(unsigned w) { return w ^ (((w >> 
 constexpr int kWalkUnroll = 4;
 constexpr int kWalkAlone = 48;
 
-// f(j, a, b) for every product of A entries [ab, ae) in warp w's share (j: the
-// column, checked by f; a, b: 0 when !NUM). With a sliced B only the entries of
-// op.slice. All 32 lanes call it; f may diverge. IT: type of the positions in B
-// (int32_t when B has fewer than 2^31 entries).
+// One round of S steps of 32 products from product q of the batch's line on (q to
+// hi are the warp's): the entries that end inside a step are one OR-reduction of
+// shifted bits, which also advances the first entry of the next step (c0). No
+// step is skipped by a branch: past hi it only idles.
+template <typename V, typename IT, bool NUM, int S, typename F>
+__device__ __forceinline__ void walk_steps(const Operands<V> &op, int incl, IT start, V av, int q, int hi, int &c0,
+                                           F &&f) {
+    const int lane = lane_id();
+    const unsigned lt = lanemask_lt();
+    int jv[S];
+    V a_u[S], b_u[S];
+    bool act[S];
+#pragma unroll
+    for (int u = 0; u < S; ++u) {
+        const int p = q + 32 * u;
+        const unsigned ends = __reduce_or_sync(kFull, bit_or_none(incl - 1 - p));
+        const int ci = (c0 + __popc(ends & lt)) & 31;   // (past the last product: any lane)
+        c0 += __popc(ends);
+        const IT idx = __shfl_sync(kFull, start, ci) + (IT)(p + lane);
+        a_u[u] = V(0);
+        b_u[u] = V(0);
+        if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci);
+        jv[u] = 0;
+        act[u] = p + lane < hi;
+        if (act[u]) {
+            jv[u] = __ldg(op.b_ci + idx);
+            if constexpr (NUM) b_u[u] = __ldg(op.b_val + idx);
+        }
+    }
+    f(jv, a_u, b_u, act);
+}
+
+// f(j, a, b, act) for every product of A entries [ab, ae) in warp w's share, two
+// or four a lane at a time (arrays; j: the columns, checked by f, 0 where the
+// lane holds no product (act); a, b: 0 when !NUM). With a sliced B only the
+// entries of op.slice. All 32 lanes call it; f may diverge. IT: type of the
+// positions in B (int32_t when B has fewer than 2^31 entries).
 template <typename V, typename IT, bool NUM, int kWarps, typename F>
 __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, int64_t ae, int w, int *err, F &&f) {
     const int lane = lane_id();
@@ -83,28 +119,30 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
         const int per = (total + kWarps - 1) / kWarps;
         int q = min(w * per, total);
         const int hi = min(q + per, total);
+        int c0 = __popc(__ballot_sync(kFull, incl <= q));   // entry of product q (any past the last)
         while (q < hi) {
-            const int c0 = __popc(__ballot_sync(kFull, incl <= q));   // entry of product q
             const int last = __shfl_sync(kFull, incl, c0);
             const int end = last < hi ? last : hi;
-            int jv[kWalkUnroll];
-            V a_u[kWalkUnroll], b_u[kWalkUnroll];
-            bool act[kWalkUnroll];
             if (end - q >= kWalkAlone) {
+                int jv[kWalkUnroll];
+                V a_u[kWalkUnroll], b_u[kWalkUnroll];
+                bool act[kWalkUnroll];
                 const IT st = __shfl_sync(kFull, start, c0) + (IT)lane;
                 V a = V(0);
                 if constexpr (NUM) a = __shfl_sync(kFull, av, c0);
                 const int32_t *pc = op.b_ci + st;
                 const V *pv = op.b_val + st;
+#pragma unroll
+                for (int u = 0; u < kWalkUnroll; ++u) a_u[u] = a;
                 for (; end - q >= 32 * kWalkUnroll; q += 32 * kWalkUnroll) {
 #pragma unroll
                     for (int u = 0; u < kWalkUnroll; ++u) {
+                        act[u] = true;
                         jv[u] = __ldg(pc + q + 32 * u);
                         b_u[u] = V(0);
                         if constexpr (NUM) b_u[u] = __ldg(pv + q + 32 * u);
                     }
-#pragma unroll
-                    for (int u = 0; u < kWalkUnroll; ++u) f(jv[u], a, b_u[u]);
+                    f(jv, a_u, b_u, act);
                 }
                 if (end - q >= kWalkAlone) {
 #pragma unroll
@@ -117,39 +155,18 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
                             if constexpr (NUM) b_u[u] = __ldg(pv + q + 32 * u);
                         }
                     }
-#pragma unroll
-                    for (int u = 0; u < kWalkUnroll; ++u)
-                        if (act[u]) f(jv[u], a, b_u[u]);
+                    f(jv, a_u, b_u, act);
                     q = end;
                 }
-                __syncwarp();
-                continue;
+                if (q == last) ++c0;
+            } else if (hi - q > 32 * (kWalkUnroll / 2)) {
+                walk_steps<V, IT, NUM, kWalkUnroll>(op, incl, start, av, q, hi, c0, f);
+                q += 32 * kWalkUnroll;
+            } else {
+                walk_steps<V, IT, NUM, kWalkUnroll / 2>(op, incl, start, av, q, hi, c0, f);
+                q += 32 * (kWalkUnroll / 2);
             }
-#pragma unroll
-            for (int u = 0; u < kWalkUnroll; ++u) {
-                const int p = q + 32 * u;
-                act[u] = p + lane < hi;
-                jv[u] = 0;
-                a_u[u] = V(0);
-                b_u[u] = V(0);
-                if (p < hi) {   // the same for all lanes
-                    const int c = __popc(__ballot_sync(kFull, incl <= p));
-                    const int e = incl - p;
-                    const unsigned ends = __reduce_or_sync(kFull, (unsigned)(e - 1) < 31u ? 1u << e : 0u);
-                    const int ci = c + __popc(ends & ((2u << lane) - 1u));
-                    const IT st = __shfl_sync(kFull, start, ci) + (IT)lane;
-                    if constexpr (NUM) a_u[u] = __shfl_sync(kFull, av, ci);
-                    if (act[u]) {
-                        jv[u] = __ldg(op.b_ci + st + p);
-                        if constexpr (NUM) b_u[u] = __ldg(op.b_val + st + p);
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kWalkUnroll; ++u)
-                if (act[u]) f(jv[u], a_u[u], b_u[u]);
             __syncwarp();
-            q = min(q + 32 * kWalkUnroll, hi);
         }
     }
     __syncwarp();

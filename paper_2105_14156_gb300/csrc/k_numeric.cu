@@ -381,15 +381,18 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
             });
         } else {
             op.slice = w;
-            block_walk<V, int32_t, true, kWarps>(op, ab, ae, wp, err, [&](int j, V a, V bkj) {
-                const unsigned off = (unsigned)(j - lo);
-                if (off < (unsigned)width) {
-                    if (!dense_used(atomicAdd(acc + column_place(off), dense_product(a, bkj))))
+            unsigned top = 0u;   // largest column, unsigned
+            block_walk<V, int32_t, true, kWarps>(op, ab, ae, wp, err, [&](auto &j, auto &a, auto &b, auto &act) {
+#pragma unroll
+                for (int u = 0; u < (int)(sizeof(act) / sizeof(act[0])); ++u) {
+                    const unsigned off = (unsigned)(j[u] - lo);
+                    top = max(top, (unsigned)j[u]);
+                    if (act[u] && off < (unsigned)width &&
+                        !dense_used(atomicAdd(acc + column_place(off), dense_product(a[u], b[u]))))
                         atomicOr(bm + word_place(off >> 5), 1u << (off & 31));
-                } else if ((unsigned)j >= (unsigned)op.ncols) {
-                    raise_err(err, kErrBadIndex);
                 }
             });
+            if (top >= (unsigned)op.ncols) raise_err(err, kErrBadIndex);
         }
         if (!arena && wp == 0) {
             // columns of the row in the windows before this one, and in this one

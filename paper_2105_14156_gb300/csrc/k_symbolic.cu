@@ -70,13 +70,25 @@ __device__ __forceinline__ void count_check(const NumCheck &nc, int i, int tot, 
     else if ((int64_t)tot != t - s) raise_err(err, kErrCountMismatch);
 }
 
+// Word of a column's bit: an aligned group of 32 words keeps its place, the banks
+// inside it are mixed with the bits above (the columns of skewed graphs crowd in
+// words whose low bits are 0: 262,144-row square 3.64 -> 3.52 ms; a third field as
+// in word_place costs more instructions than it saves conflicts, 3.66 ms).
+__device__ __forceinline__ unsigned bit_place(unsigned c) { return (c >> 5) ^ ((c >> 10) & 31u); }
+constexpr int kSpareWords = 32;   // after the bitmap: hold the bit past the last column when it fills its words
+
 // Dense rows: a bitmap over the columns of B; count = popcount. With wc.wcnt
 // the row's distinct columns are also counted per block of kSubCols columns
 // (slot = wc.slot_base + r), for the numeric dense kernel. The warps share the
 // row's products (block_walk); a warp then takes every kWarps-th block of
 // kSubCols columns, four words a lane, and counts and clears it in one pass.
-// words: of the bitmap, a multiple of kSubCols / 32. Bound by instruction issue
-// and the shared-memory pipe (half the cycles each; figures in block_walk.cuh).
+// words: of the bitmap, a multiple of kSubCols / 32. Bound by the shared-memory
+// pipe (72 % of the cycles: a test and mostly an atomic per product, the lanes'
+// words spread over the banks at random) and instruction issue (55 %, some 26
+// instructions per 32 products).
+// (Columns checked by a branch per product and steps of 32 products looked up
+// with a vote each: 262,144-row square 4.04 ms, now 3.52; training samples and
+// gradient at 65,536 rows 1.39 ms, now 1.19. No test before the atomic: 3.83 ms.)
 template <int NT, typename IT>
 __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int *rows, int count, int *token,
                                                   int words, WinCount wc, int *nnz_out, NumCheck nc, int *err) {
@@ -91,7 +103,7 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
     const int t = threadIdx.x;
     const int lane = lane_id();
     const int wp = t >> 5;
-    for (int x = t; x < words; x += NT) bm[x] = 0u;
+    for (int x = t; x < words + kSpareWords; x += NT) bm[x] = 0u;
     RowClaim<G> claim(token, s_row);   // (its barrier ends the clearing)
     for (;;) {
         const int r = claim.next(count);
@@ -107,17 +119,35 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
         } else {
             int64_t ab, ae;
             a_row_range(op, i, ab, ae, err);
-            block_walk<float, IT, false, kWarps>(op, ab, ae, wp, err, [&](int j, float, float) {
-                if ((unsigned)j < (unsigned)op.ncols) {
-                    const unsigned bit = 1u << (j & 31);
-                    unsigned *w = bm + (j >> 5);
-                    if (!(*(volatile unsigned *)w & bit)) atomicOr(w, bit);
-                } else {
-                    raise_err(err, kErrBadIndex);
+            // columns out of range share the bit past the last column: no
+            // branch per product; the bits' words are read before any is set
+            block_walk<float, IT, false, kWarps>(op, ab, ae, wp, err, [&](auto &j, auto &, auto &, auto &act) {
+                constexpr int U = sizeof(act) / sizeof(act[0]);
+                unsigned at[U], bit[U], had[U];   // (bits set meanwhile are set again)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const unsigned c = min((unsigned)j[u], (unsigned)op.ncols);
+                    at[u] = bit_place(c);
+                    bit[u] = 1u << (c & 31);
+                    had[u] = ~0u;
+                    if (act[u]) had[u] = *(volatile unsigned *)(bm + at[u]);
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (!(had[u] & bit[u])) atomicOr(bm + at[u], bit[u]);
             });
             slot = wc.slot_base + r;
             __syncthreads();
+            // the bit past the last column, by the warp that counts its word
+            if (lane == 0 && wp == (op.ncols / kSubCols) % kWarps) {
+                unsigned *w = bm + bit_place((unsigned)op.ncols);
+                const unsigned bit = 1u << (op.ncols & 31);
+                if (*w & bit) {
+                    *w &= ~bit;
+                    raise_err(err, kErrBadIndex);
+                }
+            }
+            __syncwarp();
             for (int q = wp; q * kSubWords < words; q += kWarps) {
                 uint4 *v = (uint4 *)(bm + q * kSubWords) + lane;
                 const uint4 x = *v;
@@ -254,7 +284,7 @@ static void sym_dense_shape(const HashLaunch &hl, int64_t ncols, int &nt, int &p
     int best_nt = 1024, best_b = 1, best_thr = 0;
     for (int q = 0; q < 3; ++q) {
         if (best_thr == (1 << 30)) break;
-        const size_t per_block = words * 4 + 256 + 1024;   // static variables, reserved by the driver
+        const size_t per_block = (words + kSpareWords) * 4 + 256 + 1024;   // static variables, reserved by the driver
         if (per_block > (size_t)max_smem_per_block() + 1024) continue;
         int b = (int)((size_t)sm_smem / per_block);
         if (b > 2048 / nts[q]) b = 2048 / nts[q];
@@ -288,7 +318,7 @@ static void sym_dense_go(const Operands<float> &op, const int *rows, int count, 
                          const HashLaunch &hl, const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err,
                          cudaStream_t s) {
     const int words = (int)sym_dense_words(op.ncols);
-    const size_t smem = (size_t)words * 4;
+    const size_t smem = (size_t)(words + kSpareWords) * 4;
     auto kern = op.b_nnz < INT_MAX ? k_sym_dense<NT, int32_t> : k_sym_dense<NT, int64_t>;
     allow_smem((const void *)kern);
     const int grid = resident_grid(kern, NT, smem, hl.sms, count, per_sm);

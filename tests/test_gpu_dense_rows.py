@@ -83,3 +83,24 @@ def test_dense_row_bad_columns_are_reported(handle):
         assert e.value.status == 1
     finally:
         handle.set_params(dense_ratio=4, sym_dense_ratio=64)
+
+
+@pytest.mark.parametrize("cols", [8192, 12289])
+@pytest.mark.parametrize("bad", ["cols", "cols + 1", "-1", "2**31 - 1"])
+def test_dense_row_counts_after_a_bad_column(handle, cols, bad):
+    """Columns out of range share the bit past the bitmap's last column (in a spare word where cols(B) fills the
+    others): reported once, and not left in the counts of the next rows or products."""
+    from paper_2105_14156_gb300 import smash
+    A, B = operands(cols, "int", 5)
+    good = B.col_idx.copy()
+    B.col_idx[int(B.row_ptr[15]) - 1] = eval(bad, {"cols": cols})
+    handle.set_params(sym_dense_ratio=1 << 20)
+    try:
+        with pytest.raises(smash.SmashError) as e:
+            handle.symbolic(smash.to_device(A), smash.to_device(B))
+        assert e.value.status == 1
+        B.col_idx = good
+        C = handle.spgemm(smash.to_device(A), smash.to_device(B), check=True).to_host()
+        assert_matches_oracle(C, A, B, exact=True)
+    finally:
+        handle.set_params(sym_dense_ratio=64)
