@@ -42,16 +42,14 @@ __device__ __forceinline__ int nth_set_bit(unsigned x, int n) {
     return pos;
 }
 
-// Where a column's accumulator and a bitmap word lie in shared memory. Columns of
-// skewed graphs crowd at multiples of powers of two (a low bit of an R-MAT
-// column is 0 with probability .76, so a quarter of them would share one of the
-// 32 banks); the low five bits are mixed with the bits above them, which keeps
-// every aligned group of 32 words in its place.
-// (skewed squares: float64 65,536 rows 5.90 -> 5.82 ms, one-pass float32 131,072
-// rows 11.31 -> 11.19 ms; not worth its instructions in the bitmap pass, 4.20 ->
-// 4.34 ms at 262,144 rows).
-__device__ __forceinline__ unsigned column_place(unsigned off) { return off ^ (((off >> 5) ^ (off >> 10)) & 31u); }
-__device__ __forceinline__ unsigned word_place(unsigned w) { return w ^ (((w >> 5) ^ (w >> 10)) & 31u); }
+// Where a column's accumulator lies in shared memory. Columns of skewed graphs
+// crowd at multiples of powers of two (a low bit of an R-MAT column is 0 with
+// probability .76, so a quarter of them would share one of the 32 banks); the
+// low five bits are mixed with the five above, which keeps every aligned group
+// of 32 columns in its place. (Skewed squares, none / these five bits / ten bits
+// and the bitmap's words as well: one-pass float32 131,072 rows 10.84 / 10.49 /
+// 10.65 ms, float64 65,536 rows 5.62 / 5.58 / 5.61 ms.)
+__device__ __forceinline__ unsigned column_place(unsigned off) { return off ^ ((off >> 5) & 31u); }
 
 constexpr int kWalkUnroll = 4;
 constexpr int kWalkAlone = 48;

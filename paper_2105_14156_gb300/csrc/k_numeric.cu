@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                     if (win) {
                         acc[column_place(off)] += v;
                         const unsigned bit = 1u << (off & 31);
-                        unsigned *bw = bm + word_place(off >> 5);
+                        unsigned *bw = bm + (off >> 5);
                         if (!(*(volatile unsigned *)bw & bit)) atomicOr(bw, bit);
                     }
                     __syncwarp();
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
                     top = max(top, (unsigned)j[u]);
                     if (act[u] && off < (unsigned)width &&
                         !dense_used(atomicAdd(acc + column_place(off), dense_product(a[u], b[u]))))
-                        atomicOr(bm + word_place(off >> 5), 1u << (off & 31));
+                        atomicOr(bm + (off >> 5), 1u << (off & 31));
                 }
             });
             if (top >= (unsigned)op.ncols) raise_err(err, kErrBadIndex);
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
         const int x0 = min(wp * run, wwords), x1 = min(x0 + run, wwords);
         {
             int c = 0;
-            for (int x = x0 + lane; x < x1; x += 32) c += __popc(bm[word_place(x)]);
+            for (int x = x0 + lane; x < x1; x += 32) c += __popc(bm[x]);
             c = __reduce_add_sync(kFull, c);
             if (lane == 0) s_tot[wp] = c;
         }
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *ro
         V *dst_val = (arena ? (V *)ar.val : out.c_val) + c0 + base;
         for (int xb = x0; xb < x1; xb += 32) {
             const int nx = min(32, x1 - xb);
-            unsigned *bw = bm + word_place(xb + lane);
+            unsigned *bw = bm + xb + lane;
             const unsigned word = lane < nx ? *bw : 0u;
             if (lane < nx) *bw = 0u;
             const int incl = warp_incl_scan(__popc(word));
@@ -859,7 +859,7 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     int cpc = sl.cpc;
     int subs = cpc / kSubCols;
     if (sl.nslices <= 1) {
-        cpc = (op.ncols + 1023) & ~1023;   // one window holds every column (whole groups of word_place)
+        cpc = (op.ncols + 31) & ~31;   // one window holds every column
         subs = wc.nsub;
     } else {
         op.b_ci = sl.ci;

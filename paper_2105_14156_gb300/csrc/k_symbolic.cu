@@ -72,8 +72,8 @@ __device__ __forceinline__ void count_check(const NumCheck &nc, int i, int tot, 
 
 // Word of a column's bit: an aligned group of 32 words keeps its place, the banks
 // inside it are mixed with the bits above (the columns of skewed graphs crowd in
-// words whose low bits are 0: 262,144-row square 3.64 -> 3.52 ms; a third field as
-// in word_place costs more instructions than it saves conflicts, 3.66 ms).
+// words whose low bits are 0: 262,144-row square 3.64 -> 3.52 ms; a third field
+// costs more instructions than it saves conflicts, 3.66 ms).
 __device__ __forceinline__ unsigned bit_place(unsigned c) { return (c >> 5) ^ ((c >> 10) & 31u); }
 constexpr int kSpareWords = 32;   // after the bitmap: hold the bit past the last column when it fills its words
 
