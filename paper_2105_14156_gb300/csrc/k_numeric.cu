@@ -293,8 +293,14 @@ struct WinItem {
 //
 // Bound by the shared-memory pipe (70 % of the cycles in float: an atomic add is
 // a load and a compare-and-swap) and, in double, by the FP64 pipe (60 %).
+//
+// Double values, 512 threads: the registers of the two blocks that shared memory
+// lets an SM hold are asked for (left alone the compiler spills a few: skewed
+// 65,536-row square 5.57 -> 5.50 ms). In float the same for four blocks of 256
+// is slower, 10.47 -> 10.97 ms at 131,072 rows; so are 320 and 384 threads a
+// block (10.7 ms; 640 and 768 in double 6.0 and 6.3 ms).
 template <typename V, int NT, bool OWN>
-__global__ void __launch_bounds__(NT) k_num_window(Operands<V> op, const int *rows, int count, int nw, int cpc,
+__global__ void __launch_bounds__(NT, sizeof(V) == 8 && NT == 512 && !OWN ? 2 : 0) k_num_window(Operands<V> op, const int *rows, int count, int nw, int cpc,
                                                    int subs_per_win, WinCount wc, WinArena ar, NumOutT<V> out,
                                                    unsigned long long *token, int *err) {
     const bool arena = ar.ci != nullptr;
