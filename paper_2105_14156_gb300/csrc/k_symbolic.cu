@@ -98,14 +98,14 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
     static_assert(kSubWords == 128, "a warp counts a block of columns with one 16-byte load a lane");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_row[2][1];
-    __shared__ int s_part[kWarps];
+    __shared__ int s_part[2][kWarps];   // the warps' counts of this row and of the one before
     unsigned *bm = (unsigned *)smem;
     const int t = threadIdx.x;
     const int lane = lane_id();
     const int wp = t >> 5;
     for (int x = t; x < words + kSpareWords; x += NT) bm[x] = 0u;
     RowClaim<G> claim(token, s_row);   // (its barrier ends the clearing)
-    for (;;) {
+    for (int par = 0;; par ^= 1) {
         const int r = claim.next(count);
         if (r >= count) break;
         const int i = rows[r];
@@ -158,17 +158,19 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
             }
             if (wc.wcnt && t == 0) wc.wslot[i] = (int)slot;
         }
-        if (lane == 0) s_part[wp] = c;
+        // A row counted before has this barrier alone: warp 0 may still read the
+        // counts while the other warps write the next row's, into the other half.
+        // They write this half again behind that row's barrier, which warp 0
+        // reaches after its read.
+        if (lane == 0) s_part[par][wp] = c;
         __syncthreads();
         if (wp == 0) {
-            const int tot = __reduce_add_sync(kFull, lane < kWarps ? s_part[lane] : 0);
+            const int tot = __reduce_add_sync(kFull, lane < kWarps ? s_part[par][lane] : 0);
             if (lane == 0) {
                 if (nnz_out) nnz_out[i] = tot;
                 else count_check(nc, i, tot, err);
             }
         }
-        // s_part is written again only after the next row's first barrier
-        if (counted) __syncthreads();
     }
 }
 

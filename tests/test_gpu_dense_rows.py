@@ -104,3 +104,25 @@ def test_dense_row_counts_after_a_bad_column(handle, cols, bad):
         assert_matches_oracle(C, A, B, exact=True)
     finally:
         handle.set_params(sym_dense_ratio=64)
+
+
+@pytest.mark.parametrize("kind", ["int", "f64"])
+def test_dense_rows_counted_before_and_not(handle, kind):
+    """The numeric count pass over rows that the symbolic bitmap counted (at least half the columns) and rows that it
+    did not (a few products), in turn and many to a block: the sizes of both are checked, and match."""
+    from paper_2105_14156_gb300 import smash
+    cols, rng = 7000, np.random.default_rng(8)
+    lens = [3600, 5, 3501, 1, 4097, 40, 3555, 3]   # rows of B
+    r = np.repeat(np.arange(len(lens)), lens)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lens])
+    rp, ci = csr_from_coo(len(lens), cols, r, c)
+    B = Csr(len(lens), cols, rp, ci, values_of(rng, kind, ci.size))
+    pick = rng.integers(0, len(lens), 9000)   # one row of B each: several rows for each resident block
+    rp, ci = csr_from_coo(pick.size, len(lens), np.arange(pick.size), pick)
+    A = Csr(pick.size, len(lens), rp, ci, values_of(rng, kind, ci.size))
+    handle.set_params(dense_ratio=1 << 20, sym_dense_ratio=2)
+    try:
+        assert_matches_oracle(handle.spgemm(smash.to_device(A), smash.to_device(B), check=True).to_host(), A, B,
+                              exact=kind == "int")
+    finally:
+        handle.set_params(dense_ratio=4, sym_dense_ratio=64)
