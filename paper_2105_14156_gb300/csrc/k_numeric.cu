@@ -164,17 +164,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_hash(Operands<V> op, cons
         }
         clean = false;
         if (!over) {
+            int n = tot;   // entries written
             if (GS == 32 && tot <= 32) {
-                writeout_warp_rank<V>(keys, vals, T, tot, n_exp, out, c0);
+                n = writeout_warp_rank<V>(keys, vals, T, n_exp, out, c0);
             } else if (use_bm) {
                 writeout_bitmap<V, GS, NT>(keys, vals, T, bm, pre, bm_words, n_exp, out, c0, sc.red);
             } else if (bsh >= 0 && tot <= bcap) {
-                writeout_bucket<V, GS, NT>(keys, vals, T, bc, gk, gv, bsh, tot, n_exp, out, c0, sc.red,
-                                           direct ? tot : T);
+                n = writeout_bucket<V, GS, NT>(keys, vals, T, bc, gk, gv, bsh, n_exp, out, c0, sc.red,
+                                               direct ? tot : T);
                 clean = true;
             } else {
                 writeout_bitonic<V, GS, NT>(keys, vals, T, n_exp, out, c0, sc.red);
             }
+            if (n != tot && t == 0) raise_err(err, kErrCountMismatch);   // fewer products than were counted
         }
         claim.publish();
         G::sync();

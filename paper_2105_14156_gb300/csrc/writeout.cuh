@@ -64,9 +64,10 @@ __device__ __forceinline__ bool out_range(const NumOutT<V> &o, int64_t i, int64_
 }
 
 // ----- write-out: warp rank (GS = 32, at most 32 entries) --------------------
+// Returns the number of occupied slots.
 template <typename V>
-__device__ __forceinline__ void writeout_warp_rank(int *keys, V *vals, int T, int tot, int n_exp,
-                                                   const NumOutT<V> &out, int64_t c0) {
+__device__ __forceinline__ int writeout_warp_rank(int *keys, V *vals, int T, int n_exp, const NumOutT<V> &out,
+                                                  int64_t c0) {
     const int lane = lane_id();
     int filled = 0;
     for (int s0 = 0; s0 < T; s0 += 32) {
@@ -83,15 +84,16 @@ __device__ __forceinline__ void writeout_warp_rank(int *keys, V *vals, int T, in
         filled += __popc(b);
         __syncwarp();
     }
-    const int k = lane < tot ? keys[lane] : INT_MAX;
-    const V v = lane < tot ? vals[lane] : V(0);
+    const int k = lane < filled ? keys[lane] : INT_MAX;
+    const V v = lane < filled ? vals[lane] : V(0);
     int rank = 0;
-    for (int m = 0; m < tot; ++m) rank += (__shfl_sync(kFull, k, m) < k) ? 1 : 0;
-    if (lane < tot && rank < n_exp) {
+    for (int m = 0; m < filled; ++m) rank += (__shfl_sync(kFull, k, m) < k) ? 1 : 0;
+    if (lane < filled && rank < n_exp) {
         __stcs(out.c_ci + (c0 + rank), k);
         __stcs(out.c_val + (c0 + rank), v);
     }
     __syncwarp();
+    return filled;
 }
 
 // ----- write-out: compaction + bitonic sort in shared memory ------------------
@@ -181,18 +183,21 @@ __device__ __forceinline__ int bucket_starts(int *bc, int NB, int *red) {
 // grouped by bucket, cap = 3T/4 or T/2 (what shared memory allows). The pass
 // that groups them also returns the table's occupied slots to EMPTY / 0, so
 // the next row needs no clearing. A pair's position is its bucket's start plus
-// the number of smaller columns in its bucket. Needs tot <= cap.
+// the number of smaller columns in its bucket. Needs tot <= cap. Returns the
+// number of pairs grouped and written: tot, or fewer where a staged product had
+// a bad column or a row has fewer products than were counted (the room beyond
+// them in gk holds whatever the enumeration left there).
 template <typename V, int GS, int NT>
-__device__ __forceinline__ void writeout_bucket(int *keys, V *vals, int T, int *bc, int *gk, V *gv, int sh, int tot,
-                                                int n_exp, const NumOutT<V> &out, int64_t c0, int *red,
-                                                int span = -1) {
+__device__ __forceinline__ int writeout_bucket(int *keys, V *vals, int T, int *bc, int *gk, V *gv, int sh,
+                                               int n_exp, const NumOutT<V> &out, int64_t c0, int *red,
+                                               int span = -1) {
     // span: the slots that may be occupied (the whole table unless the
     // entries were staged in its first slots)
     if (span < 0) span = T;
     using G = Group<GS, NT>;
     const int t = G::tid();
     const int NB = T >> 2;
-    bucket_starts<GS, NT>(bc, NB, red);
+    const int n = bucket_starts<GS, NT>(bc, NB, red);
     G::sync();
     // four slots per thread per round, so that their atomics overlap
     for (int s0 = t; s0 < span; s0 += 4 * GS) {
@@ -214,7 +219,7 @@ __device__ __forceinline__ void writeout_bucket(int *keys, V *vals, int T, int *
     }
     G::sync();
     // bc[b] is now the end of bucket b
-    for (int q = t; q < tot; q += GS) {
+    for (int q = t; q < n; q += GS) {
         const int k = gk[q];
         const int b = k >> sh;
         const int e = bc[b];
@@ -227,6 +232,7 @@ __device__ __forceinline__ void writeout_bucket(int *keys, V *vals, int T, int *
             __stcs(out.c_val + (c0 + pos), gv[q]);
         }
     }
+    return n;
 }
 
 // ----- write-out: bucket sort and merge of expanded products -----------------
