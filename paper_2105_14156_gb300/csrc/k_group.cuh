@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(GS) k_num_group(Operands<V> op, const int *row
         __syncthreads();
         bool over;
         if (out.row_nnz) {
-            over = full || tot > n_exp || tot > lcap;
+            // (staged products with a bad column left holes: the call fails)
+            over = full || tot > n_exp || tot > lcap || (merge && tot != (int)f_i);
             if (t == 0 && (over || !merge)) out.row_nnz[i] = over ? -1 : tot;
         } else {
             over = full || tot != n_exp || tot > lcap;

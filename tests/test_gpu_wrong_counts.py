@@ -107,3 +107,29 @@ def test_rows_of_b_emptied_after_the_counts(handle, n, params, dtype):
         expect_refused(handle, dA, dB, c_rp, nnz)
     finally:
         handle.set_params(**base)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("params", KERNELS, ids=lambda p: "-".join(p) or "default")
+@pytest.mark.parametrize("n", [24, 200, 700, 3000])
+def test_bad_columns_in_rows_sized_by_their_bound(handle, n, params, dtype):
+    """The one-pass product: rows whose products fit their room, some of them with a bad column."""
+    from paper_2105_14156_gb300 import smash
+    A, B = disjoint_pairs(n, dtype)
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    good = dB.col_idx.clone()
+    base = {k: handle.params.as_dict()[k] for k in params}
+    handle.set_params(**params)
+    try:
+        for bad in (COLS, -1, 2**31 - 1):
+            dB.col_idx[n // 3] = bad
+            dB.col_idx[10 * n:10 * n + 2 * n // 3] = bad
+            with pytest.raises(smash.SmashError) as e:
+                handle.spgemm_learned(dA, dB, None)
+            assert e.value.status == 1
+            dB.col_idx.copy_(good)
+        C, _, owner = handle.spgemm_learned(dA, dB, None)
+        assert_matches_oracle(C.to_host(), A, B)
+        owner.free()
+    finally:
+        handle.set_params(**base)
