@@ -335,7 +335,8 @@ __device__ void warp_row(const BatchArgs &p, const BatchMat &M, int64_t g, int64
     } else {
         if (lane == 0 && tot != n_exp) raise_err(p.err, kErrCountMismatch);
         NumOutT<V> out{nullptr, p.ci_pool + base, (V *)p.val_pool + base, 0, nullptr};
-        if (tot <= 32) writeout_warp_rank<V>(keys, vals, Tr, n_exp, out, c0);
+        unsigned places = 0u;   // (a table's columns are distinct)
+        if (tot <= 32) writeout_warp_rank<V>(keys, vals, Tr, n_exp, out, c0, places);
         else writeout_bitonic<V, 32, kBNT>(keys, vals, Tr, n_exp, out, c0, nullptr);
     }
     __syncwarp();

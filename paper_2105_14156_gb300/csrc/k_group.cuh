@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(GS) k_num_group(Operands<V> op, const int *row
             // 4. bc[b] is now the end of bucket b: each entry's place is its
             //    bucket's start plus the smaller columns of its bucket (equal
             //    columns, in a merged row, ordered by their grouped position)
+            int places = 0;
 #pragma unroll
             for (int x = 0; x < K; ++x) {
                 if (t + GS * x < tot) {
@@ -200,9 +201,15 @@ __global__ void __launch_bounds__(GS) k_num_group(Operands<V> op, const int *row
                         rk += (ky < kk[x] || (merge && ky == kk[x] && y < pp[x])) ? 1 : 0;
                     }
                     pp[x] = s0 + rk;
+                    places += pp[x];
                 }
             }
             if (!merge) {
+                if (direct) {
+                    // (on top of s_cnt, which every thread has read)
+                    places = __reduce_add_sync(kFull, places);
+                    if (lane == 0) atomicAdd(&s_cnt, places);
+                }
 #pragma unroll
                 for (int x = 0; x < K; ++x) {
                     if (t + GS * x < tot) {
@@ -211,6 +218,8 @@ __global__ void __launch_bounds__(GS) k_num_group(Operands<V> op, const int *row
                     }
                 }
                 __syncthreads();
+                // (no column twice where the products were stored as they came)
+                if (direct && t == 0 && (unsigned)s_cnt != (unsigned)tot + places_sum(tot)) raise_err(err, kErrCountMismatch);
                 for (int q = t; q < tot; q += GS) {
                     keys[q] = kEmpty;
                     vals[q] = V(0);

@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_hash(Operands<V> op, cons
     unsigned *bm = (unsigned *)(smem + (size_t)G::kGroups * grp_bytes);
     int *pre = (int *)(bm + bm_words);
     const int t = G::tid();
+    unsigned places = 0u;   // of the staged rows' entries, less their sums (places_sum)
     bool clean = false;   // the table is EMPTY / 0 (left so by the bucket write-out)
     RowClaimPf<G> claim(token, rows, s_row, s_rowi);
     for (;;) {
@@ -165,21 +166,35 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_hash(Operands<V> op, cons
         clean = false;
         if (!over) {
             int n = tot;   // entries written
+            unsigned row_places = 0u;
             if (GS == 32 && tot <= 32) {
-                n = writeout_warp_rank<V>(keys, vals, T, n_exp, out, c0);
+                n = writeout_warp_rank<V>(keys, vals, T, n_exp, out, c0, row_places);
             } else if (use_bm) {
                 writeout_bitmap<V, GS, NT>(keys, vals, T, bm, pre, bm_words, n_exp, out, c0, sc.red);
             } else if (bsh >= 0 && tot <= bcap) {
-                n = writeout_bucket<V, GS, NT>(keys, vals, T, bc, gk, gv, bsh, n_exp, out, c0, sc.red,
+                n = writeout_bucket<V, GS, NT>(keys, vals, T, bc, gk, gv, bsh, n_exp, out, c0, sc.red, row_places,
                                                direct ? tot : T);
                 clean = true;
             } else {
                 writeout_bitonic<V, GS, NT>(keys, vals, T, n_exp, out, c0, sc.red);
             }
             if (n != tot && t == 0) raise_err(err, kErrCountMismatch);   // fewer products than were counted
+            if (direct) places += row_places - (t == 0 ? places_sum(tot) : 0u);
         }
         claim.publish();
         G::sync();
+    }
+    if (!CAP) {
+        // no column twice in the staged rows
+        places = __reduce_add_sync(kFull, places);
+        if constexpr (GS > 32) {
+            if (t == 0) sc.red[0] = 0;
+            G::sync();
+            if (lane_id() == 0) atomicAdd(sc.red, (int)places);
+            G::sync();
+            places = (unsigned)sc.red[0];
+        }
+        if (t == 0 && places) raise_err(err, kErrCountMismatch);
     }
 }
 

@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
         vals[s] = V(0);
     }
     for (int s = lane; s < NB; s += 32) bc[s] = 0;
-    int dirty = 0;   // slots that staged rows may have left used
+    int dirty = 0;          // slots that staged rows may have left used
+    unsigned places = 0u;   // of the rows' entries that were staged as they came, less their sums (places_sum)
     __syncwarp();
     RowClaimPf<G> claim(token, rows, s_row, nullptr);
     for (;;) {
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
                 int rk = s0;
                 if (direct) {
                     for (int y = s0; y < e; ++y) rk += keys[H + y] < k ? 1 : 0;
+                    places += (unsigned)rk;
                     __stcs(out.c_ci + (c0 + rk), k);
                     __stcs(out.c_val + (c0 + rk), v);
                 } else {
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
             int rank = 0;
             for (int m = 0; m < tot; ++m) rank += __shfl_sync(kFull, k, m) < k ? 1 : 0;
             if (lane < tot) {
+                if (MODE == 2 && direct) places += (unsigned)rank;
                 __stcs(out.c_ci + (c0 + rank), k);
                 __stcs(out.c_val + (c0 + rank), v);
             }
@@ -463,6 +466,7 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
                         const int s0 = b ? bc[b - 1] : 0;
                         int rk = 0;
                         for (int y = s0; y < e; ++y) rk += keys[y] < kk[x] ? 1 : 0;
+                        if (MODE == 2 && direct) places += (unsigned)(s0 + rk);
                         pos[x] = s0 + rk;
                     }
                 }
@@ -505,6 +509,7 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
                         const int s0 = b ? bc[b - 1] : 0;
                         int rk = 0;
                         for (int y = s0; y < e; ++y) rk += keys[y] < kk[x] ? 1 : 0;
+                        if (MODE == 2 && direct) places += (unsigned)(s0 + rk);
                         __stcs(out.c_ci + (c0 + s0 + rk), kk[x]);
                         __stcs(out.c_val + (c0 + s0 + rk), vv[x]);
                     }
@@ -521,8 +526,11 @@ __global__ void __launch_bounds__(NW * 32, warp_rows_resident(sizeof(V), K)) k_n
         // the row took no bucket write-out)
         if (!over && (tot > 32 || (MODE != 2 && (direct || merge))))
             for (int s = lane; s < NB; s += 32) bc[s] = 0;
+        if (MODE != 1 && !over && direct && lane == 0) places -= places_sum(tot);
         __syncwarp();
     }
+    // no column twice in the rows staged as they came
+    if (MODE != 1 && __reduce_add_sync(kFull, places) != 0u && lane == 0) raise_err(err, kErrCountMismatch);
     if (MODE == 2 && bulk && lane == 0) bulk_wait_all();
 }
 

@@ -63,11 +63,20 @@ __device__ __forceinline__ bool out_range(const NumOutT<V> &o, int64_t i, int64_
     return true;
 }
 
+// Entries ranked by the smaller columns of their row take the places 0 .. n-1,
+// whose sum this is, exactly when no column repeats: each pair of equal columns
+// takes one from it. The kernels that store products as they come add the
+// places up over a thread's rows, take each row's sum off again, and look at the
+// remainder (modulo 2^32) once at the end. (Comparing for equality in the rank
+// loops cost 2 to 3 % of a whole product, a sum per row 1 %.)
+__device__ __forceinline__ unsigned places_sum(int n) { return (unsigned)n * (unsigned)(n - 1) / 2u; }
+
 // ----- write-out: warp rank (GS = 32, at most 32 entries) --------------------
-// Returns the number of occupied slots.
+// Returns the number of occupied slots. Adds the place of this lane's entry to
+// `places` (places_sum).
 template <typename V>
 __device__ __forceinline__ int writeout_warp_rank(int *keys, V *vals, int T, int n_exp, const NumOutT<V> &out,
-                                                  int64_t c0) {
+                                                  int64_t c0, unsigned &places) {
     const int lane = lane_id();
     int filled = 0;
     for (int s0 = 0; s0 < T; s0 += 32) {
@@ -88,6 +97,7 @@ __device__ __forceinline__ int writeout_warp_rank(int *keys, V *vals, int T, int
     const V v = lane < filled ? vals[lane] : V(0);
     int rank = 0;
     for (int m = 0; m < filled; ++m) rank += (__shfl_sync(kFull, k, m) < k) ? 1 : 0;
+    if (lane < filled) places += (unsigned)rank;
     if (lane < filled && rank < n_exp) {
         __stcs(out.c_ci + (c0 + rank), k);
         __stcs(out.c_val + (c0 + rank), v);
@@ -186,10 +196,11 @@ __device__ __forceinline__ int bucket_starts(int *bc, int NB, int *red) {
 // the number of smaller columns in its bucket. Needs tot <= cap. Returns the
 // number of pairs grouped and written: tot, or fewer where a staged product had
 // a bad column or a row has fewer products than were counted (the room beyond
-// them in gk holds whatever the enumeration left there).
+// them in gk holds whatever the enumeration left there). Adds the places of
+// this thread's pairs to `places` (places_sum).
 template <typename V, int GS, int NT>
 __device__ __forceinline__ int writeout_bucket(int *keys, V *vals, int T, int *bc, int *gk, V *gv, int sh,
-                                               int n_exp, const NumOutT<V> &out, int64_t c0, int *red,
+                                               int n_exp, const NumOutT<V> &out, int64_t c0, int *red, unsigned &places,
                                                int span = -1) {
     // span: the slots that may be occupied (the whole table unless the
     // entries were staged in its first slots)
@@ -227,6 +238,7 @@ __device__ __forceinline__ int writeout_bucket(int *keys, V *vals, int T, int *b
         int r = 0;
         for (int x = s0; x < e; ++x) r += gk[x] < k ? 1 : 0;
         const int pos = s0 + r;
+        places += (unsigned)pos;
         if (pos < n_exp) {
             __stcs(out.c_ci + (c0 + pos), k);
             __stcs(out.c_val + (c0 + pos), gv[q]);

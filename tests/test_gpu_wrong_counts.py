@@ -133,3 +133,26 @@ def test_bad_columns_in_rows_sized_by_their_bound(handle, n, params, dtype):
         owner.free()
     finally:
         handle.set_params(**base)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("params", KERNELS, ids=lambda p: "-".join(p) or "default")
+@pytest.mark.parametrize("n", [24, 200, 700, 1500, 3000])
+def test_row_pointer_with_an_entry_for_every_product(handle, n, params, dtype):
+    """A caller's row pointer that gives a row as many entries as products although one column repeats."""
+    import torch
+    A, B = disjoint_pairs(n, dtype)
+    from paper_2105_14156_gb300 import smash
+    B.col_idx[B.row_ptr[21]] = B.col_idx[B.row_ptr[20]]   # one column of the 11th row twice (rows of B may be unsorted)
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    base = {k: handle.params.as_dict()[k] for k in params}
+    handle.set_params(**params)
+    try:
+        c_rp, nnz = handle.symbolic(dA, dB)
+        assert nnz == A.rows * n - 1
+        all_products = torch.arange(A.rows + 1, dtype=torch.int64, device="cuda") * n
+        expect_refused(handle, dA, dB, all_products, A.rows * n)
+        C = handle.spgemm(dA, dB, check=True)
+        assert_matches_oracle(C.to_host(), A, B)
+    finally:
+        handle.set_params(**base)
