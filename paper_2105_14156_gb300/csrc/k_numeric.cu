@@ -758,10 +758,14 @@ static size_t num_hash_smem(int tbits, int gs, int bm_words, int bcap = 0) {
     return (size_t)groups * grp + (size_t)bm_words * 8;
 }
 
+// Dynamic shared memory that a block of k_num_hash may have: its claimed rows
+// (static variables, at most 128 bytes) count as well.
+static size_t num_hash_room() { return (size_t)max_smem_per_block() - 128; }
+
 bool num_hash_bitmap_fits(int dtype, int tbits, int ncols) {
     const int words = (ncols + 31) / 32;
     const size_t s = dtype ? num_hash_smem<double>(tbits, 1024, words) : num_hash_smem<float>(tbits, 1024, words);
-    return s <= (size_t)max_smem_per_block();
+    return s <= num_hash_room();
 }
 
 template <typename K>
@@ -781,7 +785,7 @@ static void num_hash_go(const Operands<V> &op, const int *rows, int count, int *
     constexpr int NT = GS < 64 ? 256 : GS;
     constexpr int groups = NT / GS;
     const int T = 1 << hl.tbits;
-    const size_t lim = (size_t)max_smem_per_block();
+    const size_t lim = num_hash_room();
     // bucket-rank write-out when its arrays fit next to the tables: room for
     // the rows' distinct columns, T/2 at loads up to 0.5, else 3T/4 (loads up
     // to 0.75) when that fits

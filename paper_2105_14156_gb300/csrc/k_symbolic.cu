@@ -286,7 +286,7 @@ static void sym_dense_shape(const HashLaunch &hl, int64_t ncols, int &nt, int &p
     int best_nt = 1024, best_b = 1, best_thr = 0;
     for (int q = 0; q < 3; ++q) {
         if (best_thr == (1 << 30)) break;
-        const size_t per_block = (words + kSpareWords) * 4 + 256 + 1024;   // static variables, reserved by the driver
+        const size_t per_block = (words + kSpareWords) * 4 + 320 + 1024;   // static variables, reserved by the driver
         if (per_block > (size_t)max_smem_per_block() + 1024) continue;
         int b = (int)((size_t)sm_smem / per_block);
         if (b > 2048 / nts[q]) b = 2048 / nts[q];

@@ -62,3 +62,25 @@ def test_rows_that_merge_little(handle, kind):
     C, _, owner = handle.spgemm_learned(dA, dB, None)
     assert_matches_oracle(C.to_host(), A, B, exact=kind == "int")
     owner.free()
+
+
+@pytest.mark.parametrize("kind,cols", [("f32", c) for c in (338200, 338304, 338320, 338368, 338369)]
+                         + [("f64", c) for c in (59700, 59776, 59800, 59840, 59841)])
+def test_bitmaps_that_fill_shared_memory(handle, kind, cols):
+    """Rows of the largest tables (4097 to 8192 entries) where the column bitmap beside the table takes all of a
+    block's 227 KB but the last few words, or one more than there is."""
+    from paper_2105_14156_gb300 import smash
+    rng = np.random.default_rng(cols)
+    lens = [4097, 5000, 3000, 8192]
+    r = np.repeat(np.arange(len(lens)), lens)
+    rp, ci = csr_from_coo(len(lens), cols, r, np.concatenate([rng.permutation(cols)[:n] for n in lens]))
+    dtype = np.float32 if kind == "f32" else np.float64
+    B = Csr(len(lens), cols, rp, ci, rng.uniform(-1, 1, ci.size).astype(dtype))
+    ac = [0, 1, 2, 3, 0, 2, 1, 2]   # one row of B each, then pairs
+    rp, ci = csr_from_coo(6, len(lens), np.array([0, 1, 2, 3, 4, 4, 5, 5]), np.array(ac))
+    A = Csr(6, len(lens), rp, ci, rng.uniform(-1, 1, ci.size).astype(dtype))
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B)
+    C, _, owner = handle.spgemm_learned(dA, dB, None)
+    assert_matches_oracle(C.to_host(), A, B)
+    owner.free()
