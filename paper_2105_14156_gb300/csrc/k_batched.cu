@@ -115,17 +115,17 @@ __global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p, int row_bloc
             int64_t x = q - M.seg_off;
             const int64_t eseg = (M.b_nnz + kSegEntries - 1) / kSegEntries;
             long long d;
+            bool bad = false;
             if (x < eseg) {
                 const int64_t e0 = x * kSegEntries;
                 const int64_t e1 = e0 + kSegEntries < M.b_nnz ? e0 + kSegEntries : M.b_nnz;
-                d = descents_between(M.b_ci, e0, e1, M.ncols, threadIdx.x, 256);
+                d = descents_between(M.b_ci, e0, e1, M.ncols, threadIdx.x, 256, bad);
             } else {
                 const int64_t r0 = (x - eseg) * kSegRows;
                 const int64_t r1 = r0 + kSegRows < M.b_rows ? r0 + kSegRows : M.b_rows;
-                d = -descents_at_starts(M.b_rp, M.b_ci, M.b_nnz, r0, r1, threadIdx.x, 256);
+                d = -descents_at_starts(M.b_rp, M.b_ci, M.b_nnz, r0, r1, threadIdx.x, 256, bad);
             }
-            d = warp_sum(d);
-            if (lane == 0 && d) atomicAdd((unsigned long long *)p.descents + lo, (unsigned long long)d);
+            descents_add((unsigned long long *)p.descents + lo, d, bad);
         }
         return;
     }

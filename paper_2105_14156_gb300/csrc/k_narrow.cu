@@ -147,17 +147,17 @@ __global__ void __launch_bounds__(256) k_descents(const int64_t *rp, const int32
     constexpr int64_t kEnt = 8192, kRow = 2048;
     const int64_t eseg = (nnz + kEnt - 1) / kEnt, segs = eseg + (rows + kRow - 1) / kRow;
     long long d = 0;
+    bool bad = false;
     for (int64_t q = blockIdx.x; q < segs; q += gridDim.x) {
         if (q < eseg) {
             const int64_t e0 = q * kEnt;
-            d += descents_between(ci, e0, e0 + kEnt < nnz ? e0 + kEnt : nnz, ncols, threadIdx.x, 256);
+            d += descents_between(ci, e0, e0 + kEnt < nnz ? e0 + kEnt : nnz, ncols, threadIdx.x, 256, bad);
         } else {
             const int64_t r0 = (q - eseg) * kRow;
-            d -= descents_at_starts(rp, ci, nnz, r0, r0 + kRow < rows ? r0 + kRow : rows, threadIdx.x, 256);
+            d -= descents_at_starts(rp, ci, nnz, r0, r0 + kRow < rows ? r0 + kRow : rows, threadIdx.x, 256, bad);
         }
     }
-    d = warp_sum(d);
-    if (lane_id() == 0 && d) atomicAdd((unsigned long long *)descents, (unsigned long long)d);
+    descents_add((unsigned long long *)descents, d, bad);
 }
 
 // Row i of C, room [c0, c0 + n_exp), from the accumulator.

@@ -240,30 +240,42 @@ __device__ __forceinline__ int dense_emit(V *acc, int mode, int ncols, F &&f) {
     return run;
 }
 
-// Whether every row of B ascends, from two coalesced passes: the places e of
-// the whole column array with col[e - 1] >= col[e] (descents_between, over any
-// split of the entries), less those of them where a non-empty row starts
-// (descents_at_starts, over any split of the rows), are none. A column
-// outside [0, ncols) counts as kDescentBad.
-constexpr long long kDescentBad = 1ll << 40;
+// Whether every row of B ascends below cols(B), from two coalesced passes: the
+// places e of the whole column array with col[e - 1] >= col[e]
+// (descents_between, over any split of the entries), less those of them where a
+// non-empty row starts (descents_at_starts, over any split of the rows), are
+// none. A column outside [0, ncols), or a row of B that does not end at or after
+// its start (two others may then start at one place), rules it out: `bad`.
 __device__ __forceinline__ long long descents_between(const int32_t *ci, int64_t e0, int64_t e1, int ncols, int t,
-                                                      int nt) {
+                                                      int nt, bool &bad) {
     long long d = 0;
     for (int64_t e = e0 + t; e < e1; e += nt) {
         const int j = __ldg(ci + e);
         if (e > 0 && __ldg(ci + e - 1) >= j) ++d;
-        if ((unsigned)j >= (unsigned)ncols) d += kDescentBad;
+        if ((unsigned)j >= (unsigned)ncols) bad = true;
     }
     return d;
 }
 __device__ __forceinline__ long long descents_at_starts(const int64_t *rp, const int32_t *ci, int64_t nnz, int64_t r0,
-                                                        int64_t r1, int t, int nt) {
+                                                        int64_t r1, int t, int nt, bool &bad) {
     long long d = 0;
     for (int64_t r = r0 + t; r < r1; r += nt) {
         const int64_t s = __ldg(rp + r), e = __ldg(rp + r + 1);
-        if (s > 0 && e > s && e <= nnz && __ldg(ci + s - 1) >= __ldg(ci + s)) ++d;
+        if (s < 0 || e < s || e > nnz) bad = true;
+        else if (s > 0 && e > s && __ldg(ci + s - 1) >= __ldg(ci + s)) ++d;
     }
     return d;
+}
+// A warp's share of both added to a word that is 0 when B ascends: twice the
+// places, and the lowest bit for `bad` (an even number of any sign never clears
+// it, however many there are).
+__device__ __forceinline__ void descents_add(unsigned long long *word, long long d, bool bad) {
+    d = warp_sum(d);
+    bad = __any_sync(kFull, bad);
+    if (lane_id() == 0) {
+        if (d) atomicAdd(word, (unsigned long long)(2 * d));
+        if (bad) atomicOr(word, 1ull);
+    }
 }
 
 }  // namespace smash

@@ -61,13 +61,16 @@ def b_matrix(cols, lens, k, values, seed):
     return rows_of([min(lens[q % len(lens)], cols) for q in range(k)], cols, values, seed)
 
 
-def run_batch(handle, pairs):
-    from paper_2105_14156_gb300 import smash
-    dev = [(smash.to_device(A), smash.to_device(B)) for A, B in pairs]
-    Cs, _, owner = handle.spgemm_batched(dev)
+def run_batch_device(handle, pairs):
+    Cs, _, owner = handle.spgemm_batched(pairs)
     host = [C.to_host() for C in Cs]
     owner.free()
     return host
+
+
+def run_batch(handle, pairs):
+    from paper_2105_14156_gb300 import smash
+    return run_batch_device(handle, [(smash.to_device(A), smash.to_device(B)) for A, B in pairs])
 
 
 @pytest.mark.parametrize("values", ["f32", "f64", "int"])
@@ -142,3 +145,62 @@ def test_narrow_wrong_sizes_are_reported(handle):
         handle.check()
     assert e.value.status == 1
     assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B)
+
+
+def test_bad_columns_by_the_million_are_reported(handle):
+    """2**24 rows of B that ascend and end in a column past cols(B): still no plain adds, and an error status."""
+    import torch
+    from paper_2105_14156_gb300 import smash
+    k, cols = 1 << 24, 256
+    b_rp = torch.arange(k + 1, dtype=torch.int64, device="cuda") * 3
+    b_ci = torch.tensor([3, 100, cols + 5], dtype=torch.int32, device="cuda").repeat(k)
+    B = smash.DeviceCsr(k, cols, b_rp, b_ci, torch.ones(3 * k, device="cuda"))
+    rows = 1024
+    a_rp = torch.arange(rows + 1, dtype=torch.int64, device="cuda") * (k // rows)
+    A = smash.DeviceCsr(rows, k, a_rp, torch.arange(k, dtype=torch.int32, device="cuda"), torch.ones(k, device="cuda"))
+    with pytest.raises(smash.SmashError) as e:
+        handle.spgemm_learned(A, B, None)
+    assert e.value.status == 1
+    with pytest.raises(smash.SmashError) as e:
+        handle.spgemm_batched([(A, B)])
+    assert e.value.status == 1
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_rows_of_b_that_start_twice_at_one_place(handle, dtype):
+    """A row of B whose end lies before its start, not read by A, so that two others begin at one place; the row after
+    them has a repeated column. The row counts as no more than what A reads of it."""
+    import torch
+    from paper_2105_14156_gb300 import smash
+    rng = np.random.default_rng(3)
+    cols = 64
+    first = np.sort(rng.permutation(cols)[:10])
+    second = np.sort(rng.permutation(first[-1])[:10])      # begins below the first one's end
+    third = np.sort(rng.permutation(cols)[:40])
+    third[20] = third[21]
+    ci = np.concatenate([first, second, third]).astype(np.int32)
+    val = rng.uniform(-1, 1, 60).astype(dtype)
+    rp = np.array([0, 10, 20, 10, 20, 60], np.int64)       # rows 1 and 3 are the same, row 2 has no extent
+    n = 64
+    reads = np.array([0, 1, 3, 4])
+    a_val = rng.uniform(-1, 1, 4 * n).astype(dtype)
+    B = smash.DeviceCsr(5, cols, *(torch.as_tensor(x, device="cuda") for x in (rp, ci, val)))
+    A = smash.DeviceCsr(n, 5, *(torch.as_tensor(x, device="cuda") for x in
+                                (np.arange(n + 1) * 4, np.tile(reads, n).astype(np.int32), a_val)))
+    want, room = np.zeros((n, cols)), np.zeros((n, cols))
+    for i in range(n):
+        for q, r in enumerate(reads):
+            np.add.at(want[i], ci[rp[r]:rp[r + 1]], float(a_val[4 * i + q]) * val[rp[r]:rp[r + 1]].astype(np.float64))
+            np.add.at(room[i], ci[rp[r]:rp[r + 1]], abs(float(a_val[4 * i + q])) * abs(val[rp[r]:rp[r + 1]].astype(np.float64)))
+    results = [handle.spgemm(A, B, check=True).to_host()]
+    C, _, owner = handle.spgemm_learned(A, B, None)
+    results.append(C.to_host())
+    owner.free()
+    results += run_batch_device(handle, [(A, B)])
+    tol = 8 * np.finfo(dtype).eps   # at most five terms an entry: (m - 1 + 1) * u a term, u = eps / 2
+    for C in results:
+        got = np.zeros((n, cols))
+        for i in range(n):
+            got[i, C.col_idx[C.row_ptr[i]:C.row_ptr[i + 1]]] = C.val[C.row_ptr[i]:C.row_ptr[i + 1]]
+            assert set(C.col_idx[C.row_ptr[i]:C.row_ptr[i + 1]]) == set(np.flatnonzero(room[i]))
+        assert (abs(got - want) <= tol * room).all()
