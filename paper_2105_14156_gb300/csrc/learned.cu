@@ -562,6 +562,9 @@ int spgemm_learned(smash_handle *h, const smash_csr *A, const smash_csr *B, smas
         LaunchTimer lt(h, s, "scan_rowptr", -1, 512, n, 0, 0, 0, scan_kernels(n));
         launch_scan_rowptr(row_nnz, n, C->row_ptr, ctr + 2, scan, s, scan_to_host(h, false));
     }
+    // (a launch that was refused shows here, not at the wait: the word that the
+    // scan writes would still hold the overflow count)
+    if ((st = last_cuda_status())) return st;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
     const long long cnnz = h->host[0];
     C->nnz = cnnz;
