@@ -64,6 +64,24 @@ def test_rows_that_merge_little(handle, kind):
     owner.free()
 
 
+@pytest.mark.parametrize("params", [{"bulk_copy": 1}, {"hash_kind": 2}, {"bulk_copy": 1, "hash_kind": 2}],
+                         ids=lambda p: "-".join(p))
+@pytest.mark.parametrize("kind", ["f32", "f64", "int"])
+def test_rows_that_merge_little_with_either_write_out(handle, kind, params):
+    """The same with the bulk copy-out and the order-preserving hash, which one kernel serves in both modes."""
+    from paper_2105_14156_gb300 import smash
+    A, B = overlapping_pairs(kind)
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    handle.set_params(**params)
+    try:
+        assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=kind == "int")
+        C, _, owner = handle.spgemm_learned(dA, dB, None)
+        assert_matches_oracle(C.to_host(), A, B, exact=kind == "int")
+        owner.free()
+    finally:
+        handle.set_params(bulk_copy=0, hash_kind=1)
+
+
 @pytest.mark.parametrize("kind,cols", [("f32", c) for c in (338200, 338304, 338320, 338368, 338369)]
                          + [("f64", c) for c in (59700, 59776, 59800, 59840, 59841)])
 def test_bitmaps_that_fill_shared_memory(handle, kind, cols):
