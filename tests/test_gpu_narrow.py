@@ -204,3 +204,14 @@ def test_rows_of_b_that_start_twice_at_one_place(handle, dtype):
             got[i, C.col_idx[C.row_ptr[i]:C.row_ptr[i + 1]]] = C.val[C.row_ptr[i]:C.row_ptr[i + 1]]
             assert set(C.col_idx[C.row_ptr[i]:C.row_ptr[i + 1]]) == set(np.flatnonzero(room[i]))
         assert (abs(got - want) <= tol * room).all()
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+def test_narrow_phases_of_long_rows_alike(handle, values):
+    """Rows of A all longer than the least heavy row: a warp each where they are many, a block where they are few."""
+    from paper_2105_14156_gb300 import smash
+    for rows in (20, 6000):
+        B = b_matrix(1000, [2, 3, 1], 400, values, 5)
+        A = rows_of([147 + 3 * (q % 5) for q in range(rows)], 400, values, 6)
+        dA, dB = smash.to_device(A), smash.to_device(B)
+        assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=values == "int")
