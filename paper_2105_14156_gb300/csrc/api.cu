@@ -323,7 +323,7 @@ int run_symbolic(smash_handle *h, const RawOperands &op, int64_t n, Plan &pl, in
                 const HashLaunch hl = hash_launch(h, 0, op.ncols);
                 LaunchTimer lt(h, bs, "sym_dense", b, sym_dense_threads(hl, op.ncols), counts[b], sums[b], sums[16 + b],
                                sums[32 + b]);
-                launch_sym_dense(op, rows, counts[b], tok, hl, wc, nnz_out, NumCheck{}, err, bs);
+                launch_sym_dense(op, rows, counts[b], sums[b], sums[16 + b], tok, hl, wc, nnz_out, NumCheck{}, err, bs);
             }
             wcache_set(h, op, nsub, counts[b]);
         } else if (b == kBinSpill) {
@@ -494,8 +494,8 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
             {
                 LaunchTimer lt(h, s, "num_dense_count", bd, sym_dense_threads(hld, op.ncols), counts[bd], sums[bd],
                                sums[16 + bd], sums[32 + bd]);
-                launch_sym_dense(op, pl.bb.rows + offsets[bd], counts[bd], pl.bb.tokens + bd, hld, wc, nullptr, nc,
-                                 err, s);
+                launch_sym_dense(op, pl.bb.rows + offsets[bd], counts[bd], sums[bd], sums[16 + bd],
+                                 pl.bb.tokens + bd, hld, wc, nullptr, nc, err, s);
             }
             h->wcache.slots = base + counts[bd];
         }
@@ -534,8 +534,8 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
             // (row, window) items
             LaunchTimer lt(h, bs, "num_dense_window", b, 1024 / hld.dense_blocks, counts[b], sums[b], sums[16 + b],
                            sums[32 + b]);
-            launch_num_window(dt, op, rows, counts[b], (unsigned long long *)h->split.ptr, hld, sl, wc,
-                              arena ? *arena : WinArena{}, out, err, bs);
+            launch_num_window(dt, op, rows, counts[b], sums[b], sums[16 + b], (unsigned long long *)h->split.ptr, hld,
+                              sl, wc, arena ? *arena : WinArena{}, out, err, bs);
         } else if (b == kBinSpill || b == kBinDense) {
             if (!spill_stream) spill_stream = fk.get(q++);
             cudaStream_t bs = spill_stream;

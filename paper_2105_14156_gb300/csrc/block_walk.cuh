@@ -23,6 +23,8 @@
 // the one-pass float32 131,072-row square 11.05 -> 10.65 ms.
 #pragma once
 
+#include <climits>
+
 #include "device_common.cuh"
 
 namespace smash {
@@ -53,6 +55,26 @@ __device__ __forceinline__ unsigned column_place(unsigned off) { return off ^ ((
 
 constexpr int kWalkUnroll = 4;
 constexpr int kWalkAlone = 48;
+
+// The least entries of A from which a row's warps take whole batches in turn
+// (apart) instead of a part of each. entries, products: of the rows of a launch
+// (entries once for each window); warps: of a block. Every warp loads and scans
+// each batch that it has a part of, which costs more than walking the part where
+// the rows of B are short: every row below kWalkShort products an entry, the rows
+// with a batch for every fourth warp below kWalkShort * 2, with one for every warp
+// below kWalkMedium.
+// (Values of 800 dense rows of 100,000 columns, 13,750 entries of 8 products, in
+// parts and apart: float 6.21 and 1.13 ms, double 12.3 and 1.27 ms; 5,500 of 20: 2.65
+// and 0.68, 5.18 and 0.84 ms. Counts of rows of 1,100 entries of 8: 154 and 110 us; of
+// 59 entries of 50 products 121 us in parts, 145 us apart. The skewed float64 square
+// of 65,536 rows: 5.49 ms in parts, 5.52 so, 5.84 with a batch for every fourth
+// warp below kWalkMedium, 9.6 with every row apart.)
+constexpr int kWalkShort = 16, kWalkMedium = 128;
+inline int walk_apart_from(long long entries, long long products, int warps) {
+    if (products < kWalkShort * entries) return 0;
+    if (products < kWalkShort * 2 * entries) return 8 * warps > 128 ? 8 * warps : 128;
+    return products < kWalkMedium * entries ? 32 * warps : INT_MAX;
+}
 
 // One round of S steps of 32 products from product q of the batch's line on (q to
 // hi are the warp's): the entries that end inside a step are one OR-reduction of
@@ -91,10 +113,13 @@ __device__ __forceinline__ void walk_steps(const Operands<V> &op, int incl, IT s
 // lane holds no product (act); a, b: 0 when !NUM). With a sliced B only the
 // entries of op.slice. All 32 lanes call it; f may diverge. IT: type of the
 // positions in B (int32_t when B has fewer than 2^31 entries).
+// apart: the warps take whole batches in turn instead of a part of each.
 template <typename V, typename IT, bool NUM, int kWarps, typename F>
-__device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, int64_t ae, int w, int *err, F &&f) {
+__device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, int64_t ae, int w, bool apart, int *err,
+                                           F &&f) {
     const int lane = lane_id();
-    for (int64_t base = ab; base < ae; base += 32) {
+    const int step = apart ? 32 * kWarps : 32;
+    for (int64_t base = apart ? ab + 32 * w : ab; base < ae; base += step) {
         int len = 0;
         int64_t bs64 = 0;
         V av = V(0);
@@ -114,8 +139,8 @@ __device__ __forceinline__ void block_walk(const Operands<V> &op, int64_t ab, in
         const int incl = warp_incl_scan(len);
         const int total = __shfl_sync(kFull, incl, 31);
         const IT start = bs - (IT)(incl - len);   // product p of this entry reads B at start + p
-        const int per = (total + kWarps - 1) / kWarps;
-        int q = min(w * per, total);
+        const int per = apart ? total : (total + kWarps - 1) / kWarps;
+        int q = apart ? 0 : min(w * per, total);
         const int hi = min(q + per, total);
         int c0 = __popc(__ballot_sync(kFull, incl <= q));   // entry of product q (any past the last)
         while (q < hi) {

@@ -318,8 +318,8 @@ struct WinItem {
 // block (10.7 ms; 640 and 768 in double 6.0 and 6.3 ms).
 template <typename V, int NT, bool OWN>
 __global__ void __launch_bounds__(NT, sizeof(V) == 8 && NT == 512 && !OWN ? 2 : 0) k_num_window(Operands<V> op, const int *rows, int count, int nw, int cpc,
-                                                   int subs_per_win, WinCount wc, WinArena ar, NumOutT<V> out,
-                                                   unsigned long long *token, int *err) {
+                                                   int subs_per_win, int apart_from, WinCount wc, WinArena ar,
+                                                   NumOutT<V> out, unsigned long long *token, int *err) {
     const bool arena = ar.ci != nullptr;
     constexpr int kWarps = NT / 32;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(NT, sizeof(V) == 8 && NT == 512 && !OWN ? 2 : 
         } else {
             op.slice = w;
             unsigned top = 0u;   // largest column, unsigned
-            block_walk<V, int32_t, true, kWarps>(op, ab, ae, wp, err, [&](auto &j, auto &a, auto &b, auto &act) {
+            block_walk<V, int32_t, true, kWarps>(op, ab, ae, wp, ae - ab >= apart_from, err, [&](auto &j, auto &a, auto &b, auto &act) {
 #pragma unroll
                 for (int u = 0; u < (int)(sizeof(act) / sizeof(act[0])); ++u) {
                     const unsigned off = (unsigned)(j[u] - lo);
@@ -879,8 +879,8 @@ int num_window_cols(int dtype, int blocks_per_sm, bool own) {
 }
 
 template <typename V, int NT>
-static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, int count, unsigned long long *token,
-                          const HashLaunch &hl, const WinCount &wc, const WinArena &ar, const NumOutT<V> &out,
+static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, int count, long long entries,
+                          long long products, unsigned long long *token, const HashLaunch &hl, const WinCount &wc, const WinArena &ar, const NumOutT<V> &out,
                           int *err, cudaStream_t s) {
     const bool own = sl.per_win > 1;   // one slice per warp: owner computes
     int cpc = sl.cpc;
@@ -896,40 +896,41 @@ static void num_window_go(Operands<V> op, const BSlices &sl, const int *rows, in
     }
     const int nw = sl.nslices <= 1 ? 1 : sl.nslices / sl.per_win;
     const long long items = (long long)count * nw;
+    const int apart_from = walk_apart_from(entries * nw, products, NT / 32);
     const size_t smem = window_smem<V>(cpc, NT, own);
     if (own) {
         auto kern = k_num_window<V, NT, true>;
         allow_smem((const void *)kern);
         const int grid = resident_grid(kern, NT, smem, hl.sms, items);
-        kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, wc, ar, out, token, err);
+        kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, apart_from, wc, ar, out, token, err);
     } else {
         auto kern = k_num_window<V, NT, false>;
         allow_smem((const void *)kern);
         const int grid = resident_grid(kern, NT, smem, hl.sms, items);
-        kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, wc, ar, out, token, err);
+        kern<<<grid, NT, smem, s>>>(op, rows, count, nw, cpc, subs, apart_from, wc, ar, out, token, err);
     }
 }
 
 template <typename V>
-static void num_window_typed(const RawOperands &r, const int *rows, int count, unsigned long long *token,
-                             const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
+static void num_window_typed(const RawOperands &r, const int *rows, int count, long long entries, long long products,
+                             unsigned long long *token, const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
                              const NumOut &o, int *err, cudaStream_t s) {
     const Operands<V> op = num_operands<V>(r);
     const NumOutT<V> out = num_out<V>(o);
     switch (window_threads(hl.dense_blocks)) {
-        case 1024: num_window_go<V, 1024>(op, sl, rows, count, token, hl, wc, ar, out, err, s); break;
-        case 512: num_window_go<V, 512>(op, sl, rows, count, token, hl, wc, ar, out, err, s); break;
-        default: num_window_go<V, 256>(op, sl, rows, count, token, hl, wc, ar, out, err, s); break;
+        case 1024: num_window_go<V, 1024>(op, sl, rows, count, entries, products, token, hl, wc, ar, out, err, s); break;
+        case 512: num_window_go<V, 512>(op, sl, rows, count, entries, products, token, hl, wc, ar, out, err, s); break;
+        default: num_window_go<V, 256>(op, sl, rows, count, entries, products, token, hl, wc, ar, out, err, s); break;
     }
 }
 
-void launch_num_window(int dtype, const RawOperands &r, const int *rows, int count, unsigned long long *token,
-                       const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
+void launch_num_window(int dtype, const RawOperands &r, const int *rows, int count, long long entries,
+                       long long products, unsigned long long *token, const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
                        const NumOut &out, int *err, cudaStream_t s) {
     if (count <= 0) return;
     cudaMemsetAsync(token, 0, sizeof(unsigned long long), s);
-    if (dtype) num_window_typed<double>(r, rows, count, token, hl, sl, wc, ar, out, err, s);
-    else num_window_typed<float>(r, rows, count, token, hl, sl, wc, ar, out, err, s);
+    if (dtype) num_window_typed<double>(r, rows, count, entries, products, token, hl, sl, wc, ar, out, err, s);
+    else num_window_typed<float>(r, rows, count, entries, products, token, hl, sl, wc, ar, out, err, s);
 }
 
 // One warp per (row, window) item of the arena rows: the window's columns go

@@ -91,7 +91,8 @@ constexpr int kSpareWords = 32;   // after the bitmap: hold the bit past the las
 // gradient at 65,536 rows 1.39 ms, now 1.19. No test before the atomic: 3.83 ms.)
 template <int NT, typename IT>
 __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int *rows, int count, int *token,
-                                                  int words, WinCount wc, int *nnz_out, NumCheck nc, int *err) {
+                                                  int words, int apart_from, WinCount wc, int *nnz_out, NumCheck nc,
+                                                  int *err) {
     using G = Group<NT, NT>;
     constexpr int kWarps = NT / 32;
     constexpr int kSubWords = kSubCols / 32;
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int 
             a_row_range(op, i, ab, ae, err);
             // columns out of range share the bit past the last column: no
             // branch per product; the bits' words are read before any is set
-            block_walk<float, IT, false, kWarps>(op, ab, ae, wp, err, [&](auto &j, auto &, auto &, auto &act) {
+            block_walk<float, IT, false, kWarps>(op, ab, ae, wp, ae - ab >= apart_from, err, [&](auto &j, auto &, auto &, auto &act) {
                 constexpr int U = sizeof(act) / sizeof(act[0]);
                 unsigned at[U], bit[U], had[U];   // (bits set meanwhile are set again)
 #pragma unroll
@@ -316,7 +317,7 @@ int sym_dense_threads(const HashLaunch &hl, int64_t ncols) {
 }
 
 template <int NT>
-static void sym_dense_go(const Operands<float> &op, const int *rows, int count, int *token, int per_sm,
+static void sym_dense_go(const Operands<float> &op, const int *rows, int count, int apart_from, int *token, int per_sm,
                          const HashLaunch &hl, const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err,
                          cudaStream_t s) {
     const int words = (int)sym_dense_words(op.ncols);
@@ -324,18 +325,20 @@ static void sym_dense_go(const Operands<float> &op, const int *rows, int count, 
     auto kern = op.b_nnz < INT_MAX ? k_sym_dense<NT, int32_t> : k_sym_dense<NT, int64_t>;
     allow_smem((const void *)kern);
     const int grid = resident_grid(kern, NT, smem, hl.sms, count, per_sm);
-    kern<<<grid, NT, smem, s>>>(op, rows, count, token, words, wc, nnz_out, nc, err);
+    kern<<<grid, NT, smem, s>>>(op, rows, count, token, words, apart_from, wc, nnz_out, nc, err);
 }
 
-void launch_sym_dense(const RawOperands &r, const int *rows, int count, int *token, const HashLaunch &hl,
-                      const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err, cudaStream_t s) {
+void launch_sym_dense(const RawOperands &r, const int *rows, int count, long long entries, long long products,
+                      int *token, const HashLaunch &hl, const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err,
+                      cudaStream_t s) {
     if (count <= 0) return;
     const Operands<float> op = sym_operands(r);
     int nt, per_sm;
     sym_dense_shape(hl, r.ncols, nt, per_sm);
-    if (nt == 256) sym_dense_go<256>(op, rows, count, token, per_sm, hl, wc, nnz_out, nc, err, s);
-    else if (nt == 512) sym_dense_go<512>(op, rows, count, token, per_sm, hl, wc, nnz_out, nc, err, s);
-    else sym_dense_go<1024>(op, rows, count, token, per_sm, hl, wc, nnz_out, nc, err, s);
+    const int apart_from = walk_apart_from(entries, products, nt / 32);
+    if (nt == 256) sym_dense_go<256>(op, rows, count, apart_from, token, per_sm, hl, wc, nnz_out, nc, err, s);
+    else if (nt == 512) sym_dense_go<512>(op, rows, count, apart_from, token, per_sm, hl, wc, nnz_out, nc, err, s);
+    else sym_dense_go<1024>(op, rows, count, apart_from, token, per_sm, hl, wc, nnz_out, nc, err, s);
 }
 
 int sym_spill_grid(const HashLaunch &hl) {

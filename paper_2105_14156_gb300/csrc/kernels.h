@@ -160,8 +160,10 @@ void launch_sym_hash(const RawOperands &op, const int *rows, int count, int *tok
                      int *nnz_out, int *err, cudaStream_t s);
 // Dense rows: bitmap over all columns of B. Symbolic use: nnz_out != nullptr.
 // Numeric count pass: nnz_out == nullptr, sizes checked by nc.
-void launch_sym_dense(const RawOperands &op, const int *rows, int count, int *token, const HashLaunch &hl,
-                      const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err, cudaStream_t s);
+// entries, products: of the listed rows (entries of A).
+void launch_sym_dense(const RawOperands &op, const int *rows, int count, long long entries, long long products,
+                      int *token, const HashLaunch &hl, const WinCount &wc, int *nnz_out, const NumCheck &nc, int *err,
+                      cudaStream_t s);
 int sym_dense_threads(const HashLaunch &hl, int64_t ncols);   // block size launch_sym_dense picks
 int sym_spill_grid(const HashLaunch &hl);
 void launch_sym_spill(const RawOperands &op, const int *rows, int count, int *token, const HashLaunch &hl,
@@ -285,8 +287,9 @@ struct WinArena {
 };
 // (row, window) work items of the dense rows; counts from wc (or arena mode
 // when ar.ci != nullptr); token: a 64-bit item counter (zeroed here).
-void launch_num_window(int dtype, const RawOperands &op, const int *rows, int count, unsigned long long *token,
-                       const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
+// entries, products: of the listed rows (entries of A).
+void launch_num_window(int dtype, const RawOperands &op, const int *rows, int count, long long entries,
+                       long long products, unsigned long long *token, const HashLaunch &hl, const BSlices &sl, const WinCount &wc, const WinArena &ar,
                        const NumOut &out, int *err, cudaStream_t s);
 // Copies the arena rows (ovf[i] == 2) of the dense bin into C.
 void launch_arena_compact(int dtype, const int *rows, int count, int nw, const WinArena &ar, const uint8_t *ovf,

@@ -126,3 +126,31 @@ def test_dense_rows_counted_before_and_not(handle, kind):
                               exact=kind == "int")
     finally:
         handle.set_params(dense_ratio=4, sym_dense_ratio=64)
+
+
+@pytest.mark.parametrize("kind", ["f32", "f64", "int"])
+@pytest.mark.parametrize("per", [1, 3, 15, 17, 60, 130])
+def test_dense_rows_of_short_rows_of_b(handle, per, kind):
+    """Rows of B from one entry to more than a batch is worth: the warps of a block take whole batches of a row of A in
+    turn below 16 products an entry, and up to 128 the rows with a batch for a fourth of the warps or for each."""
+    from paper_2105_14156_gb300 import smash
+    cols, k, rng = 9001, 1200, np.random.default_rng(per)
+    lens = rng.integers(max(0, per - 2), per + 3, k)
+    r = np.repeat(np.arange(k), lens)
+    c = np.concatenate([rng.permutation(cols)[:n] for n in lens])
+    rp, ci = csr_from_coo(k, cols, r, c)
+    B = Csr(k, cols, rp, ci, values_of(rng, kind, ci.size))
+    a_lens = [1, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1024, 1025, k]
+    r = np.repeat(np.arange(len(a_lens)), a_lens)
+    c = np.concatenate([rng.permutation(k)[:n] for n in a_lens])
+    rp, ci = csr_from_coo(len(a_lens), k, r, c)
+    A = Csr(len(a_lens), k, rp, ci, values_of(rng, kind, ci.size))
+    handle.set_params(dense_ratio=1 << 20, sym_dense_ratio=1 << 20)
+    try:
+        dA, dB = smash.to_device(A), smash.to_device(B)
+        assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=kind == "int")
+        C, _, owner = handle.spgemm_learned(dA, dB, None)
+        assert_matches_oracle(C.to_host(), A, B, exact=kind == "int")
+        owner.free()
+    finally:
+        handle.set_params(dense_ratio=4, sym_dense_ratio=64)
