@@ -516,7 +516,7 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
     // both spill launches (when there are two) share the tables: one stream
     cudaStream_t spill_stream = nullptr;
     int order[kNumBins];
-    const int nb = bin_order(sums, order);
+    const int nb = bin_order(sums, order, narrow && !narrow_few(counts[bd], h->sms));
     Fork fk(h, s, bins_used(counts));
     int q = 0;
     for (int x = 0; x < nb; ++x) {
@@ -526,9 +526,9 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
         int *tok = pl.bb.tokens + b;
         if (b == kBinDense && narrow) {
             cudaStream_t bs = fk.get(q++);
-            LaunchTimer lt(h, bs, "num_narrow", b, 256, counts[b], sums[b], sums[16 + b], sums[32 + b], 2);
-            launch_narrow_num(dt, op, rows, counts[b], sums[b], sums[16 + b], tok, h->sms, (long long *)h->split.ptr,
-                              out, err, bs);
+            LaunchTimer lt(h, bs, "num_narrow", b, 256, counts[b], sums[b], sums[16 + b], sums[32 + b], 0);
+            lt.add_kernels(launch_narrow_num(dt, op, rows, counts[b], sums[b], sums[16 + b], tok, h->sms,
+                                             (long long *)h->split.ptr, out, err, bs));
         } else if (b == kBinDense && windows) {
             cudaStream_t bs = fk.get(q++);
             // (row, window) items

@@ -261,14 +261,17 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
         d.ncols = (int32_t)B[m].cols;
         d.mode = -1;
         if (B[m].cols * (int64_t)vsz <= kDenseWarpBytes) {
-            d.mode = dense_mode(B[m].nnz, B[m].rows, d.ncols, (int)vsz);
+            // plain adds need a pass over B, which fewer products than B has entries
+            // (estimated: nnz(A) times B's mean row) don't pay for
+            d.mode = A[m].nnz < B[m].rows ? kDenseFlat
+                                              : dense_mode(B[m].nnz, B[m].rows, d.ncols, (int)vsz, nrows <= h->sms * kBW);
             const size_t bytes = dense_warp_bytes(d.mode, d.ncols, (int)vsz);
             if (bytes > dense_bytes) dense_bytes = bytes;
         } else {
             wide = true;
         }
         d.seg_off = nseg;
-        if (d.mode >= 0)
+        if (d.mode > kDenseFlat)
             nseg += (B[m].nnz + kSegEntries - 1) / kSegEntries + (B[m].rows + kSegRows - 1) / kSegRows;
         d.row_off = ro;
         hrs[m] = ro;

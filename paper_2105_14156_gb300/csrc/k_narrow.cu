@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kNarrowNT) k_narrow_num(Operands<V> op, const 
     const int w = threadIdx.x >> 5;
     V *all = (V *)smem;
     V *acc = all + (size_t)w * warp_words;
-    const bool ascend = *descents == 0;
+    const bool ascend = *descents == 0;   // (flat adds: of no account)
     dense_clear(acc, warp_words);
     __syncwarp();
     narrow_heavy(op.a_rp, op.a_nnz, rows, count, sh.heavy, [&](int i) {
@@ -277,6 +277,7 @@ static int narrow_grid(K kernel, size_t smem, int sms, int count, long long entr
 }
 
 bool narrow_symbolic(int64_t ncols) { return ncols <= kNarrowSymCols; }
+bool narrow_few(int64_t rows, int sms) { return rows <= (int64_t)sms * kNarrowWarps; }
 bool narrow_numeric(int dtype, int64_t ncols) { return ncols * (dtype ? 8 : 4) <= kDenseWarpBytes; }
 
 void launch_narrow_count(const RawOperands &r, const int *rows, int count, long long entries, long long products,
@@ -288,35 +289,39 @@ void launch_narrow_count(const RawOperands &r, const int *rows, int count, long 
     NarrowShare sh;
     const int grid = narrow_grid(k_narrow_count, smem, sms, count, entries, words, sh);
     // (no accumulator copies to fit: the lane group by the mean row length alone)
-    const int mode = dense_mode(products, entries, 32, 4);
+    const int mode = dense_mode(products, entries, 32, 4, true);
     k_narrow_count<<<grid, kNarrowNT, smem, s>>>(narrow_operands<float>(r), rows, count, token,
                                                  mode == kDenseFlat ? kDenseW8 : mode, words, sh, nnz_out, err);
 }
 
 template <typename V>
-static void narrow_num_typed(const RawOperands &r, const int *rows, int count, long long entries, long long products,
-                         int *token, int sms,
-                             const long long *descents, const NumOut &o, int *err, cudaStream_t s) {
+static int narrow_num_typed(const RawOperands &r, const int *rows, int count, long long entries, long long products,
+                            int *token, int sms, long long *descents, const NumOut &o, int *err, cudaStream_t s) {
     const NumOutT<V> out{o.c_rp, o.c_ci, (V *)o.c_val, o.c_nnz, o.row_nnz};
-    const int mode = dense_mode(products, entries, r.ncols, sizeof(V));
+    // plain adds need a pass over B, which fewer products than B has entries don't pay for
+    const bool few = narrow_few(count, sms);
+    const int mode = products < r.b_nnz ? kDenseFlat : dense_mode(products, entries, r.ncols, sizeof(V), few);
+    if (mode != kDenseFlat) {
+        cudaMemsetAsync(descents, 0, sizeof(long long), s);
+        const int64_t segs = r.b_nnz / 8192 + r.b_rows / 2048 + 2;
+        k_descents<<<(int)(segs < 8ll * sms ? segs : 8ll * sms), 256, 0, s>>>(r.b_rp, r.b_ci, r.b_rows, r.b_nnz,
+                                                                            r.ncols, descents);
+    }
     const size_t warp_bytes = dense_warp_bytes(mode, r.ncols, sizeof(V));
     const size_t smem = kNarrowWarps * warp_bytes;
     NarrowShare sh;
     const int grid = narrow_grid(k_narrow_num<V>, smem, sms, count, entries, (int)(warp_bytes / sizeof(V)), sh);
     k_narrow_num<V><<<grid, kNarrowNT, smem, s>>>(narrow_operands<V>(r), rows, count, token, mode,
                                                   (int)(warp_bytes / sizeof(V)), sh, descents, out, err);
+    return mode != kDenseFlat ? 2 : 1;
 }
 
-void launch_narrow_num(int dtype, const RawOperands &r, const int *rows, int count, long long entries, long long products,
-                         int *token,
-                       int sms, long long *descents, const NumOut &out, int *err, cudaStream_t s) {
-    if (count <= 0) return;
-    cudaMemsetAsync(descents, 0, sizeof(long long), s);
-    const int64_t segs = r.b_nnz / 8192 + r.b_rows / 2048 + 2;
-    k_descents<<<(int)(segs < 8ll * sms ? segs : 8ll * sms), 256, 0, s>>>(r.b_rp, r.b_ci, r.b_rows, r.b_nnz, r.ncols,
-                                                                        descents);
-    if (dtype) narrow_num_typed<double>(r, rows, count, entries, products, token, sms, descents, out, err, s);
-    else narrow_num_typed<float>(r, rows, count, entries, products, token, sms, descents, out, err, s);
+int launch_narrow_num(int dtype, const RawOperands &r, const int *rows, int count, long long entries,
+                      long long products, int *token, int sms, long long *descents, const NumOut &out, int *err,
+                      cudaStream_t s) {
+    if (count <= 0) return 0;
+    if (dtype) return narrow_num_typed<double>(r, rows, count, entries, products, token, sms, descents, out, err, s);
+    return narrow_num_typed<float>(r, rows, count, entries, products, token, sms, descents, out, err, s);
 }
 
 }  // namespace smash

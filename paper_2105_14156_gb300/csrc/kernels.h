@@ -241,12 +241,14 @@ void launch_num_tiny(int dtype, const RawOperands &op, const int *rows, int coun
 constexpr int kNarrowSymCols = 3072;
 bool narrow_symbolic(int64_t ncols);
 bool narrow_numeric(int dtype, int64_t ncols);
+bool narrow_few(int64_t rows, int sms);   // one block an SM has a warp for every row
 // entries, products: of the listed rows (entries of A).
 void launch_narrow_count(const RawOperands &op, const int *rows, int count, long long entries, long long products,
                          int *token, int sms, int *nnz_out, int *err, cudaStream_t s);
-// descents: device scratch of one long long.
-void launch_narrow_num(int dtype, const RawOperands &op, const int *rows, int count, long long entries,
-                       long long products, int *token, int sms, long long *descents, const NumOut &out, int *err, cudaStream_t s);
+// descents: device scratch of one long long. Returns the number of kernels launched.
+int launch_narrow_num(int dtype, const RawOperands &op, const int *rows, int count, long long entries,
+                      long long products, int *token, int sms, long long *descents, const NumOut &out, int *err,
+                      cudaStream_t s);
 // Column windows of the dense rows (k_split.cu): slices of B regrouped by
 // window of cpc columns; woff[B.rows][nslices+1] (nslices > 1 only).
 struct BSlices {

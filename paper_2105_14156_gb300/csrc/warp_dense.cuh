@@ -31,23 +31,38 @@
 
 namespace smash {
 
-// Lane groups by B's mean row length: the narrowest group that holds most
-// rows in one step keeps the most lanes busy; below 3 entries a row even eight
-// lanes would mostly idle, and 32 products of many rows share a step instead
-// (kDenseFlat, atomic adds). Copies that would not fit the accumulator's room
-// take wider groups.
+// How a warp adds a row's products (mode). W lanes to a row of B with an
+// accumulator copy per lane group: W by B's mean row length, the narrowest group
+// that holds most rows in one step. Copies are cleared, added up and scanned with
+// every row, and shared memory for them leaves fewer blocks resident, so they may
+// take kDenseCopyBytes together; wider accumulators have one copy and take 32
+// lanes a row of B from a mean of more than 16 entries on. Everything else adds
+// atomically (kDenseFlat: 32 products of any rows of B a step), and so does double,
+// where plain adds were nowhere faster.
+// (Values of 40,000 rows times 1,024 columns in float, rows of A x rows of B: 18 x 4
+// entries two copies 169 us, one with 32 lanes a row 134, flat 125; 25 x 12: 185, 144,
+// 143; 59 x 20: 32 lanes 106, flat 116. Double, 512 columns, 74 x 4: 458, 433, 162.
+// 256 columns in float, skewed graph of 50,021 rows: two copies 146 us, flat 170.)
+// With rows for no more warps than one block an SM has, residency is no matter: the
+// copies may take all of an accumulator's room (square of a skewed graph of 1,024
+// rows, whose crowded columns make atomic adds wait: 79 us, flat 84).
 enum : int { kDenseFlat = 0, kDenseW8 = 1, kDenseW16 = 2, kDenseW32 = 3 };
 __host__ __device__ constexpr int dense_copies(int mode) { return mode == kDenseW8 ? 4 : mode == kDenseW16 ? 2 : 1; }
 // Words of one accumulator copy.
 __host__ __device__ constexpr int dense_stride(int ncols) { return (ncols + 31) & ~31; }
-// Most bytes a warp's accumulator may take (eight warps of a block: 192 KB).
+// Most bytes a warp's accumulator may take (eight warps of a block: 192 KB), and
+// most that several copies may take.
 constexpr int kDenseWarpBytes = 24 * 1024;
+constexpr int kDenseCopyBytes = 2 * 1024;
 
-// entries: of `rows` rows of B (all, or each as often as a product reads it).
-__host__ __device__ inline int dense_mode(int64_t entries, int64_t rows, int ncols, int vsz) {
-    int m = entries < 3 * rows ? kDenseFlat : entries <= 8 * rows ? kDenseW8 : entries <= 16 * rows ? kDenseW16
-                                                                                                      : kDenseW32;
-    while (dense_copies(m) > 1 && (int64_t)dense_copies(m) * dense_stride(ncols) * vsz > kDenseWarpBytes) ++m;
+// entries: of `rows` rows of B (all, or each as often as a product reads it). few:
+// one block an SM has a warp for every row of the product.
+__host__ __device__ inline int dense_mode(int64_t entries, int64_t rows, int ncols, int vsz, bool few) {
+    if (vsz == 8 || entries < 3 * rows) return kDenseFlat;
+    int m = entries <= 8 * rows ? kDenseW8 : entries <= 16 * rows ? kDenseW16 : kDenseW32;
+    const int64_t copy = (int64_t)dense_stride(ncols) * vsz;
+    if (!few) return dense_copies(m) == 1 || dense_copies(m) * copy <= kDenseCopyBytes ? m : kDenseFlat;
+    while (dense_copies(m) > 1 && dense_copies(m) * copy > kDenseWarpBytes) ++m;
     return m;
 }
 __host__ __device__ inline size_t dense_warp_bytes(int mode, int ncols, int vsz) {
@@ -185,7 +200,7 @@ template <typename V>
 __device__ __forceinline__ void dense_accumulate(const Operands<V> &op, int mode, bool ascend, int64_t first,
                                                  int64_t ae, int64_t step, V *acc, int *err) {
     const int stride = dense_stride(op.ncols);
-    if (!ascend) mode = kDenseFlat;
+    if (!ascend || sizeof(V) == 8) mode = kDenseFlat;
     // (the barrier orders a step before the next one's loads of the same words)
     auto add = [&](int group, bool act, int j, V a, V b) {
         if (act) acc[group * stride + j] += dense_product(a, b);

@@ -215,3 +215,20 @@ def test_narrow_phases_of_long_rows_alike(handle, values):
         A = rows_of([147 + 3 * (q % 5) for q in range(rows)], 400, values, 6)
         dA, dB = smash.to_device(A), smash.to_device(B)
         assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=values == "int")
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+@pytest.mark.parametrize("cols", [64, 129, 256, 257, 2048])
+@pytest.mark.parametrize("rows", [3, 4, 400])
+def test_narrow_products_few_and_many(handle, rows, cols, values):
+    """Fewer products than B has entries (added atomically) and more (with lane groups where copies fit)."""
+    from paper_2105_14156_gb300 import smash
+    pairs = []
+    for q, per in enumerate((2, 6, 12, 40)):
+        B = b_matrix(cols, [per, per + 1], 600, values, 7 + q)
+        A = rows_of([150] * rows, 600, values, 8 + q)   # 600 entries of A and up: as many as B has rows
+        pairs.append((A, B))
+        C = handle.spgemm(smash.to_device(A), smash.to_device(B), check=True).to_host()
+        assert_matches_oracle(C, A, B, exact=values == "int")
+    for (A, B), C in zip(pairs, run_batch(handle, pairs)):
+        assert_matches_oracle(C, A, B, exact=values == "int")
