@@ -60,18 +60,20 @@ constexpr int kWalkAlone = 48;
 // (apart) instead of a part of each. entries, products: of the rows of a launch
 // (entries once for each window); warps: of a block. Every warp loads and scans
 // each batch that it has a part of, which costs more than walking the part where
-// the rows of B are short: every row below kWalkShort products an entry, the rows
-// with a batch for every fourth warp below kWalkShort * 2, with one for every warp
-// below kWalkMedium.
+// the rows of B are short: every row below 6 products an entry, the rows with three
+// batches below kWalkShort, with one for every fourth warp below kWalkShort * 2, with
+// one for every warp below kWalkMedium.
 // (Values of 800 dense rows of 100,000 columns, 13,750 entries of 8 products, in
 // parts and apart: float 6.21 and 1.13 ms, double 12.3 and 1.27 ms; 5,500 of 20: 2.65
 // and 0.68, 5.18 and 0.84 ms. Counts of rows of 1,100 entries of 8: 154 and 110 us; of
-// 59 entries of 50 products 121 us in parts, 145 us apart. The skewed float64 square
+// 59 entries of 50 products 121 us in parts, 145 us apart; values of 25,510 rows of 49
+// entries of 12, 1,024 columns: 350 and 391 us. The skewed float64 square
 // of 65,536 rows: 5.49 ms in parts, 5.52 so, 5.84 with a batch for every fourth
 // warp below kWalkMedium, 9.6 with every row apart.)
 constexpr int kWalkShort = 16, kWalkMedium = 128;
 inline int walk_apart_from(long long entries, long long products, int warps) {
-    if (products < kWalkShort * entries) return 0;
+    if (products < 6 * entries) return 0;
+    if (products < kWalkShort * entries) return 96;
     if (products < kWalkShort * 2 * entries) return 8 * warps > 128 ? 8 * warps : 128;
     return products < kWalkMedium * entries ? 32 * warps : INT_MAX;
 }
