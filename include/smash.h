@@ -77,9 +77,10 @@ typedef struct {
     int32_t num_max_tbits;  /* largest shared-memory numeric table, log2 slots; [5, 14]; default 14 */
     int32_t group_shift;    /* threads per row = clamp(T >> group_shift, 32, 1024); [0, 10]; default 4 */
     int32_t dense_ratio;    /* a row whose bound b satisfies b * dense_ratio >= cols(B) uses the dense
-                               accumulator (the paper's "dense row"), four times as short a row when a warp
-                               owns all columns (B of at most 6144 columns in float, 3072 in double, with
-                               dense_blocks and dense_owner at 0); 0 disables; default 4 */
+                               accumulator (the paper's "dense row"); with dense_blocks and dense_owner at 0,
+                               where a warp may own all columns, rows four times as short (B of at most
+                               1536 columns in float, 1024 in double) or twice as short (3072, 1536) do;
+                               0 disables; default 4 */
     int32_t bitmap_ratio;   /* numeric write-out ranks by a column bitmap when cols(B)/32 <=
                                bitmap_ratio * nnz(row); 0 disables; default 4 */
     int32_t spill_blocks_per_sm; /* resident blocks per SM of the spill and dense kernels; default 1 */

@@ -460,7 +460,7 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
     // counts and the slices of B are prepared on s before the bins fork.
     const int bd = kBinDense;
     int cpc = 0, nw = 0, per = 1;
-    const bool narrow = counts[bd] && use_narrow_num(h, op.ncols, dt);
+    const bool narrow = use_narrow_num(h, op.ncols, dt, counts[bd], sums[bd], sums[16 + bd]);
     const bool windows = counts[bd] && !narrow && dense_windows(h, op, dt, sums[16 + bd], cpc, nw, per);
     if (narrow && (st = ensure(h, h->split, 256, s))) return st;
     HashLaunch hld = hash_launch(h, 0, op.ncols);

@@ -598,8 +598,11 @@ inline bool tiny_first(const smash_handle *h, const BinRule &r, int bin, int cou
 inline bool use_narrow_sym(const smash_handle *h, int64_t ncols) {
     return h->params.sym_dense_blocks == 0 && narrow_symbolic(ncols);
 }
-inline bool use_narrow_num(const smash_handle *h, int64_t ncols, int dtype) {
-    return h->params.dense_blocks == 0 && !h->params.dense_owner && narrow_numeric(dtype, ncols);
+inline bool narrow_asked(const smash_handle *h) { return h->params.dense_blocks == 0 && !h->params.dense_owner; }
+// rows, entries, products: of the phase's dense rows (entries of A).
+inline bool use_narrow_num(const smash_handle *h, int64_t ncols, int dtype, long long rows, long long entries,
+                           long long products) {
+    return rows > 0 && narrow_asked(h) && narrow_numeric(dtype, ncols, rows, entries, products, h->sms);
 }
 
 inline BinRule sym_rule(const smash_handle *h, int64_t ncols) {
@@ -623,9 +626,9 @@ inline BinRule num_rule(const smash_handle *h, int64_t ncols, int dtype) {
     // column window that fits shared memory
     const bool dense_fits = ncols <= dense_bitmap_max_cols() && num_window_cols(dtype, dense_blocks_of(h, dtype), false) > 0;
     r.dense_ok = (h->params.dense_ratio > 0 && dense_fits) ? 1 : 0;
-    // (a warp that owns all columns clears and scans them for about a quarter
-    // of what a block's window costs, so it takes rows four times as short)
-    const int64_t ratio = (int64_t)h->params.dense_ratio * (use_narrow_num(h, ncols, dtype) ? 4 : 1);
+    // (a warp that owns all columns clears and scans them for less than a block's
+    // window costs, so it takes shorter rows)
+    const int64_t ratio = (int64_t)h->params.dense_ratio * (narrow_asked(h) ? narrow_ratio(dtype, ncols) : 1);
     r.dense_min = r.dense_ok ? (ncols + ratio - 1) / ratio : (1ll << 62);
     if (r.dense_min < 1) r.dense_min = 1;
     int mt = h->params.num_max_tbits;

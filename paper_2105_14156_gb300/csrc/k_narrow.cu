@@ -278,7 +278,37 @@ static int narrow_grid(K kernel, size_t smem, int sms, int count, long long entr
 
 bool narrow_symbolic(int64_t ncols) { return ncols <= kNarrowSymCols; }
 bool narrow_few(int64_t rows, int sms) { return rows <= (int64_t)sms * kNarrowWarps; }
-bool narrow_numeric(int dtype, int64_t ncols) { return ncols * (dtype ? 8 : 4) <= kDenseWarpBytes; }
+
+// Which numeric rows a warp's accumulator serves, by the bytes of one. An
+// accumulator is cleared and scanned for every row, and 8 of them decide how many
+// blocks are resident; the alternatives are a table (rows below a quarter of the
+// columns) and column windows with a block a row.
+//   Up to 6 KB in float, 8 KB in double: every dense row, down to a sixteenth of the
+// columns (us, accumulator and alternative, rows of a sixteenth / a quarter / all of
+// the columns: float 1,024 columns 108 and 131 / 134 and 371 / 113 and 235, double 129
+// and 137 / 164 and 587 / 148 and 414).
+//   Up to 12 KB: from an eighth on (double 1,536 columns, a sixteenth 169 and 169, an
+// eighth 211 and 245, a quarter 225 and 594; float 2,048 columns 176 and 174, 195 and
+// 261, 170 and 320), where there is a row for more than one block's warps an SM and the
+// rows' products are at most twice the columns (2,048-row skewed square, 300 rows:
+// 145 and 120; 3,000 columns, products four times as many: 275 and 182).
+//   Up to 24 KB in double: from a quarter on, where an entry of A has 8 products or more
+// besides (2,048 columns, 49 entries of 12 products 347 and 493, 294 of 2 599 and 460).
+// In float windows are better beyond 12 KB (4,000 columns, a quarter 310 and 270).
+constexpr int narrow_short_bytes(int dtype) { return dtype ? 8 * 1024 : 6 * 1024; }
+constexpr int kNarrowMediumBytes = 12 * 1024;
+
+int narrow_ratio(int dtype, int64_t ncols) {
+    const int64_t bytes = ncols * (dtype ? 8 : 4);
+    return bytes <= narrow_short_bytes(dtype) ? 4 : bytes <= kNarrowMediumBytes ? 2 : 1;
+}
+bool narrow_numeric(int dtype, int64_t ncols, long long rows, long long entries, long long products, int sms) {
+    const int64_t bytes = ncols * (dtype ? 8 : 4);
+    if (bytes <= narrow_short_bytes(dtype)) return true;
+    if (bytes > (dtype ? kDenseWarpBytes : kNarrowMediumBytes)) return false;
+    if (narrow_few(rows, sms) || products > 2 * ncols * rows) return false;
+    return bytes <= kNarrowMediumBytes || products >= 8 * entries;
+}
 
 void launch_narrow_count(const RawOperands &r, const int *rows, int count, long long entries, long long products,
                          int *token, int sms,

@@ -235,12 +235,14 @@ void launch_sym_tiny(const RawOperands &op, const int *rows, int count, int tbit
 void launch_num_tiny(int dtype, const RawOperands &op, const int *rows, int count, int tbits, float max_load,
                      int sms, const NumOut &out, int *err, cudaStream_t s);
 // Narrow B (k_narrow.cu): dense rows whose columns one warp owns. Whether B's
-// columns fit a warp's flags / accumulator; the symbolic limit is the double
-// accumulator's, so that a phase pair never mixes a narrow symbolic phase with
-// column windows that would have to count their columns again.
+// columns fit a warp's flags, and whether its accumulator is the better choice for
+// these rows. (A narrow symbolic phase leaves no counts for column windows: they
+// count the rows again, which the lines in narrow_numeric() allow for.)
 constexpr int kNarrowSymCols = 3072;
 bool narrow_symbolic(int64_t ncols);
-bool narrow_numeric(int dtype, int64_t ncols);
+bool narrow_numeric(int dtype, int64_t ncols, long long rows, long long entries, long long products,
+                    int sms);
+int narrow_ratio(int dtype, int64_t ncols);   // how much shorter the rows that it may take than a window's
 bool narrow_few(int64_t rows, int sms);   // one block an SM has a warp for every row
 // entries, products: of the listed rows (entries of A).
 void launch_narrow_count(const RawOperands &op, const int *rows, int count, long long entries, long long products,

@@ -490,7 +490,8 @@ int spgemm_learned(smash_handle *h, const smash_csr *A, const smash_csr *B, smas
     const int nd = bp.counts[kBinDense];
     const int *drows = pl.bb.rows + bp.offsets[kBinDense];   // valid until the next plan_buffers()
     int cpc = 0, nw = 0, per = 1;
-    const bool use_arena = nd > 0 && !use_narrow_num(h, op.ncols, dt) &&
+    const bool use_arena = nd > 0 &&
+                           !use_narrow_num(h, op.ncols, dt, nd, bp.sums[kBinDense], bp.sums[16 + kBinDense]) &&
                            dense_windows(h, op, dt, bp.sums[16 + kBinDense], cpc, nw, per);
     WinArena ar;
     const int *arena_rows = nullptr;

@@ -232,3 +232,19 @@ def test_narrow_products_few_and_many(handle, rows, cols, values):
         assert_matches_oracle(C, A, B, exact=values == "int")
     for (A, B), C in zip(pairs, run_batch(handle, pairs)):
         assert_matches_oracle(C, A, B, exact=values == "int")
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+@pytest.mark.parametrize("cols", [1024, 1025, 1536, 1537, 3072, 3073])
+@pytest.mark.parametrize("per,entries", [(12, 60), (3, 240), (40, 250)])
+def test_narrow_rows_or_windows(handle, cols, per, entries, values):
+    """Columns around the sizes where a warp's accumulator gives way to tables and windows, with 3 and with 12 products
+    an entry, about half the columns or more than twice as many (the widest: as many) products a row."""
+    from paper_2105_14156_gb300 import smash
+    B = b_matrix(cols, [per], 400, values, 3)
+    A = rows_of([entries, max(1, entries // 3), max(1, entries // 9)] * 30, 400, values, 4)
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    assert_matches_oracle(handle.spgemm(dA, dB, check=True).to_host(), A, B, exact=values == "int")
+    C, _, owner = handle.spgemm_learned(dA, dB, None)
+    assert_matches_oracle(C.to_host(), A, B, exact=values == "int")
+    owner.free()
