@@ -371,8 +371,9 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
                    smash_csr *C, smash_batched_stats *stats, void *stream);
 
 /* Per-warp hash-table size of the batched kernel, 2^bits slots, bits in [6, 12] (default 10).
- * (Products whose B is narrow enough for a warp to own every column, at most
- * 24 KB of values, use dense accumulators instead, whatever the size.) */
+ * (Products whose B is narrow enough for a warp to own every column, some 8 KB of
+ * values in float and 14 in double, and up to 24 KB where their rows are full enough,
+ * use dense accumulators instead, whatever the size.) */
 int smash_batched_set_table_bits(smash_handle *h, int bits);
 int smash_batched_get_table_bits(smash_handle *h, int *bits);
 

@@ -17,6 +17,7 @@ enum : uint8_t { kRowEmpty = 0, kRowSmall = 1, kRowBig = 2, kRowHuge = 3, kRowMe
 // once), up to kBigFlop by a warp that claims it alone, above by a block.
 constexpr int kMedFlop = 512;
 constexpr int kBigFlop = 8192;
+constexpr int kBatchLongRow = 512;   // products above which a row outgrows the default warp table
 constexpr int kSegEntries = 8192;
 constexpr int kSegRows = 2048;
 
@@ -52,7 +53,8 @@ struct BatchArgs {
     int *longs;             // [nrows] list of rows counted by a warp (k_batch_rowinfo_long)
     int *counters;          // [16]: 0 nbig, 1 nhuge, 2..3 item tokens, 4 med token, 5 matrix token, 6..7 barrier,
                             // 8..9 row-chunk tokens of the two row phases, 12 nmed, 13 nlong
-    unsigned long long *sums;   // [4]: sum ub, sum flop
+    unsigned long long *sums;   // [4]: sum ub, sum flop, flop of long rows (kBatchLongRow) of products with a large accumulator
+    int large_cols;             // columns above which an accumulator is large
     long long *descents;    // [nmat] 0: every row of B ascends (warp_dense.cuh)
     int64_t nseg;           // segments of all products
     int chunk;              // rows a warp claims at once (1 .. 32)

@@ -1,6 +1,7 @@
 // C ABI of the batched path: many C_m = A_m * B_m in one persistent launch,
 // plus the autotuner of its table size.
 #include <algorithm>
+#include <cstdint>
 #include <cstdio>
 #include <map>
 
@@ -114,6 +115,58 @@ struct Layout {
     long long *descents;
     int64_t *base, *totals;
 };
+
+// Whether the products of a batch with a large accumulator (more than large_cols columns,
+// at most kDenseWarpBytes) use accumulators or hash tables. All or none, as the widest
+// accumulator's bytes are every block's shared memory. Products are estimated at nnz(A)
+// times B's mean row.
+//   Smaller accumulators, some 8 KB in float and 14 KB in double, are always taken: a
+// default table has 8 and 12 KB, so no more blocks would be resident with tables (double,
+// 1,700 columns, a 64th of them products a row: 498 and 581 us; float, 2,500 columns, one
+// entry by one: 328 and 224).
+//   Below a quarter of the batch's products: tables. (255 products of 256 columns with
+// 1, 16 and 32 of 5,000, 1,024 products a row, 2, 25 and 40 % of all; us, accumulators
+// and tables, float: 2,432 and 1,245, 2,843 and 2,719, 3,254 and 4,242.)
+//   A row clears and scans its columns whatever it holds. From a kDenseFill-th of the
+// columns products a row on: accumulators. (64 products of 1,500 rows, 4,000 columns,
+// float: 16 x 16 entries 2,050 and 1,791, 21 x 16 2,203 and 2,337.)
+//   Down to an eighth of that by the rows, which k_batch_rowinfo looks at: accumulators
+// where rows that outgrow a warp's table hold a quarter of the products, as the graphs'
+// heavy rows do (100 skewed graphs, 3,000 columns, a seventeenth: 464 and 836; 24,
+// 5,000 columns, a thirtieth: 321 and 1,296), else tables (4,000 columns, a 32nd in every
+// row: 1,685 and 968). Below: tables (5,000 columns, one entry by one: 710 and 236).
+constexpr int kDenseFill = 16;
+enum class Large { kTables, kAccumulators, kByRows };
+
+int large_cols(int vsz) { return vsz == 8 ? 1792 : 2048; }
+bool is_large(const smash_csr &B, int vsz) {
+    return B.cols > large_cols(vsz) && B.cols * vsz <= kDenseWarpBytes;
+}
+double products_of(const smash_csr &A, const smash_csr &B) {
+    return B.rows > 0 ? (double)A.nnz * (double)B.nnz / (double)B.rows : 0.0;
+}
+
+Large large_products(int count, const smash_csr *A, const smash_csr *B, int vsz) {
+    double all = 0, large = 0, cols = 0;
+    for (int m = 0; m < count; ++m) {
+        const double f = products_of(A[m], B[m]);
+        all += f;
+        if (!is_large(B[m], vsz)) continue;
+        large += f;
+        cols += (double)B[m].cols * (double)A[m].rows;
+    }
+    if (large * 4 < all || large * kDenseFill * 8 < cols) return Large::kTables;
+    return large * kDenseFill >= cols ? Large::kAccumulators : Large::kByRows;
+}
+
+// The accumulator of a product's rows: a mode of warp_dense.cuh, or -1 (hash tables).
+// few: one block an SM has a warp for every row of the batch. (Plain adds need a pass
+// over B, which fewer products than its entries don't pay for.)
+int product_mode(const smash_csr &A, const smash_csr &B, int vsz, bool large, bool few) {
+    if (B.cols > large_cols(vsz) && !(large && is_large(B, vsz))) return -1;
+    if (products_of(A, B) < (double)B.nnz) return kDenseFlat;
+    return dense_mode(B.nnz, B.rows, (int)B.cols, vsz, few);
+}
 
 }  // namespace
 
@@ -240,93 +293,99 @@ int spgemm_batched(smash_handle *h, int count, const smash_csr *A, const smash_c
     cudaStreamSynchronize(s);   // the pinned staging may still feed a previous copy
     BatchMat *hm = (BatchMat *)bs.pinned;
     int64_t *hrs = (int64_t *)((char *)bs.pinned + ((char *)L.row_start - (char *)L.mats));
-    int64_t ro = 0;
-    // a product whose B fits a warp's dense accumulator is narrow, the others
-    // are wide: their rows take hash tables
+    // a product whose rows a warp's dense accumulator serves is narrow, the
+    // others are wide: their rows take hash tables
+    Large large = large_products(count, A, B, (int)vsz);
+    const bool few = nrows <= (int64_t)h->sms * kBW;
     bool wide = false;
-    size_t dense_bytes = 0;
-    int64_t nseg = 0;
-    for (int m = 0; m < count; ++m) {
-        BatchMat &d = hm[m];
-        d.a_rp = A[m].row_ptr;
-        d.a_ci = A[m].col_idx;
-        d.a_val = A[m].val;
-        d.b_rp = B[m].row_ptr;
-        d.b_ci = B[m].col_idx;
-        d.b_val = B[m].val;
-        d.a_nnz = A[m].nnz;
-        d.b_nnz = B[m].nnz;
-        d.a_rows = (int32_t)A[m].rows;
-        d.b_rows = (int32_t)B[m].rows;
-        d.ncols = (int32_t)B[m].cols;
-        d.mode = -1;
-        if (B[m].cols * (int64_t)vsz <= kDenseWarpBytes) {
-            // plain adds need a pass over B, which fewer products than B has entries
-            // (estimated: nnz(A) times B's mean row) don't pay for
-            d.mode = A[m].nnz < B[m].rows ? kDenseFlat
-                                              : dense_mode(B[m].nnz, B[m].rows, d.ncols, (int)vsz, nrows <= h->sms * kBW);
-            const size_t bytes = dense_warp_bytes(d.mode, d.ncols, (int)vsz);
-            if (bytes > dense_bytes) dense_bytes = bytes;
-        } else {
-            wide = true;
-        }
-        d.seg_off = nseg;
-        if (d.mode > kDenseFlat)
-            nseg += (B[m].nnz + kSegEntries - 1) / kSegEntries + (B[m].rows + kSegRows - 1) / kSegRows;
-        d.row_off = ro;
-        hrs[m] = ro;
-        ro += A[m].rows;
-    }
-    hrs[count] = ro;
-    size_t warp_bytes = wide ? batched_table_bytes(dt, bs.tw_bits) : 128;
-    if (dense_bytes > warp_bytes) warp_bytes = dense_bytes;
-    if (cudaMemcpyAsync(L.mats, hm, desc_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(L.counters, 0, ctr_bytes, s) != cudaSuccess)
-        return SMASH_ERR_CUDA;
     BatchArgs p;
-    memset(&p, 0, sizeof(p));
-    p.mats = L.mats;
-    p.nmat = count;
-    p.nrows = nrows;
-    p.row_start = L.row_start;
-    p.cls = L.cls;
-    p.ub = L.ub;
-    p.nnz = L.nnz;
-    p.big = L.big;
-    p.huge = L.huge;
-    p.med = L.med;
-    p.longs = L.longs;
-    p.counters = L.counters;
-    p.sums = L.sums;
-    p.descents = L.descents;
-    p.nseg = nseg;
-    p.base = L.base;
-    p.totals = L.totals;
-    p.err = (int *)h->err.ptr;
-    p.tw_bits = bs.tw_bits;
-    p.warp_bits = bs.tw_bits - bs.warp_less;
-    p.block_bits = bs.tw_bits + bs.block_more;
-    p.wait_spins = bs.wait_spins;
-    p.missing = bs.missing;
-    p.warp_bytes = (int)warp_bytes;
-    p.dense_words = (int)(dense_bytes / vsz);
-    p.hc = HashCfg{h->params.hash_kind, 0};
-    p.inv_load = 1.0f / h->params.max_load;
-    {
-        LaunchTimer lt(h, s, "batch_rowinfo", -1, 256, nrows, 0, 0, 0, 2);
-        launch_batch_rowinfo(p, h->sms, s);
-    }
-    if ((st = last_cuda_status())) return st;
-    // sizes for the pools
-    char *hb = (char *)h->host;
-    if (read_small(h, 0, L.counters, 80, s) || cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
     int nbig, nhuge, nmed;
-    unsigned long long sum_ub, sum_f;
-    memcpy(&nbig, hb, 4);
-    memcpy(&nhuge, hb + 4, 4);
-    memcpy(&nmed, hb + 48, 4);
-    memcpy(&sum_ub, hb + 64, 8);
-    memcpy(&sum_f, hb + 72, 8);
+    unsigned long long sum_ub, sum_f, sum_long;
+    for (;;) {
+        wide = false;
+        size_t dense_bytes = 0;
+        int64_t nseg = 0, ro = 0;
+        double large_f = 0;
+        for (int m = 0; m < count; ++m) {
+            BatchMat &d = hm[m];
+            d.a_rp = A[m].row_ptr;
+            d.a_ci = A[m].col_idx;
+            d.a_val = A[m].val;
+            d.b_rp = B[m].row_ptr;
+            d.b_ci = B[m].col_idx;
+            d.b_val = B[m].val;
+            d.a_nnz = A[m].nnz;
+            d.b_nnz = B[m].nnz;
+            d.a_rows = (int32_t)A[m].rows;
+            d.b_rows = (int32_t)B[m].rows;
+            d.ncols = (int32_t)B[m].cols;
+            d.mode = product_mode(A[m], B[m], (int)vsz, large != Large::kTables, few);
+            if (d.mode >= 0) {
+                const size_t bytes = dense_warp_bytes(d.mode, d.ncols, (int)vsz);
+                if (bytes > dense_bytes) dense_bytes = bytes;
+                if (is_large(B[m], (int)vsz)) large_f += products_of(A[m], B[m]);
+            } else {
+                wide = true;
+            }
+            d.seg_off = nseg;
+            if (d.mode > kDenseFlat)
+                nseg += (B[m].nnz + kSegEntries - 1) / kSegEntries + (B[m].rows + kSegRows - 1) / kSegRows;
+            d.row_off = ro;
+            hrs[m] = ro;
+            ro += A[m].rows;
+        }
+        hrs[count] = ro;
+        size_t warp_bytes = wide ? batched_table_bytes(dt, bs.tw_bits) : 128;
+        if (dense_bytes > warp_bytes) warp_bytes = dense_bytes;
+        if (cudaMemcpyAsync(L.mats, hm, desc_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+            cudaMemsetAsync(L.counters, 0, ctr_bytes, s) != cudaSuccess)
+            return SMASH_ERR_CUDA;
+        memset(&p, 0, sizeof(p));
+        p.mats = L.mats;
+        p.nmat = count;
+        p.nrows = nrows;
+        p.row_start = L.row_start;
+        p.cls = L.cls;
+        p.ub = L.ub;
+        p.nnz = L.nnz;
+        p.big = L.big;
+        p.huge = L.huge;
+        p.med = L.med;
+        p.longs = L.longs;
+        p.counters = L.counters;
+        p.sums = L.sums;
+        p.large_cols = large_cols((int)vsz);
+        p.descents = L.descents;
+        p.nseg = nseg;
+        p.base = L.base;
+        p.totals = L.totals;
+        p.err = (int *)h->err.ptr;
+        p.tw_bits = bs.tw_bits;
+        p.warp_bits = bs.tw_bits - bs.warp_less;
+        p.block_bits = bs.tw_bits + bs.block_more;
+        p.wait_spins = bs.wait_spins;
+        p.missing = bs.missing;
+        p.warp_bytes = (int)warp_bytes;
+        p.dense_words = (int)(dense_bytes / vsz);
+        p.hc = HashCfg{h->params.hash_kind, 0};
+        p.inv_load = 1.0f / h->params.max_load;
+        {
+            LaunchTimer lt(h, s, "batch_rowinfo", -1, 256, nrows, 0, 0, 0, 2);
+            launch_batch_rowinfo(p, h->sms, s);
+        }
+        if ((st = last_cuda_status())) return st;
+        // sizes for the pools
+        char *hb = (char *)h->host;
+        if (read_small(h, 0, L.counters, 88, s) || cudaStreamSynchronize(s) != cudaSuccess) return SMASH_ERR_CUDA;
+        memcpy(&nbig, hb, 4);
+        memcpy(&nhuge, hb + 4, 4);
+        memcpy(&nmed, hb + 48, 4);
+        memcpy(&sum_ub, hb + 64, 8);
+        memcpy(&sum_f, hb + 72, 8);
+        memcpy(&sum_long, hb + 80, 8);
+        if (large != Large::kByRows || (double)sum_long * 4 >= large_f) break;
+        large = Large::kTables;   // (the copy from the pinned descriptors is over)
+    }
     ls.big_rows = nbig;
     ls.huge_rows = nhuge;
     ls.flop = (int64_t)sum_f;

@@ -99,6 +99,11 @@ __device__ __forceinline__ long long batch_classify(const BatchArgs &p, const Ba
     return ub;
 }
 
+// f, if row and accumulator are such that it speaks for accumulators (batched_modes).
+__device__ __forceinline__ long long batch_long(const BatchArgs &p, const BatchMat &M, long long f) {
+    return M.mode >= 0 && M.ncols > p.large_cols && f > kBatchLongRow ? f : 0;
+}
+
 // The first row_blocks blocks count rows, the others pass over the narrow
 // products' B (whether its rows ascend).
 __global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p, int row_blocks) {
@@ -130,7 +135,7 @@ __global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p, int row_bloc
         return;
     }
     const int64_t threads = (int64_t)row_blocks * blockDim.x;
-    unsigned long long my_ub = 0, my_f = 0;
+    unsigned long long my_ub = 0, my_f = 0, my_long = 0;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < p.nrows; g += threads) {
         const int mi = find_mat(p.row_start, p.nmat, g);
         const BatchMat &M = p.mats[mi];
@@ -155,12 +160,15 @@ __global__ void __launch_bounds__(256) k_batch_rowinfo(BatchArgs p, int row_bloc
         }
         my_ub += (unsigned long long)batch_classify(p, M, g, f);
         my_f += (unsigned long long)f;
+        my_long += (unsigned long long)batch_long(p, M, f);
     }
     my_ub = warp_sum(my_ub);
     my_f = warp_sum(my_f);
+    my_long = warp_sum(my_long);
     if (lane == 0) {
         atomicAdd(p.sums + 0, my_ub);
         atomicAdd(p.sums + 1, my_f);
+        if (my_long) atomicAdd(p.sums + 2, my_long);
     }
 }
 
@@ -168,7 +176,7 @@ __global__ void __launch_bounds__(256) k_batch_rowinfo_long(BatchArgs p) {
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int n = p.counters[13];
-    unsigned long long my_ub = 0, my_f = 0;
+    unsigned long long my_ub = 0, my_f = 0, my_long = 0;
     for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n; q += warps) {
         const int64_t g = p.longs[q];
         const int mi = find_mat(p.row_start, p.nmat, g);
@@ -189,11 +197,13 @@ __global__ void __launch_bounds__(256) k_batch_rowinfo_long(BatchArgs p) {
         if (lane == 0) {
             my_ub += (unsigned long long)batch_classify(p, M, g, f);
             my_f += (unsigned long long)f;
+            my_long += (unsigned long long)batch_long(p, M, f);
         }
     }
     if (lane == 0 && my_f) {
         atomicAdd(p.sums + 0, my_ub);
         atomicAdd(p.sums + 1, my_f);
+        if (my_long) atomicAdd(p.sums + 2, my_long);
     }
 }
 

@@ -248,3 +248,24 @@ def test_narrow_rows_or_windows(handle, cols, per, entries, values):
     C, _, owner = handle.spgemm_learned(dA, dB, None)
     assert_matches_oracle(C.to_host(), A, B, exact=values == "int")
     owner.free()
+
+
+@pytest.mark.parametrize("values", ["f32", "f64", "int"])
+@pytest.mark.parametrize("mix", ["sparse", "filled", "one wide", "half wide", "even", "skewed"])
+def test_batched_accumulators_or_tables(handle, mix, values):
+    """Wide-ish products whose rows are too empty for a warp's accumulator, or full enough; one of them among many
+    narrow ones, which keep their shared memory, or enough of them to be worth it; rows in between, all alike or a few
+    that outgrow a warp's table."""
+    cols = 2900 if values == "f64" else 5800   # below the widest accumulator, above the default table's bytes
+
+    def pair(n, a, c, b, seed):
+        lens = [a] * n if isinstance(a, int) else [a[q % len(a)] for q in range(n)]
+        return rows_of(lens, 60, values, seed), b_matrix(c, [b], 60, values, seed + 1)
+    empty, full = (100, 2, cols, 5), (100, 40, cols, 40)
+    small = [(80, 8, 256, 12)] * 12
+    sizes = {"sparse": [empty] * 6, "filled": [full] * 6, "one wide": small + [full[:1] + (3,) + full[2:]],
+             "half wide": small + [full] * 3, "even": [(100, 8, cols, 18)] * 6,
+             "skewed": [(100, (2, 2, 60, 2, 2), cols, 18)] * 6}[mix]
+    pairs = [pair(*s, 5 * q) for q, s in enumerate(sizes)]
+    for (A, B), C in zip(pairs, run_batch(handle, pairs)):
+        assert_matches_oracle(C, A, B, exact=values == "int")
