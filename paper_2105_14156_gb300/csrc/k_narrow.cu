@@ -112,14 +112,14 @@ __global__ void __launch_bounds__(kNarrowNT) k_narrow_count(Operands<float> op, 
         __syncthreads();
     });
     for (;;) {
-        int r0 = 0;
-        if (lane == 0) r0 = atomicAdd(token, sh.chunk);
+        unsigned r0 = 0;   // (claims past the last of up to 2^31 - 1 rows stay below 2^32)
+        if (lane == 0) r0 = atomicAdd((unsigned *)token, (unsigned)sh.chunk);
         r0 = __shfl_sync(kFull, r0, 0);
-        if (r0 >= count) break;
+        if (r0 >= (unsigned)count) break;
         int il = 0;
         int64_t abl = 0, ael = 0;
         bool light = false;
-        if (lane < sh.chunk && r0 + lane < count) {
+        if (lane < sh.chunk && r0 + lane < (unsigned)count) {
             il = rows[r0 + lane];
             a_row_range(op, il, abl, ael, err);
             light = ael - abl <= sh.heavy;
@@ -215,14 +215,14 @@ __global__ void __launch_bounds__(kNarrowNT) k_narrow_num(Operands<V> op, const 
         __syncthreads();
     });
     for (;;) {
-        int r0 = 0;
-        if (lane == 0) r0 = atomicAdd(token, sh.chunk);
+        unsigned r0 = 0;
+        if (lane == 0) r0 = atomicAdd((unsigned *)token, (unsigned)sh.chunk);
         r0 = __shfl_sync(kFull, r0, 0);
-        if (r0 >= count) break;
+        if (r0 >= (unsigned)count) break;
         int il = 0, nl = 0;
         int64_t abl = 0, ael = 0, cl = 0;
         bool light = false;
-        if (lane < sh.chunk && r0 + lane < count) {
+        if (lane < sh.chunk && r0 + lane < (unsigned)count) {
             il = rows[r0 + lane];
             const int64_t s = out.c_rp[il], t = out.c_rp[il + 1];
             a_row_range(op, il, abl, ael, err);
