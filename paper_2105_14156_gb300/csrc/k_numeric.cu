@@ -798,16 +798,18 @@ static void num_hash_go(const Operands<V> &op, const int *rows, int count, int *
     // holds a bit and a count per column of B: kept ready for rows that never
     // choose it, it left one 64-thread block per SM at 524,288 columns
     // (5.77 -> 2.12 ms for the mild square of that size, 1.05 -> 0.77 ms for the
-    // values of a 100,003-row float64 product).
+    // values of a 100,003-row float64 product). A bitmap that would not fit beside
+    // the bucket arrays takes as much room as they do, and only with them are the rows'
+    // products stored as they come (rows of 6,000 entries, 300,000 columns, float: 382
+    // us with the bitmap, 342 with buckets).
     int bm_words = 0;
     if (GS == NT && bitmap_ratio > 0) {
         const int words = (op.ncols + 31) / 32;
         const long long least = (long long)((T / 2) / inv_load) + 1, most = (long long)(T / inv_load) + 1;
-        const bool fits = num_hash_smem<V>(hl.tbits, GS, words, 0) <= lim;
-        if (fits && words <= bitmap_ratio * least) {
+        if (words <= bitmap_ratio * least && num_hash_smem<V>(hl.tbits, GS, words, bcap) <= lim) {
             bm_words = words;
             bcap = 0;
-        } else if (fits && bcap == 0 && words <= bitmap_ratio * most) {
+        } else if (bcap == 0 && words <= bitmap_ratio * most && num_hash_smem<V>(hl.tbits, GS, words, 0) <= lim) {
             bm_words = words;
         }
     }
