@@ -5,12 +5,11 @@
 // it away from another). The two questions cost several microseconds per launch,
 // a product of a thousand rows makes a dozen launches.
 //
-// Kept per host thread and device, a bounded number of them; nothing depends on
-// the data.
+// Kept per host thread and device, in arrays of a fixed size (no allocation that
+// could throw under the C entry points); nothing depends on the data.
 #pragma once
 
 #include <cstddef>
-#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -23,17 +22,19 @@ inline void allow_smem(const void *kernel) {
         const void *kernel;
         int dev;
     };
-    thread_local std::vector<Known> known;
+    thread_local Known known[256];
+    thread_local int n = 0;
     int dev = 0;
     cudaGetDevice(&dev);
-    for (const Known &k : known)
-        if (k.kernel == kernel && k.dev == dev) return;
+    for (int x = 0; x < n; ++x)
+        if (known[x].kernel == kernel && known[x].dev == dev) return;
     cudaFuncAttributes a;
     if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess) return;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              max_smem_per_block() - (int)a.sharedSizeBytes) != cudaSuccess)
         return;
-    known.push_back(Known{kernel, dev});
+    if (n == 256) n = 0;
+    known[n++] = Known{kernel, dev};
 }
 
 // Resident blocks per SM of nt threads with smem bytes of dynamic shared memory
@@ -44,16 +45,19 @@ inline int resident_per_sm(const void *kernel, int nt, size_t smem) {
         size_t smem;
         int dev, nt, blocks;
     };
-    thread_local std::vector<Known> known;
+    thread_local Known known[256];
+    thread_local int n = 0;
     int dev = 0;
     cudaGetDevice(&dev);
-    for (const Known &k : known)
+    for (int x = 0; x < n; ++x) {
+        const Known &k = known[x];
         if (k.kernel == kernel && k.smem == smem && k.nt == nt && k.dev == dev) return k.blocks;
+    }
     allow_smem(kernel);
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, nt, smem) != cudaSuccess) return 0;
-    if (known.size() >= 256) known.clear();
-    known.push_back(Known{kernel, smem, dev, nt, blocks});
+    if (n == 256) n = 0;
+    known[n++] = Known{kernel, smem, dev, nt, blocks};
     return blocks;
 }
 
