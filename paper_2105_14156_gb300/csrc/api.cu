@@ -472,7 +472,9 @@ int run_bins(smash_handle *h, const RawOperands &op, int64_t n, int dt, const Nu
             // 1. per-block column counts of the dense rows: from the symbolic
             //    phase of the same operands, else counted here (and sizes checked)
             const int nsub = (int)((op.ncols + kSubCols - 1) / kSubCols);
-            if (!wcache_matches(h, op) || h->wcache.nsub != nsub) {
+            // (slots are given out anew in every call, also to rows that have one:
+            // with more than two for each row all are counted again)
+            if (!wcache_matches(h, op) || h->wcache.nsub != nsub || h->wcache.slots + counts[bd] > 2 * n) {
                 if ((st = ensure(h, h->wslot, sizeof(int) * (size_t)n, s))) return st;
                 if (cudaMemsetAsync(h->wslot.ptr, 0xff, sizeof(int) * (size_t)n, s) != cudaSuccess)
                     return SMASH_ERR_CUDA;

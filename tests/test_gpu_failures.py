@@ -125,3 +125,26 @@ def test_allocation_failure_leaves_nothing_behind(handle, path):
             owner.free()
     if model is not None:
         model.close()
+
+
+def test_repeated_numeric_calls_keep_their_scratch(handle):
+    """Values again and again on one structure with dense rows: the scratch of the column counts does not grow."""
+    from paper_2105_14156_gb300 import smash
+    from tests.helpers import random_csr
+    A, B = random_csr(64, 30, 0.5, 1, values="f32"), random_csr(30, 40000, 0.05, 2, values="f32")
+    dA, dB = smash.to_device(A), smash.to_device(B)
+    al = CountingAllocator(0)
+    handle.set_allocator(al.alloc, al.free)
+    try:
+        c_rp, nnz = handle.symbolic(dA, dB)
+        out = handle.numeric(dA, dB, c_rp, nnz)
+        for _ in range(5):
+            handle.numeric(dA, dB, c_rp, nnz, out=out)
+        before = sum(al.live.values())
+        for _ in range(300):
+            handle.numeric(dA, dB, c_rp, nnz, out=out)
+        handle.check()
+        assert sum(al.live.values()) == before
+        assert_matches_oracle(out.to_host(), A, B)
+    finally:
+        handle.set_allocator(None)
