@@ -20,9 +20,12 @@ def gpu_spgemm(handle, A, B, dtype=None, **params):
     return C.to_host()
 
 
-def assert_matches_oracle(C, A, B, exact: bool = False, rows=None, ref=None):
+def assert_matches_oracle(C, A, B, exact: bool = False, rows=None, ref=None, terms: int = 0):
     """Structure bit-exact; values exact (integer-valued data) or within TOL*s_ij.
-    ref: the oracle's result for these rows, when already computed."""
+    ref: the oracle's result for these rows, when already computed. terms: the most
+    products in an entry, where TOL is less than the bound of their sum in any
+    order, terms * u (u: half the type's epsilon; a product's rounding and at most
+    terms - 1 additions)."""
     if ref is None:
         ref = oracle.spgemm(A, B, rows=rows)
     if rows is None:
@@ -43,7 +46,7 @@ def assert_matches_oracle(C, A, B, exact: bool = False, rows=None, ref=None):
     if exact:
         assert np.array_equal(got, ref.val), "values differ (exact case)"
     else:
-        tol = TOL[np.dtype(C.val.dtype)]
+        tol = max(TOL[np.dtype(C.val.dtype)], terms * float(np.finfo(C.val.dtype).eps) / 2)
         err = np.abs(got - ref.val)
         bad = err > tol * ref.abs + 1e-300
         assert not bad.any(), "max err/s = %g" % np.max(err / np.maximum(ref.abs, 1e-300))

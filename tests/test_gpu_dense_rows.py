@@ -1,11 +1,13 @@
 """Dense rows whose products are shared out over a block's warps: rows of B
 around the lengths where a warp changes from steps over several rows to rounds
-inside one (32 and 128 products), rows of A around a batch of 32 entries,
+inside one (48 products left) and from a masked round to a whole one (128; 48
+beyond one: 176), also as the only row of B that a row of A reads, so that the
+warps' parts of it end on either side; rows of A around a batch of 32 entries,
 entries without products, bitmap words and windows with a ragged end, zero
 products of either sign. Values are held to |c - c*| <= tol * sum |a||b| (1e-5
-float32, 1e-12 float64; entries have at most a few hundred terms, and (m - 1) *
-2^-24 is 1.5e-5 at m = 256 for all-equal signs, a sixteenth of it for the
-random signs here); small integers, zeros among them, must be exact."""
+float32, 1e-12 float64). An entry of C has at most 84 terms (as many
+as B has rows; 35 in the tests with more rows), and a sum of m products in any order
+is within m * 2^-24 of it: 5.0e-6; small integers, zeros among them, must be exact."""
 import numpy as np
 import pytest
 
@@ -15,7 +17,8 @@ from tests.helpers import random_csr
 
 pytestmark = pytest.mark.gpu
 
-LENS = [0, 1, 31, 32, 33, 0, 64, 127, 128, 129, 160, 255, 256, 257, 1000, 4096, 6000]
+LENS = [0, 1, 31, 32, 33, 47, 48, 49, 0, 64, 127, 128, 129, 160, 175, 176, 177, 255, 256, 257, 1000, 4096, 6000]
+PER_WARP = [m * w for w in (8, 16, 32) for m in (47, 48, 49, 128, 176)]   # lengths of the parts of 8 to 32 warps
 
 
 @pytest.fixture(scope="module")
@@ -38,15 +41,15 @@ def values_of(rng, kind, n):
 
 def operands(cols, kind, seed):
     rng = np.random.default_rng(seed)
-    lens = [min(n, cols) for n in LENS * 3]
+    lens = [min(n, cols) for n in LENS * 3 + PER_WARP]
     k = len(lens)
     r = np.repeat(np.arange(k), lens)
     c = np.concatenate([rng.permutation(cols)[:n] for n in lens])
     rp, ci = csr_from_coo(k, cols, r, c)
     B = Csr(k, cols, rp, ci, values_of(rng, kind, ci.size))
-    a_lens = [1, 2, 3, 31, 32, 33, k, 17, 5, 40]
+    a_lens = [1, 2, 3, 31, 32, 33, k, 17, 5, 40] + [1] * len(PER_WARP)
     r = np.repeat(np.arange(len(a_lens)), a_lens)
-    c = np.concatenate([rng.permutation(k)[:n] for n in a_lens])
+    c = np.concatenate([rng.permutation(k)[:n] for n in a_lens[:10]] + [np.arange(k - len(PER_WARP), k)])
     rp, ci = csr_from_coo(len(a_lens), k, r, c)
     return Csr(len(a_lens), k, rp, ci, values_of(rng, kind, ci.size)), B
 
