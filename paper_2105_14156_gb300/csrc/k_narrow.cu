@@ -19,12 +19,12 @@
 //
 // Measured (50,021-row skewed graph times 256 columns at 5 %, float; before: a
 // block of 256 threads per row): counts 0.31 -> 0.09 ms, values 0.28 -> 0.10 ms,
-// the whole product 0.79 -> 0.35 ms; a 1024-row graph's square 240 -> 165 us
+// the whole product 0.71 -> 0.35 ms; a 1024-row graph's square 235 -> 167 us
 // (both with the fewer launches of small products).
 // What is left waits for the chain of loads (row list, row of A, row pointer
-// of B, row of B) of the heavy rows' blocks: 23 % of the issue slots are used.
-// Fetching the next batch's row pointers ahead cost more instructions than the
-// wait it hid (512 batched products 1.69 -> 1.94 ms).
+// of B, row of B) of the heavy rows' blocks: 19 % of the issue slots are used by the
+// counts, 35 % by the values. Fetching the next batch's row pointers ahead cost more
+// instructions than the wait it hid (512 batched products 1.69 -> 1.94 ms).
 #include <climits>
 
 #include "device_common.cuh"

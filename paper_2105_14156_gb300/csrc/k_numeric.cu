@@ -94,7 +94,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_hash(Operands<V> op, cons
         // expanded, sorted and merged by the bucket write-out. Each product is
         // staged at its index. (Exact rows with repeated columns hashed: mild
         // float32 square of 1,048,576 rows 4.12 -> 4.01 ms, values of a 100,003-row
-        // float64 product 0.77 -> 0.73 ms; the skewed float64 one is the same.)
+        // float64 product 0.77 -> 0.73 ms; the skewed float64 one is the same. The line is
+        // flat: an eighth, a quarter and a half more products, here and in the warp rows,
+        // 3.57, 3.56 and 3.58 ms, 0.603, 0.604 and 0.604, 16,384-row pair 0.42, 0.42, 0.43.)
         const long long f_i = ok ? f_rec : -1;
         const bool direct = !CAP && bsh >= 0 && f_i >= 0 && f_i == (long long)n_exp && f_i <= bcap;
         const bool merge = bsh >= 0 && !use_bm && f_i >= 0 && 2 * f_i <= T && f_i <= bcap && !direct &&
@@ -308,8 +310,9 @@ struct WinItem {
 // lane that reads itself back adds; the others try again), so no atomic and
 // no compare-and-swap retry, and each product costs one add.
 //
-// Bound by the shared-memory pipe (70 % of the cycles in float: an atomic add is
-// a load and a compare-and-swap) and, in double, by the FP64 pipe (60 %).
+// Bound by the shared-memory pipe and instruction issue in float (60 and 57 % of the
+// cycles: an atomic add is a load and a compare-and-swap; 65,536-row skewed square, one
+// pass) and by the FP64 pipe in double (64 %; 32,768 rows).
 //
 // Double values, 512 threads: the registers of the two blocks that shared memory
 // lets an SM hold are asked for (left alone the compiler spills a few: skewed

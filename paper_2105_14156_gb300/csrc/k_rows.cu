@@ -85,6 +85,8 @@ struct RowStats {
 // may be busy with such a row for as long as all blocks are with the others, so
 // it must not start last (counts of the 65,536-row skewed square 0.89 -> 0.75
 // ms, its float64 product 6.03 -> 5.86 ms).
+// (From 2^14, 2^17 and 2^20 on: training samples of that square 1.23, 1.18 and 1.42 ms,
+// the product 5.60, 5.54 and 5.78 ms.)
 constexpr long long kHeavyFlop = 1 << 17;
 constexpr int kHeavyBit = 0x80;
 
@@ -228,8 +230,9 @@ void launch_read_small(const void *src, void *dst_mapped, size_t bytes, cudaStre
 
 // Short rows: LPR lanes per row. Long rows: appended to long_list. With few rows
 // (every row on its own lanes at once) eight lanes share a row, whose entries
-// would otherwise wait for one another: 1024 rows 27 -> 19 us, 16,384 rows 35 ->
-// 21 us.
+// would otherwise wait for one another (16 entries a row, eight lanes and one, us:
+// 4,096 rows 16 and 21, 16,384 20 and 24, 30,000 23 and 25, 38,000 26 and 26, 60,000 32
+// and 27; the line is at 256 rows an SM, 38,912).
 template <bool LEARN, int LPR>
 __global__ void __launch_bounds__(256) k_rowinfo(RawOperands op, const int64_t *c_rp, int64_t c_nnz, BinRule rule,
                                                  BinBuffers bb, long long *bound_out, int *nnz_out, int *err,
@@ -465,7 +468,8 @@ __global__ void __launch_bounds__(1024) k_scan_top(long long *part, int64_t npar
 }
 
 // The whole scan by one block, for the few rows where three launches cost more
-// than the block's passes (1024 rows: 14 -> 7 us).
+// than the block's passes (one block and three launches, us: 1,024 rows 7 and 15, 8,192
+// 11 and 16, 16,384 16 and 16).
 constexpr int64_t kScanOne = 16384;
 __global__ void __launch_bounds__(1024) k_scan_one(const int *nnz, int64_t n, int64_t *c_rp, long long *total,
                                                    ScanPublish pub) {

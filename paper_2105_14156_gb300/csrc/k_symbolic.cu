@@ -83,11 +83,11 @@ constexpr int kSpareWords = 32;   // after the bitmap: hold the bit past the las
 // row's products (block_walk); a warp then takes every kWarps-th block of
 // kSubCols columns, four words a lane, and counts and clears it in one pass.
 // words: of the bitmap, a multiple of kSubCols / 32. Bound by the shared-memory
-// pipe (72 % of the cycles: a test and mostly an atomic per product, the lanes'
-// words spread over the banks at random) and instruction issue (55 %, some 26
-// instructions per 32 products).
+// pipe (71 % of the cycles: a test and mostly an atomic per product, the lanes'
+// words spread over the banks at random) and instruction issue (61 %, some 27
+// instructions per 32 products; 131,072-row skewed square, 1.10 ms).
 // (Columns checked by a branch per product and steps of 32 products looked up
-// with a vote each: 262,144-row square 4.04 ms, now 3.52; training samples and
+// with a vote each: 262,144-row square 4.04 ms, now 3.56; training samples and
 // gradient at 65,536 rows 1.39 ms, now 1.19. No test before the atomic: 3.83 ms.)
 template <int NT, typename IT>
 __global__ void __launch_bounds__(NT) k_sym_dense(Operands<float> op, const int *rows, int count, int *token,

@@ -3,22 +3,23 @@
 // every column, shared by the batched kernel (k_batched.cu) and the narrow-B
 // rows of the two phases (k_narrow.cu).
 //
-// The shared-memory float add has no native atomic on this GPU (a
-// compare-and-swap loop: 3.4 op/clk/SM in float, 0.8 in double), so the
-// products are added with plain loads and stores. Nobody else touches the
-// warp's accumulator, and the columns inside one row of B are distinct: the
-// warp walks the rows of B that a row of A selects, W lanes to a row of B
-// (W = 8, 16 or 32, by B's mean row length), each of the 32 / W lane groups
-// with an accumulator copy of its own, so no two lanes of one step ever hit
-// one word. That holds when every row of B ascends, which a pass over B's
-// columns shows beforehand (descents_*, below; it checks their range too); for
-// any other B the products are added atomically and checked one by one.
+// A shared-memory float add has no native atomic on this GPU (a compare-and-swap
+// loop: 3.4 op/clk/SM in float, 0.8 in double), but nobody else touches the warp's
+// accumulator and few lanes of a step meet in a word: most rows simply add atomically,
+// 32 products of any rows of B a step (dense_mode). In float, long rows of B, and shorter
+// ones where copies cost nothing, take plain loads and stores: the columns inside one
+// row of B are distinct, so the warp walks the rows of B that a row of A selects, W
+// lanes to a row (W = 8, 16 or 32), each of the 32 / W lane groups with an accumulator
+// copy of its own, and no two lanes of one step ever hit one word. That holds when
+// every row of B ascends, which a pass over B's columns shows beforehand (descents_*,
+// below; it checks their range too); else those products are added atomically as well,
+// and checked one by one.
 //
 // Measured: 512 batched products of 256-column B (12.5 entries a row, float)
-// 4.40 -> 1.63 ms a call and 24 of 3000 columns (double) 1.46 -> 0.34 ms,
-// against atomic adds with a lane's row found by search, and hash tables with a
-// bitonic sort; the batched kernel now issues on 55 % of the cycles and waits
-// for loads of B otherwise.
+// 4.49 -> 1.63 ms a call and 24 of 3000 columns (double) 1.38 -> 0.33 ms,
+// against a block's tables and accumulators with a lane's row found by search, and hash
+// tables with a bitonic sort; the batched kernel now issues on 50 % of the cycles and
+// waits for loads of B otherwise.
 //
 // Occupancy needs no bitmap: an unused word holds -0.0, which no sum of
 // products reaches (a product that is -0.0 is added as +0.0, and a sum is -0.0
