@@ -129,13 +129,17 @@ struct Layout {
 // and tables, float: 2,432 and 1,245, 2,843 and 2,719, 3,254 and 4,242.)
 //   A row clears and scans its columns whatever it holds. From a kDenseFill-th of the
 // columns products a row on: accumulators. (64 products of 1,500 rows, 4,000 columns,
-// float: 16 x 16 entries 2,050 and 1,791, 21 x 16 2,203 and 2,337.)
-//   Down to an eighth of that by the rows, which k_batch_rowinfo looks at: accumulators
-// where rows that outgrow a warp's table hold a quarter of the products, as the graphs'
-// heavy rows do (100 skewed graphs, 3,000 columns, a seventeenth: 464 and 836; 24,
-// 5,000 columns, a thirtieth: 321 and 1,296), else tables (4,000 columns, a 32nd in every
-// row: 1,685 and 968). Below: tables (5,000 columns, one entry by one: 710 and 236).
+// float: 16 x 16 entries 2,050 and 1,791, 21 x 16 2,203 and 2,337.) Of accumulators up to
+// kLightBytes, which leave a block its sixteen warps, half as many products are enough
+// (float, 3,500 columns: 5 x 16 entries 798 and 715, 7 x 16 861 and 901, 13 x 16 1,003
+// and 1,493).
+//   Down to an eighth of a kDenseFill-th by the rows, which k_batch_rowinfo looks at:
+// accumulators where rows that outgrow a warp's table hold a quarter of the products, as
+// the graphs' heavy rows do (100 skewed graphs, 3,000 columns, a seventeenth: 464 and 836;
+// 24, 5,000 columns, a thirtieth: 321 and 1,296), else tables (4,000 columns, a 32nd in
+// every row: 1,685 and 968). Below: tables (5,000 columns, one entry by one: 710 and 236).
 constexpr int kDenseFill = 16;
+constexpr int kLightBytes = 14 << 10;
 enum class Large { kTables, kAccumulators, kByRows };
 
 int large_cols(int vsz) { return vsz == 8 ? 1792 : 2048; }
@@ -147,16 +151,18 @@ double products_of(const smash_csr &A, const smash_csr &B) {
 }
 
 Large large_products(int count, const smash_csr *A, const smash_csr *B, int vsz) {
-    double all = 0, large = 0, cols = 0;
+    double all = 0, large = 0, cols = 0, fill = 0;
     for (int m = 0; m < count; ++m) {
         const double f = products_of(A[m], B[m]);
         all += f;
         if (!is_large(B[m], vsz)) continue;
         large += f;
-        cols += (double)B[m].cols * (double)A[m].rows;
+        const double c = (double)B[m].cols * (double)A[m].rows;
+        cols += c;
+        fill += B[m].cols * vsz <= kLightBytes ? c / 2 : c;
     }
     if (large * 4 < all || large * kDenseFill * 8 < cols) return Large::kTables;
-    return large * kDenseFill >= cols ? Large::kAccumulators : Large::kByRows;
+    return large * kDenseFill >= fill ? Large::kAccumulators : Large::kByRows;
 }
 
 // The accumulator of a product's rows: a mode of warp_dense.cuh, or -1 (hash tables).

@@ -272,3 +272,15 @@ def test_batched_accumulators_or_tables(handle, mix, values):
     pairs = [pair(*s, 5 * q) for q, s in enumerate(sizes)]
     for (A, B), C in zip(pairs, run_batch(handle, pairs)):
         assert_matches_oracle(C, A, B, exact=values == "int")
+
+
+@pytest.mark.parametrize("values", ["f32", "int"])
+@pytest.mark.parametrize("cols", [2049, 3584, 3585])
+@pytest.mark.parametrize("entries", [5, 8])
+def test_batched_light_accumulators(handle, cols, entries, values):
+    """Rows that fill more and less than a 32nd of B's columns, up to the last accumulator of which a block holds one
+    for each of its warps, and one column more."""
+    per = cols // (30 * 5)
+    pairs = [(rows_of([entries] * 90, 60, values, 3 * q), b_matrix(cols, [per], 60, values, 3 * q + 1)) for q in range(5)]
+    for (A, B), C in zip(pairs, run_batch(handle, pairs)):
+        assert_matches_oracle(C, A, B, exact=values == "int")
